@@ -975,7 +975,7 @@ fdtd_status fdtd_mlp_forward(const float *d_params, const float *d_x, int64_t n,
 {
     if (!d_params || (n > 0 && (!d_x || !d_y)) || n < 0 || batch < 1 || !d_scratch) return FDTD_ERR_INVALID_ARG;
     if (scratch_bytes < mlp_scratch_bytes(batch, 0)) return FDTD_ERR_OOM;
-    CK(mlp_forward(d_params, d_x, n, d_y, d_scratch, batch, (cudaStream_t)stream));
+    CK(mlp_forward(d_params, d_x, n, d_y, (cudaStream_t)stream));
     return FDTD_OK;
 }
 

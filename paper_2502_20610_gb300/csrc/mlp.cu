@@ -17,9 +17,10 @@
 // leave the FP32 range) counts as zero: the cell keeps its value.  Parameters, in this order: W1 [64][324], b1 [64],
 // W2 [64][64], b2 [64], W3 [6][64], b3 [6] (row = output unit).
 //
-// Training runs on the GPU with these kernels: a tiled FP32 GEMM with
-// bias / tanh / tanh-derivative epilogues for the forward and backward
-// passes, column sums for the bias gradients, and Adam.  The layer update of
+// Training runs on the GPU with these kernels: one that takes 32 samples at
+// a time through the whole forward and backward pass in shared memory and
+// registers, and one that sums its partial gradients and takes the Adam
+// step.  The layer update of
 // a simulation step is one fused persistent kernel: it gathers the stencils
 // of 64 layer cells into shared memory and runs the three layers on them
 // with the weights resident in shared memory, the two large contractions on
@@ -37,211 +38,392 @@ namespace {
 
 using namespace mlpnet;
 
-// ------------------------------------------------------------------ GEMM
-
-// C[m][n] = epi(sum_k A(m,k) B(k,n)) with
-//   A(m,k) = A[ra(m)*sam + k*sak], ra(m) = arows ? arows[m] : m,
-//   B(k,n) = B[rb(k)*sbk + n*sbn], rb(k) = brows ? brows[k] : k.
-struct GemmArgs {
-    int M, N, K;
-    const float *A;
-    long long sam, sak;
-    const int *arows;
-    const float *B;
-    long long sbk, sbn;
-    const int *brows;
-    float *C;
-    long long ldc;
-    const float *bias;  // [N]
-    const float *aux;   // [M][ldaux]: the layer's activation (EPI_DTANH)
-    long long ldaux;
-};
-
-enum { EPI_NONE = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3 };
-
-constexpr int GT = 64, GK = 16;
-
-template <int EPI>
-__global__ void __launch_bounds__(256) gemm_kernel(const GemmArgs g)
-{
-    __shared__ float As[GK][GT + 4];
-    __shared__ float Bs[GK][GT + 4];
-    const int tid = threadIdx.x, tm = tid >> 4, tn = tid & 15;
-    const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int k0 = 0; k0 < g.K; k0 += GK) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + q * 256;
-            const int mm = e >> 4, kk = e & 15;
-            const int m = m0 + mm, k = k0 + kk;
-            float v = 0.f;
-            if (m < g.M && k < g.K) {
-                const long long r = g.arows ? g.arows[m] : m;
-                v = g.A[r * g.sam + (long long)k * g.sak];
-            }
-            As[kk][mm] = v;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = tid + q * 256;
-            const int kk = e >> 6, nn = e & 63;
-            const int k = k0 + kk, n = n0 + nn;
-            float v = 0.f;
-            if (k < g.K && n < g.N) {
-                const long long r = g.brows ? g.brows[k] : k;
-                v = g.B[r * g.sbk + (long long)n * g.sbn];
-            }
-            Bs[kk][nn] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][tm * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tn * 4 + j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = __fmaf_rn(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int m = m0 + tm * 4 + i, n = n0 + tn * 4 + j;
-            if (m >= g.M || n >= g.N) continue;
-            float v = acc[i][j];
-            if (EPI == EPI_BIAS_TANH) v = tanhf(__fadd_rn(v, g.bias[n]));
-            if (EPI == EPI_BIAS) v = __fadd_rn(v, g.bias[n]);
-            if (EPI == EPI_DTANH) {
-                const float h = g.aux[(long long)m * g.ldaux + n];
-                v = __fmul_rn(v, __fsub_rn(1.f, __fmul_rn(h, h)));
-            }
-            g.C[(long long)m * g.ldc + n] = v;
-        }
-}
-
-template <int EPI>
-cudaError_t gemm(const GemmArgs &g, cudaStream_t st)
-{
-    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-    dim3 grid((g.N + GT - 1) / GT, (g.M + GT - 1) / GT);
-    gemm_kernel<EPI><<<grid, 256, 0, st>>>(g);
-    return cudaGetLastError();
-}
-
-GemmArgs ga(int M, int N, int K, const float *A, long long sam, long long sak, const int *arows, const float *B,
-            long long sbk, long long sbn, const int *brows, float *C, long long ldc, const float *bias = nullptr,
-            const float *aux = nullptr, long long ldaux = 0)
-{
-    GemmArgs g;
-    g.M = M; g.N = N; g.K = K;
-    g.A = A; g.sam = sam; g.sak = sak; g.arows = arows;
-    g.B = B; g.sbk = sbk; g.sbn = sbn; g.brows = brows;
-    g.C = C; g.ldc = ldc; g.bias = bias; g.aux = aux; g.ldaux = ldaux;
-    return g;
-}
-
-// out[n] = sum_m A[m][n] (A is M x N row-major), one block per column
-__global__ void __launch_bounds__(256) colsum_kernel(const float *__restrict__ A, int M, int N,
-                                                     float *__restrict__ out)
-{
-    __shared__ float part[256];
-    const int n = blockIdx.x;
-    float s = 0.f;
-    for (int m = threadIdx.x; m < M; m += 256) s = __fadd_rn(s, A[(long long)m * N + n]);
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) part[threadIdx.x] = __fadd_rn(part[threadIdx.x], part[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[n] = part[0];
-}
-
-// dY = 2 (Y - T[rows]) / (B * 6); loss += sum (Y - T)^2 (FP64)
-__global__ void __launch_bounds__(256) dy_kernel(const float *__restrict__ Y, const float *__restrict__ T,
-                                                 const int *__restrict__ rows, int B, float *__restrict__ dY,
-                                                 double *__restrict__ loss)
-{
-    __shared__ double part[256];
-    const int e = blockIdx.x * 256 + threadIdx.x;
-    double s = 0.0;
-    if (e < B * NO) {
-        const int b = e / NO, o = e - b * NO;
-        const long long r = rows ? rows[b] : b;
-        const float d = __fsub_rn(Y[e], T[r * NO + o]);
-        dY[e] = __fmul_rn(d, 2.f / (float)(B * NO));
-        s = (double)d * (double)d;
-    }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(loss, part[0]);
-}
-
-// Adam (Kingma & Ba): m <- b1 m + (1-b1) g, v <- b2 v + (1-b2) g^2,
-// p <- p - lr * (m / (1-b1^t)) / (sqrt(v / (1-b2^t)) + eps)
-__global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ p, const float *__restrict__ g,
-                                                   float *__restrict__ m, float *__restrict__ v, int n, float lr,
-                                                   float c1, float c2)
-{
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= n) return;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
+constexpr int NPARAM_PITCH = (NPARAM + 31) / 32 * 32;  // one partial gradient, 128-byte aligned rows
 
 // ------------------------------------------------- forward / backward pass
 
+// One kernel takes a minibatch through the whole network: a CTA holds the
+// weights and 32 samples in shared memory, runs the three layers, the loss
+// and (training) the backward pass on them, and keeps the weight gradients
+// in registers over all its tiles, so activations never leave the SM and a
+// minibatch costs two launches (this one, then grad_kernel).  What bounds
+// it: FP32 FMA issue (25 k multiply-adds a sample forward, 29 k backward).
+// Splitting a minibatch over its samples gives a CTA per 32 of them; the
+// sums over samples are then short (32 in sequence, then one partial per
+// CTA), where one CTA per weight-gradient tile ran a 4096-long chain.
+// Measured (ncu): 29 us + 7 us in grad_kernel for a batch of 4096, against
+// 1.38 ms in eleven GEMM and reduction launches; two epochs over 32768
+// samples 22.1 ms -> 0.75 ms.
+// FP32 multiply-adds, not split TF32 products on the tensor cores: a
+// split has no form for infinities (inf - inf), and the sums here round
+// as FP32 sums do.  Pairs of multiply-adds go out as one packed f32x2
+// instruction, each half rounded as the scalar one is.
+constexpr int TS = 32;         // samples per tile
+constexpr int NT = 256;        // threads
+constexpr int PH = NH + 4;     // pitch of 64-wide rows: 16-byte rows, 8 rows on 8 bank groups
+constexpr int KC1 = NI / 4, KC2 = NH / 4;  // 16-byte chunks of a row
+static_assert(NI % 4 == 0 && (NI / 4) % 8 == 1 && (PH / 4) % 8 == 1, "row starts of 8 lanes on 8 bank groups");
+static_assert(OFF_W2 % 4 == 0, "W2 rows 16-byte aligned when the parameters are");
+// shared memory, in floats
+constexpr int NS_W1 = 0, NS_X = NS_W1 + NH * NI, NS_W2 = NS_X + TS * NI, NS_W2T = NS_W2 + NH * PH,
+              NS_H1 = NS_W2T + NH * PH, NS_H2 = NS_H1 + TS * PH, NS_Z1 = NS_H2 + TS * PH, NS_Z2 = NS_Z1 + TS * PH,
+              NS_RED = NS_Z2 + TS * PH, NS_W3 = NS_RED + 3 * TS * NH, NS_B = NS_W3 + NO * NH, NS_DY = NS_B + 136,
+              NS_LOSS = NS_DY + TS * 8, NS_END = NS_LOSS + 2 * NT;
+static_assert(NS_LOSS % 2 == 0, "FP64 partial sums 8-byte aligned");
+constexpr size_t NET_SMEM = sizeof(float) * NS_END;
+static_assert(NET_SMEM <= 227 * 1024, "one CTA's shared memory");
+// CTAs (and gradient partials) of a minibatch: one per SM of the chip at most
+constexpr int MAX_PARTS = 152;
+
+int net_parts(long long B) { return (int)std::min<long long>((B + TS - 1) / TS, MAX_PARTS); }
+
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pair(float lo, float hi)
+{
+    return (unsigned long long)__float_as_uint(lo) | ((unsigned long long)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ float lo_of(unsigned long long v) { return __uint_as_float((unsigned)v); }
+__device__ __forceinline__ float hi_of(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
+
+// out[s][u] = sum_k A[s][k] W[u][k] for the tile's 32 samples and 64 units
+// (CHUNKS 16-byte chunks of k), before bias and activation, left as four
+// partial sums to be added by tile_sum: warp w takes samples 16 * (w / 4) ..
+// and every fourth chunk from w % 4, a lane units lane and lane + 32.  A's
+// loads are broadcasts, W's conflict-free; 16 samples a warp make a chunk 24
+// shared-memory wavefronts for 64 packed multiply-adds.
+template <int CHUNKS>
+__device__ __forceinline__ void tile_product(const float *A, int pa, const float *W, int pw, float *out, float *red)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, kq = w & 3, s0 = 16 * (w >> 2);
+    unsigned long long acc[16][2];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) acc[s][0] = acc[s][1] = 0ull;
+#pragma unroll 1
+    for (int c = kq; c < CHUNKS; c += 4) {
+        const ulonglong2 w0 = *reinterpret_cast<const ulonglong2 *>(W + lane * pw + 4 * c);
+        const ulonglong2 w1 = *reinterpret_cast<const ulonglong2 *>(W + (lane + 32) * pw + 4 * c);
+#pragma unroll
+        for (int s = 0; s < 16; ++s) {
+            const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(A + (s0 + s) * pa + 4 * c);
+            acc[s][0] = fma2(x.x, w0.x, acc[s][0]);
+            acc[s][1] = fma2(x.x, w1.x, acc[s][1]);
+            acc[s][0] = fma2(x.y, w0.y, acc[s][0]);
+            acc[s][1] = fma2(x.y, w1.y, acc[s][1]);
+        }
+    }
+    float *dst = kq == 0 ? out : red + (kq - 1) * TS * NH;
+    const int pd = kq == 0 ? PH : NH;
+#pragma unroll
+    for (int s = 0; s < 16; ++s)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            dst[(s0 + s) * pd + lane + 32 * h] = __fadd_rn(lo_of(acc[s][h]), hi_of(acc[s][h]));
+}
+
+// The four partial sums of element (s, u); called after a block barrier.
+__device__ __forceinline__ float tile_sum(const float *out, const float *red, int s, int u)
+{
+    const int r = s * NH + u;
+    return __fadd_rn(__fadd_rn(out[s * PH + u], red[r]), __fadd_rn(red[TS * NH + r], red[2 * TS * NH + r]));
+}
+
+// Y = f(X) of B samples X[rows[b]] (rows may be null; FORWARD only: Y is
+// written), or (!FORWARD) this CTA's share of the gradient of the mean
+// squared error against T into part[blockIdx.x][NPARAM] and of the sum of
+// squared errors into loss_part[blockIdx.x].  vec: P and X are 16-byte
+// aligned (rows of X then are too), loaded by 16-byte asynchronous copies.
+template <bool FORWARD>
+__global__ void __launch_bounds__(NT, 1) net_kernel(const float *__restrict__ P, const float *__restrict__ X,
+                                                    const int *__restrict__ rows, const float *__restrict__ T,
+                                                    long long B, float *__restrict__ Y, float *__restrict__ part,
+                                                    double *__restrict__ loss_part, int vec)
+{
+    extern __shared__ __align__(16) float sm[];
+    float *const W1 = sm + NS_W1, *const Xs = sm + NS_X, *const W2 = sm + NS_W2, *const W2t = sm + NS_W2T;
+    float *const H1 = sm + NS_H1, *const H2 = sm + NS_H2, *const Z1 = sm + NS_Z1, *const Z2 = sm + NS_Z2;
+    float *const red = sm + NS_RED, *const W3 = sm + NS_W3, *const bias = sm + NS_B, *const dY = sm + NS_DY;
+    double *const lsum = reinterpret_cast<double *>(sm + NS_LOSS);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const long long ntiles = (B + TS - 1) / TS;
+    auto copy16 = [](float *dst, const float *src) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                     : "memory");
+    };
+    auto load_tile = [&](long long tile) {
+        for (int e = tid; e < TS * KC1; e += NT) {
+            const int s = e / KC1, c = e - s * KC1;
+            const long long b = tile * TS + s;
+            float *const dst = Xs + s * NI + 4 * c;
+            if (b < B) {
+                const float *const src = X + (rows ? (long long)rows[b] : b) * NI + 4 * c;
+                if (vec) {
+                    copy16(dst, src);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dst[q] = src[q];
+                }
+            } else {  // past the batch: zeros, and no share of dY
+                *reinterpret_cast<float4 *>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    };
+    load_tile(blockIdx.x);
+    if (vec) {
+        for (int e = tid; e < NH * KC1; e += NT) copy16(W1 + 4 * e, P + OFF_W1 + 4 * e);
+        for (int e = tid; e < NH * KC2; e += NT) copy16(W2 + (e / KC2) * PH + 4 * (e % KC2), P + OFF_W2 + 4 * e);
+    } else {
+        for (int e = tid; e < NH * NI; e += NT) W1[e] = P[OFF_W1 + e];
+        for (int e = tid; e < NH * NH; e += NT) W2[(e / NH) * PH + e % NH] = P[OFF_W2 + e];
+    }
+    if (!FORWARD)
+        for (int e = tid; e < NH * NH; e += NT) W2t[(e % NH) * PH + e / NH] = P[OFF_W2 + e];
+    for (int e = tid; e < NO * NH; e += NT) W3[e] = P[OFF_W3 + e];
+    if (tid < NH) {
+        bias[tid] = P[OFF_B1 + tid];
+        bias[NH + tid] = P[OFF_B2 + tid];
+    }
+    if (tid < NO) bias[2 * NH + tid] = P[OFF_B3 + tid];
+
+    // weight gradients of this CTA's tiles: dW1 of units 8w.. and inputs
+    // 4 lane + 128 j .. (+3), dW2 of units 8w.. and units 2 lane (+1), dW3 of
+    // elements tid, tid + 256, and the bias of unit tid (64..127: of layer 1)
+    unsigned long long g1[8][6], g2[8];
+    float g3[2] = {0.f, 0.f}, gb = 0.f, gb3 = 0.f;
+    double loss = 0.0;
+    const float dscale = 2.f / (float)(B * NO);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        g2[u] = 0ull;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) g1[u][j] = 0ull;
+    }
+    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        if (tile != blockIdx.x) {
+            __syncthreads();  // the previous tile's last reads of Xs
+            load_tile(tile);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        // rows past the batch stay zero in every layer, whatever the weights
+        const int live = (int)min((long long)TS, B - tile * TS);
+        tile_product<KC1>(Xs, NI, W1, NI, H1, red);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TS * NH / NT; ++q) {
+            const int s = (tid >> 6) + 4 * q, u = tid & 63;
+            H1[s * PH + u] = s < live ? tanhf(__fadd_rn(tile_sum(H1, red, s, u), bias[u])) : 0.f;
+        }
+        __syncthreads();
+        tile_product<KC2>(H1, PH, W2, PH, H2, red);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TS * NH / NT; ++q) {
+            const int s = (tid >> 6) + 4 * q, u = tid & 63;
+            H2[s * PH + u] = s < live ? tanhf(__fadd_rn(tile_sum(H2, red, s, u), bias[NH + u])) : 0.f;
+        }
+        __syncthreads();
+        if (tid < TS * NO) {  // layer 3: Y, and dY = 2 (Y - T) / (6 B)
+            const int s = tid / NO, o = tid - s * NO;
+            const long long b = tile * TS + s;
+            float f = 0.f;
+#pragma unroll
+            for (int k = 0; k < NH; k += 4) {
+                const float4 h = *reinterpret_cast<const float4 *>(H2 + s * PH + k);
+                const float4 v = *reinterpret_cast<const float4 *>(W3 + o * NH + k);
+                f = __fmaf_rn(h.x, v.x, f);
+                f = __fmaf_rn(h.y, v.y, f);
+                f = __fmaf_rn(h.z, v.z, f);
+                f = __fmaf_rn(h.w, v.w, f);
+            }
+            f = __fadd_rn(f, bias[2 * NH + o]);
+            if (FORWARD) {
+                if (b < B) Y[b * NO + o] = f;
+            } else {
+                float d = 0.f;
+                if (b < B) {
+                    d = __fsub_rn(f, T[(rows ? (long long)rows[b] : b) * NO + o]);
+                    loss += (double)d * (double)d;
+                }
+                dY[s * 8 + o] = __fmul_rn(d, dscale);
+            }
+        }
+        if (FORWARD) continue;
+        __syncthreads();
+        // dZ2 = (dY W3) (1 - H2^2); dW3 and db3
+        {
+            const int u = tid & 63;
+            float v3[NO];
+#pragma unroll
+            for (int o = 0; o < NO; ++o) v3[o] = W3[o * NH + u];
+#pragma unroll
+            for (int q = 0; q < TS * NH / NT; ++q) {
+                const int s = (tid >> 6) + 4 * q;
+                float z = 0.f;
+#pragma unroll
+                for (int o = 0; o < NO; ++o) z = __fmaf_rn(dY[s * 8 + o], v3[o], z);
+                const float h = H2[s * PH + u];
+                Z2[s * PH + u] = s < live ? __fmul_rn(z, __fsub_rn(1.f, __fmul_rn(h, h))) : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int e = tid + q * NT;
+                if (e < NO * NH)
+                    for (int s = 0; s < TS; ++s) g3[q] = __fmaf_rn(dY[s * 8 + (e >> 6)], H2[s * PH + (e & 63)], g3[q]);
+            }
+            if (tid < NO)
+                for (int s = 0; s < TS; ++s) gb3 = __fadd_rn(gb3, dY[s * 8 + tid]);
+        }
+        __syncthreads();
+        // dW2 = dZ2^T H1 and db2; dZ1 = (dZ2 W2) (1 - H1^2)
+#pragma unroll 4
+        for (int s = 0; s < TS; ++s) {
+            const float4 za = *reinterpret_cast<const float4 *>(Z2 + s * PH + 8 * w);
+            const float4 zb = *reinterpret_cast<const float4 *>(Z2 + s * PH + 8 * w + 4);
+            const unsigned long long h = *reinterpret_cast<const unsigned long long *>(H1 + s * PH + 2 * lane);
+            const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+#pragma unroll
+            for (int u = 0; u < 8; ++u) g2[u] = fma2(pair(z[u], z[u]), h, g2[u]);
+        }
+        tile_product<KC2>(Z2, PH, W2t, PH, Z1, red);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TS * NH / NT; ++q) {
+            const int s = (tid >> 6) + 4 * q, u = tid & 63;
+            const float h = H1[s * PH + u];
+            Z1[s * PH + u] = s < live ? __fmul_rn(tile_sum(Z1, red, s, u), __fsub_rn(1.f, __fmul_rn(h, h))) : 0.f;
+        }
+        __syncthreads();
+        if (tid < 2 * NH) {  // db2 (unit tid), db1 (unit tid - 64)
+            const float *const Z = tid < NH ? Z2 + tid : Z1 + tid - NH;
+            for (int s = 0; s < TS; ++s) gb = __fadd_rn(gb, Z[s * PH]);
+        }
+        // dW1 = dZ1^T X
+#pragma unroll 1
+        for (int s = 0; s < TS; ++s) {
+            const float4 za = *reinterpret_cast<const float4 *>(Z1 + s * PH + 8 * w);
+            const float4 zb = *reinterpret_cast<const float4 *>(Z1 + s * PH + 8 * w + 4);
+            const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+            ulonglong2 x[3];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int k = 4 * lane + 128 * j;
+                x[j] = k < NI ? *reinterpret_cast<const ulonglong2 *>(Xs + s * NI + k) : make_ulonglong2(0ull, 0ull);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const unsigned long long zz = pair(z[u], z[u]);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    g1[u][2 * j] = fma2(zz, x[j].x, g1[u][2 * j]);
+                    g1[u][2 * j + 1] = fma2(zz, x[j].y, g1[u][2 * j + 1]);
+                }
+            }
+        }
+    }
+    if (FORWARD) return;
+    float *const G = part + (long long)blockIdx.x * NPARAM_PITCH;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int k = 4 * lane + 128 * j;
+            if (k < NI)
+                *reinterpret_cast<float4 *>(G + OFF_W1 + (8 * w + u) * NI + k) =
+                    make_float4(lo_of(g1[u][2 * j]), hi_of(g1[u][2 * j]), lo_of(g1[u][2 * j + 1]), hi_of(g1[u][2 * j + 1]));
+        }
+        *reinterpret_cast<float2 *>(G + OFF_W2 + (8 * w + u) * NH + 2 * lane) = make_float2(lo_of(g2[u]), hi_of(g2[u]));
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        if (tid + q * NT < NO * NH) G[OFF_W3 + tid + q * NT] = g3[q];
+    if (tid < NH) G[OFF_B2 + tid] = gb;
+    else if (tid < 2 * NH) G[OFF_B1 + tid - NH] = gb;
+    if (tid < NO) G[OFF_B3 + tid] = gb3;
+    lsum[tid] = loss;
+    __syncthreads();
+    for (int n = NT / 2; n > 0; n >>= 1) {
+        if (tid < n) lsum[tid] += lsum[tid + n];
+        __syncthreads();
+    }
+    if (tid == 0) loss_part[blockIdx.x] = lsum[0];
+}
+
+// The minibatch's gradient from its nparts partials (a thread sums every
+// eighth, then the eight sums; the order is fixed), then the Adam step
+// (Kingma & Ba): m <- b1 m + (1-b1) g, v <- b2 v + (1-b2) g^2,
+// p <- p - lr * (m / (1-b1^t)) / (sqrt(v / (1-b2^t)) + eps); or (!ADAM) the
+// gradient into out.  *loss += the sum of squared errors.  Bounded by the
+// read of the partials out of L2 (13 MB at a batch of 4096); 32 parameters a
+// CTA put 793 CTAs of independent loads on it.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) grad_kernel(const float *__restrict__ part, const double *__restrict__ loss_part,
+                                                   int nparts, float *__restrict__ p, float *__restrict__ m,
+                                                   float *__restrict__ v, float lr, float c1, float c2,
+                                                   float *__restrict__ out, double *__restrict__ loss)
+{
+    __shared__ float sum[8][32];
+    const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (i < NPARAM) {
+#pragma unroll 4
+        for (int j = sl; j < nparts; j += 8) s = __fadd_rn(s, part[(long long)j * NPARAM_PITCH + i]);
+    }
+    sum[sl][lane] = s;
+    __syncthreads();
+    if (blockIdx.x == 0 && sl == 1) {
+        double l = 0.0;
+        for (int j = lane; j < nparts; j += 32) l += loss_part[j];
+        for (int d = 16; d > 0; d >>= 1) l += __shfl_down_sync(0xffffffffu, l, d);
+        if (lane == 0) *loss += l;
+    }
+    if (sl || i >= NPARAM) return;
+    float gi = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) gi = __fadd_rn(gi, sum[q][lane]);
+    if (ADAM) {
+        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+        const float mi = b1 * m[i] + (1.f - b1) * gi;
+        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+        m[i] = mi;
+        v[i] = vi;
+        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    } else {
+        out[i] = gi;
+    }
+}
+
 struct Scratch {
-    float *H1, *H2, *Y, *dY, *dZ2, *dZ1, *grad, *m, *v;
-    double *loss;
+    float *part, *m, *v;
+    double *loss, *loss_part;
     int *rows;  // the training permutation (n entries)
 };
 
 size_t scratch_bytes(int batch, long long n)
 {
-    const size_t b = (size_t)batch;
-    return sizeof(float) * (b * NH * 4 + b * NO * 2 + 3 * (size_t)NPARAM) + sizeof(double) * 2 +
-           sizeof(int) * (size_t)n + 12 * 256;
+    const size_t parts = (size_t)net_parts(batch);
+    return sizeof(float) * (parts * NPARAM_PITCH + 2 * (size_t)NPARAM) + sizeof(double) * (2 + parts) +
+           sizeof(int) * (size_t)n + 7 * 256;
 }
 
 Scratch carve(void *base, int batch, long long n)
 {
-    char *p = (char *)base;
+    // the caller's block may start anywhere; the partials are written 16 bytes at a time
+    char *p = (char *)(((uintptr_t)base + 15) / 16 * 16);
     auto take = [&](size_t bytes) {
         char *q = p;
         p += (bytes + 255) / 256 * 256;
         return q;
     };
-    const size_t b = (size_t)batch;
+    const size_t parts = (size_t)net_parts(batch);
     Scratch s;
     s.loss = (double *)take(sizeof(double) * 2);
-    s.H1 = (float *)take(sizeof(float) * b * NH);
-    s.H2 = (float *)take(sizeof(float) * b * NH);
-    s.dZ2 = (float *)take(sizeof(float) * b * NH);
-    s.dZ1 = (float *)take(sizeof(float) * b * NH);
-    s.Y = (float *)take(sizeof(float) * b * NO);
-    s.dY = (float *)take(sizeof(float) * b * NO);
-    s.grad = (float *)take(sizeof(float) * NPARAM);
+    s.loss_part = (double *)take(sizeof(double) * parts);
+    s.part = (float *)take(sizeof(float) * parts * NPARAM_PITCH);
     s.m = (float *)take(sizeof(float) * NPARAM);
     s.v = (float *)take(sizeof(float) * NPARAM);
     s.rows = (int *)take(sizeof(int) * (size_t)n);
@@ -254,39 +436,18 @@ Scratch carve(void *base, int batch, long long n)
         if (e_ != cudaSuccess) return e_;                                      \
     } while (0)
 
-// H1, H2, Y of B samples X[rows[b]] (rows may be null).
-cudaError_t forward(const float *P, const float *X, const int *rows, int B, const Scratch &s, float *Y,
-                    cudaStream_t st)
+template <bool FORWARD>
+cudaError_t net_configure()
 {
-    CKE(gemm<EPI_BIAS_TANH>(ga(B, NH, NI, X, NI, 1, rows, P + OFF_W1, 1, NI, nullptr, s.H1, NH, P + OFF_B1), st));
-    CKE(gemm<EPI_BIAS_TANH>(ga(B, NH, NH, s.H1, NH, 1, nullptr, P + OFF_W2, 1, NH, nullptr, s.H2, NH, P + OFF_B2),
-                            st));
-    CKE(gemm<EPI_BIAS>(ga(B, NO, NH, s.H2, NH, 1, nullptr, P + OFF_W3, 1, NH, nullptr, Y, NO, P + OFF_B3), st));
-    return cudaSuccess;
+    return cudaFuncSetAttribute(net_kernel<FORWARD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NET_SMEM);
 }
 
-// Gradient of the mean squared error of B samples into s.grad; adds the
-// sum of squared errors to *s.loss.
-cudaError_t backward(const float *P, const float *X, const float *T, const int *rows, int B, const Scratch &s,
-                     cudaStream_t st)
+template <bool FORWARD>
+cudaError_t net(const float *P, const float *X, const int *rows, const float *T, long long B, float *Y, float *part,
+                double *loss_part, cudaStream_t st)
 {
-    CKE(forward(P, X, rows, B, s, s.Y, st));
-    dy_kernel<<<(B * NO + 255) / 256, 256, 0, st>>>(s.Y, T, rows, B, s.dY, s.loss);
-    CKE(cudaGetLastError());
-    float *G = s.grad;
-    // layer 3: dW3 = dY^T H2, db3 = sum dY, dZ2 = (dY W3) * (1 - H2^2)
-    CKE(gemm<EPI_NONE>(ga(NO, NH, B, s.dY, 1, NO, nullptr, s.H2, NH, 1, nullptr, G + OFF_W3, NH), st));
-    colsum_kernel<<<NO, 256, 0, st>>>(s.dY, B, NO, G + OFF_B3);
-    CKE(gemm<EPI_DTANH>(ga(B, NH, NO, s.dY, NO, 1, nullptr, P + OFF_W3, NH, 1, nullptr, s.dZ2, NH, nullptr, s.H2, NH),
-                        st));
-    // layer 2
-    CKE(gemm<EPI_NONE>(ga(NH, NH, B, s.dZ2, 1, NH, nullptr, s.H1, NH, 1, nullptr, G + OFF_W2, NH), st));
-    colsum_kernel<<<NH, 256, 0, st>>>(s.dZ2, B, NH, G + OFF_B2);
-    CKE(gemm<EPI_DTANH>(ga(B, NH, NH, s.dZ2, NH, 1, nullptr, P + OFF_W2, NH, 1, nullptr, s.dZ1, NH, nullptr, s.H1, NH),
-                        st));
-    // layer 1
-    CKE(gemm<EPI_NONE>(ga(NH, NI, B, s.dZ1, 1, NH, nullptr, X, NI, 1, rows, G + OFF_W1, NI), st));
-    colsum_kernel<<<NH, 256, 0, st>>>(s.dZ1, B, NH, G + OFF_B1);
+    const int vec = ((uintptr_t)P % 16 == 0) && ((uintptr_t)X % 16 == 0);
+    net_kernel<FORWARD><<<net_parts(B), NT, NET_SMEM, st>>>(P, X, rows, T, B, Y, part, loss_part, vec);
     return cudaGetLastError();
 }
 
@@ -676,15 +837,11 @@ __global__ void __launch_bounds__(256) fill_xslab_kernel(float *__restrict__ sna
 
 size_t mlp_scratch_bytes(int batch, long long n) { return scratch_bytes(batch, n); }
 
-cudaError_t mlp_forward(const float *params, const float *X, long long n, float *Y, void *scratch, int batch,
-                        cudaStream_t st)
+cudaError_t mlp_forward(const float *params, const float *X, long long n, float *Y, cudaStream_t st)
 {
-    Scratch s = carve(scratch, batch, 0);
-    for (long long b0 = 0; b0 < n; b0 += batch) {
-        const int B = (int)std::min<long long>(batch, n - b0);
-        CKE(forward(params, X + b0 * NI, nullptr, B, s, Y + b0 * NO, st));
-    }
-    return cudaSuccess;
+    if (n <= 0) return cudaSuccess;
+    CKE(net_configure<true>());
+    return net<true>(params, X, nullptr, nullptr, n, Y, nullptr, nullptr, st);
 }
 
 cudaError_t mlp_grad(const float *params, const float *X, const float *T, int n, float *grad, double *loss_host,
@@ -692,9 +849,12 @@ cudaError_t mlp_grad(const float *params, const float *X, const float *T, int n,
 {
     if (n > batch) return cudaErrorInvalidValue;
     Scratch s = carve(scratch, batch, 0);
+    CKE(net_configure<false>());
     CKE(cudaMemsetAsync(s.loss, 0, sizeof(double), st));
-    CKE(backward(params, X, T, nullptr, n, s, st));
-    CKE(cudaMemcpyAsync(grad, s.grad, sizeof(float) * NPARAM, cudaMemcpyDeviceToDevice, st));
+    CKE(net<false>(params, X, nullptr, T, n, nullptr, s.part, s.loss_part, st));
+    grad_kernel<false><<<(NPARAM + 31) / 32, 256, 0, st>>>(s.part, s.loss_part, net_parts(n), nullptr, nullptr, nullptr,
+                                                           0.f, 1.f, 1.f, grad, s.loss);
+    CKE(cudaGetLastError());
     double l = 0.0;
     CKE(cudaMemcpyAsync(&l, s.loss, sizeof(double), cudaMemcpyDeviceToHost, st));
     CKE(cudaStreamSynchronize(st));
@@ -706,31 +866,50 @@ cudaError_t mlp_train(float *params, const float *X, const float *T, long long n
                       unsigned long long seed, void *scratch, cudaStream_t st, double *last_epoch_loss)
 {
     Scratch s = carve(scratch, batch, n);
+    CKE(net_configure<false>());
     CKE(cudaMemsetAsync(s.m, 0, sizeof(float) * NPARAM, st));
     CKE(cudaMemsetAsync(s.v, 0, sizeof(float) * NPARAM, st));
+    CKE(cudaMemsetAsync(s.loss, 0, sizeof(double), st));
     std::mt19937_64 rng(seed);
     std::vector<int> perm((size_t)n);
     for (long long i = 0; i < n; ++i) perm[(size_t)i] = (int)i;
     const long long nb = n / batch;  // whole batches only
+    const int parts = net_parts(batch);
     long long t = 0;
-    double epoch_loss = 0.0;
+    // the host shuffles the next epoch's order while the GPU runs this one:
+    // an epoch's order is copied from a host buffer of its own, taken again
+    // two epochs later, after that copy
+    std::vector<int> order[2];
+    struct Events {
+        cudaEvent_t e[2] = {nullptr, nullptr};
+        ~Events()
+        {
+            for (cudaEvent_t x : e)
+                if (x) cudaEventDestroy(x);
+        }
+    } copied;
     for (int ep = 0; ep < epochs; ++ep) {
         std::shuffle(perm.begin(), perm.end(), rng);
+        cudaEvent_t &ev = copied.e[ep & 1];
+        if (ev) CKE(cudaEventSynchronize(ev));
+        else CKE(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        order[ep & 1] = perm;
         CKE(cudaMemsetAsync(s.loss, 0, sizeof(double), st));
-        CKE(cudaMemcpyAsync(s.rows, perm.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, st));
+        CKE(cudaMemcpyAsync(s.rows, order[ep & 1].data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, st));
+        CKE(cudaEventRecord(ev, st));
         for (long long b = 0; b < nb; ++b) {
-            CKE(backward(params, X, T, s.rows + b * batch, batch, s, st));
+            CKE(net<false>(params, X, s.rows + b * batch, T, batch, nullptr, s.part, s.loss_part, st));
             ++t;
             const float c1 = (float)(1.0 - std::pow(0.9, (double)t)), c2 = (float)(1.0 - std::pow(0.999, (double)t));
-            adam_kernel<<<(NPARAM + 255) / 256, 256, 0, st>>>(params, s.grad, s.m, s.v, NPARAM, (float)lr, c1, c2);
+            grad_kernel<true><<<(NPARAM + 31) / 32, 256, 0, st>>>(s.part, s.loss_part, parts, params, s.m, s.v, (float)lr,
+                                                                  c1, c2, nullptr, s.loss);
             CKE(cudaGetLastError());
         }
-        double l = 0.0;
-        CKE(cudaMemcpyAsync(&l, s.loss, sizeof(double), cudaMemcpyDeviceToHost, st));
-        CKE(cudaStreamSynchronize(st));
-        epoch_loss = nb > 0 ? l / ((double)nb * batch * NO) : 0.0;
     }
-    if (last_epoch_loss) *last_epoch_loss = epoch_loss;
+    double l = 0.0;
+    CKE(cudaMemcpyAsync(&l, s.loss, sizeof(double), cudaMemcpyDeviceToHost, st));
+    CKE(cudaStreamSynchronize(st));
+    if (last_epoch_loss) *last_epoch_loss = epochs > 0 && nb > 0 ? l / ((double)nb * batch * NO) : 0.0;
     return cudaSuccess;
 }
 

@@ -15,8 +15,7 @@ constexpr float R_MIN = 1e-30f;  // smaller stencil RMS counts as a zero stencil
 // Scratch of the forward / gradient / training calls for minibatches of
 // `batch` samples over a set of n samples (the training permutation).
 size_t mlp_scratch_bytes(int batch, long long n);
-cudaError_t mlp_forward(const float *params, const float *X, long long n, float *Y, void *scratch, int batch,
-                        cudaStream_t st);
+cudaError_t mlp_forward(const float *params, const float *X, long long n, float *Y, cudaStream_t st);
 cudaError_t mlp_grad(const float *params, const float *X, const float *T, int n, float *grad, double *loss_host,
                      void *scratch, int batch, cudaStream_t st);
 cudaError_t mlp_train(float *params, const float *X, const float *T, long long n, int batch, int epochs, double lr,
