@@ -8,8 +8,9 @@
  *     H^{n+1/2} = H^{n-1/2} - dt * curl_f E^n
  *     E^{n+1}   = E^n + (dt/eps) * curl_b H^{n+1/2}   (+ point sources)
  * Two schedules compute it (both bit-identical in FP32):
- *   FDTD_SCHEME_NAIVE    one kernel per half-step over the whole grid, the
- *                        straightforward streaming update of Sec. 2;
+ *   FDTD_SCHEME_NAIVE    one pass per half-step over the whole grid, the
+ *                        straightforward streaming update of Sec. 2, with a
+ *                        grid-wide synchronisation after each;
  *   FDTD_SCHEME_SYSTOLIC one persistent kernel per call in which each CTA
  *                        keeps a subdomain on chip and scans it along the
  *                        x-y-z-t diagonal, exchanging only boundary faces
@@ -168,9 +169,13 @@ fdtd_status fdtd_add_source(fdtd_handle h, int32_t component, int32_t i, int32_t
  * Errors: INVALID_ARG, CUDA. */
 fdtd_status fdtd_write_fields(fdtd_handle h, const float *src);
 
-/* Advance n >= 0 whole steps with the handle's scheme (the naive scheme runs
+/* Advance n >= 0 whole steps with the handle's scheme.  The naive scheme runs
  * a grid of at most 1024 cells in one thread block per call, with block
- * barriers between the half-steps).  Asynchronous:
+ * barriers between the half-steps, a grid whose state is at most twice the
+ * GPU's L2 in one cooperative launch, with grid barriers, and a larger one as
+ * a kernel per half-step.  A systolic handle takes calls of one or two steps
+ * as such a cooperative launch too (the results are the same bits).
+ * Asynchronous:
  * returns once the kernels are enqueued; launch errors are returned here,
  * device-side wait timeouts at the next fdtd_sync / fdtd_read_fields.
  * Errors: INVALID_ARG (n < 0), STATE (an earlier device error not cleared

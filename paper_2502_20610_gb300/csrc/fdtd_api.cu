@@ -22,6 +22,7 @@ constexpr size_t ALIGN = 256;
 constexpr int DEFAULT_SOURCE_STEPS = 65536;
 constexpr int DEFAULT_STEPS_PER_LAUNCH = 1024;
 constexpr unsigned EPOCH_LIMIT = 1u << 30;
+constexpr int CTRL_BARRIER = 16;  // the grid barrier's words among the 64 control words
 
 size_t align_up(size_t x) { return (x + ALIGN - 1) / ALIGN * ALIGN; }
 
@@ -474,10 +475,12 @@ struct fdtd_sim {
     int cap_lo[3] = {0, 0, 0}, cap_hi[3] = {0, 0, 0};
     long long cap_bc = 0, cap_s0 = 0;
     long long launches;
+    int sms;       // of the handle's device
     int max_ctas;
     std::vector<long long> count_le;  // tiles with start <= s
     int dbg_kind;
     long long dbg_ticket, dbg_param, dbg_param2;
+    int dbg_order = 0;  // FDTD_DEBUG_ORDER's order, 0 = the usual one
     bool failed;
     CUtensorMap tm[3][2];  // shell maps of the register kernel
 };
@@ -519,6 +522,48 @@ bool is_device_pointer(const void *p)
         cudaError_t e_ = (x);                                                  \
         if (e_ != cudaSuccess) return cuda_status(e_);                         \
     } while (0)
+
+// One step of the naive schedule on h's state (any scheme: the systolic
+// schedule gives the same bits).
+cudaError_t naive_step(fdtd_sim *h)
+{
+    cudaError_t e = launch_naive_h(h->f, h->fmt, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -(float)h->c.dt, h->sc, h->stream);
+    if (e == cudaSuccess)
+        e = launch_naive_e(h->f, h->fmt, h->ce, h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->step, h->src, h->sc,
+                           h->stream);
+    if (e != cudaSuccess) return e;
+    h->launches += 2;
+    h->step += 1;
+    return e;
+}
+
+// n steps of the naive schedule in one cooperative launch.
+cudaError_t coop_steps(fdtd_sim *h, int n)
+{
+    const double to = std::max(h->c.wait_timeout_s, 2.0);  // a half-step of a large grid takes milliseconds
+    const cudaError_t e = launch_naive_coop(h->f[0], (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb, h->fmt, h->ce,
+                                            h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -(float)h->c.dt, h->step, n,
+                                            h->src, h->sc, h->ctrl + CTRL_BARRIER, h->ctrl + 1, (long long)(to * 1e9),
+                                            h->sms, h->stream);
+    if (e != cudaSuccess) return e;
+    h->launches += 1;
+    h->step += n;
+    return e;
+}
+
+// Does a systolic call of n steps run on the naive kernels instead?  A
+// systolic launch of few steps pays for filling and draining its pipeline of
+// tiles: measured (FP32, us, systolic / naive) for one step 101 / 15 at 64^3,
+// 168 / 22 at 112^3, 253 / 64 at 160^3, 558 / 232 at 256^3, 1562 / 742 at
+// 384^3; for two steps 109 / 29, 180 / 43, 277 / 127, 645 / 463, 2030 / 1482;
+// for three steps 384^3 is about equal (2374 / 2223) and 256^3 near it.  Not
+// under a test hook, while capturing or in cluster pairs, which are the
+// systolic kernel's own.
+bool short_call(const fdtd_sim *h, int64_t n)
+{
+    if (h->cap || h->dbg_kind != FDTD_DEBUG_NONE || h->dbg_order != 0 || h->L.cl != 1) return false;
+    return n <= 2;
+}
 
 fdtd_status upload_tiles(fdtd_sim *h, int order, unsigned seed)
 {
@@ -680,12 +725,13 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
 
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return fail(cuda_status(e));
+    h->sms = sms;
     if (coeffs->scheme == FDTD_SCHEME_SYSTOLIC) {
         e = systolic_configure(L.variant, h->fmt, h->ca != nullptr, L.cl);
-        if (e != cudaSuccess) return fail(cuda_status(e));
-        int dev = 0, sms = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return fail(cuda_status(e));
         if (L.cl == 2) {  // co-resident clusters of two
             const int pairs = systolic_reg_max_pairs(L.variant - 2, h->fmt);
@@ -763,7 +809,9 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src)
                                  h->stream));
         }
     }
-    CK(cudaMemsetAsync(h->ctrl + 1, 0, 3 * sizeof(int), h->stream));
+    // the error word and its details, and the grid barrier (a launch that
+    // timed out may have left arrivals in it)
+    CK(cudaMemsetAsync(h->ctrl + 1, 0, (CTRL_BARRIER + 8 - 1) * sizeof(int), h->stream));
     // S^{n-1} := 0 (both band snapshots: which is "previous" alternates)
     if (h->prev) CK(cudaMemsetAsync(h->ws + h->L.prev, 0, h->L.layer - h->L.prev, h->stream));
     h->failed = false;
@@ -816,13 +864,22 @@ fdtd_status fdtd_step(fdtd_handle h, int64_t n)
             }
             return FDTD_OK;
         }
-        for (int64_t s = 0; s < n; ++s) {
-            CK(launch_naive_h(h->f, h->fmt, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, ndt, h->sc, h->stream));
-            CK(launch_naive_e(h->f, h->fmt, h->ce, h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->step, h->src,
-                              h->sc, h->stream));
-            h->launches += 2;
-            h->step += 1;
+        // one cooperative launch a call while the state (six components and
+        // dt/eps) is at most twice L2, where its barriers cost less than kernel
+        // boundaries: FP32, us a step, 32^3 14.4 -> 6.8, 64^3 14.4 -> 7.7, 112^3
+        // 20.5 -> 16.4, 160^3 57 -> 51; beyond, the pair of kernels is level or
+        // ahead (256^3 222 against 227)
+        const bool coop = (double)cells * (6.0 * h->L.eb + 4.0) <= 256e6;
+        while (coop && n > 0) {
+            const int T = (int)std::min<int64_t>(n, 1 << 20);
+            CK(coop_steps(h, T));
+            n -= T;
         }
+        for (; n > 0; --n) CK(naive_step(h));
+        return FDTD_OK;
+    }
+    if (short_call(h, n)) {  // too few steps to fill the skewed pipeline: the streaming kernels, the same results
+        CK(coop_steps(h, (int)n));
         return FDTD_OK;
     }
     while (n > 0) {
@@ -1150,15 +1207,7 @@ fdtd_status fdtd_adjoint_gradient(fdtd_handle h, const fdtd_overlap_objective *o
     // step unless the register kernel can capture the box) use the naive
     // kernel pair, which the systolic schedule reproduces bit for bit
     const bool reg_kernel = h->c.scheme == FDTD_SCHEME_SYSTOLIC && h->L.variant >= 2;
-    auto one_step = [&]() -> cudaError_t {
-        cudaError_t e = launch_naive_h(h->f, h->fmt, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -dt, h->sc, st);
-        if (e == cudaSuccess)
-            e = launch_naive_e(h->f, h->fmt, h->ce, h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->step, h->src,
-                               h->sc, st);
-        h->launches += 2;
-        h->step += 1;
-        return e;
-    };
+    auto one_step = [&]() -> cudaError_t { return naive_step(h); };
     // m steps of h, the box's E after step r (r = 1..m) into plane p0 + r of
     // buf: captured by the register kernel, or copied after single steps
     auto run_capture = [&](long long m, float *buf, long long p0) -> fdtd_status {
@@ -1287,6 +1336,7 @@ fdtd_status fdtd_debug_set(fdtd_handle h, int32_t kind, int64_t ticket, int64_t 
     if (kind == FDTD_DEBUG_ORDER) {
         if (param < 0 || param > 2) return FDTD_ERR_INVALID_ARG;
         if (h->c.scheme != FDTD_SCHEME_SYSTOLIC) return FDTD_OK;
+        h->dbg_order = (int)param;
         return upload_tiles(h, (int)param, (unsigned)ticket);
     }
     h->dbg_kind = kind;

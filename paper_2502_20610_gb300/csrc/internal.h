@@ -48,6 +48,15 @@ cudaError_t launch_naive_block(void *const f[6], int fmt, const float *ce, const
                                int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src,
                                const Scales &sc, cudaStream_t st);
 
+// Naive scheme, all of `nsteps` steps in one cooperative launch of at most one
+// CTA per SM (`sms`), grid barriers between the half-steps; component c at
+// f + c*fs.  bar: 8 ints of device memory that start at zero and belong to
+// these launches; err: the device error word a barrier sets (and reads) when
+// it waits longer than timeout_ns.
+cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, const float *ca, int nx, int ny, int nz,
+                              int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc,
+                              int *bar, int *err, long long timeout_ns, int sms, cudaStream_t st);
+
 // FP32 <-> storage conversion of one component (convert.cu): `dense` holds
 // nx*ny*nz values, `pitched` rows of `pitch` elements.
 cudaError_t launch_to_storage(void *pitched, const float *dense, int storage, int nx, int ny, int nz, int pitch,

@@ -10,6 +10,7 @@
 // Fields are stored as FP32, FP16 or BF16 (storage.cuh); arithmetic is FP32.
 #include "internal.h"
 #include "storage.cuh"
+#include "sys_common.cuh"
 #include "yee_cell.cuh"
 
 namespace {
@@ -57,12 +58,12 @@ __global__ void __launch_bounds__(NAIVE_BX *NAIVE_BY)
 naive_e_kernel(typename S::T *__restrict__ ex_, typename S::T *__restrict__ ey_, typename S::T *__restrict__ ez_,
                typename S::T *__restrict__ hx_, typename S::T *__restrict__ hy_, typename S::T *__restrict__ hz_,
                const float *__restrict__ ce_, const float *__restrict__ ca_, int nx, int ny, int nz, int pitch,
-               long long step, const SrcSet src, const Scales sc)
+               long long step, const SrcSet src, const Scales sc, bool back)
 {
     using T = typename S::T;
     const int i = blockIdx.x * NAIVE_BX + threadIdx.x;
     const int j = blockIdx.y * NAIVE_BY + threadIdx.y;
-    const int k0 = blockIdx.z * NAIVE_KZ;
+    const int k0 = (back ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * NAIVE_KZ;
     if (i >= nx || j >= ny || k0 >= nz) return;
     const int k1 = min(k0 + NAIVE_KZ, nz);
     const long long sxy = (long long)pitch * ny;
@@ -162,10 +163,160 @@ naive_block_kernel(typename S::T *__restrict__ ex_, typename S::T *__restrict__ 
     }
 }
 
+// Mid-size domains: all the steps of a call in one cooperative launch, one
+// CTA per SM, with a grid barrier after each half-step in place of a kernel
+// boundary.  Bounded by the barriers (about 2 us each) on small grids and by
+// L2 bandwidth on larger ones; a pair of launches a step costs 14 us however
+// small the grid.  A warp takes 32 consecutive x of kz rows in z (z neighbours
+// in registers), the warps of a CTA consecutive y, so neighbour rows are
+// L1 hits.  Loads are plain (coherent): the barrier's acquire orders them
+// after the other CTAs' stores.
+constexpr int COOP_NT = 1024;
+
+// Grid barrier: count of arrivals in bar[0], generation in bar[4]; the last
+// arrival resets the count and bumps the generation, so a launch needs no
+// state from the host.  Bounded wait; false (in every thread) past it.
+__device__ bool grid_barrier(int *bar, unsigned &gen, int *err, long long timeout_ns)
+{
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int good = 1;
+        unsigned *const g = reinterpret_cast<unsigned *>(bar + 4);
+        __threadfence();
+        if (atomicAdd(bar, 1) == (int)gridDim.x - 1) {
+            *reinterpret_cast<volatile int *>(bar) = 0;
+            sysc::st_release(g, gen + 1u);
+        } else {
+            const unsigned long long t0 = sysc::globaltimer();
+            while (sysc::ld_acquire(g) == gen) {
+                if (sysc::ld_volatile(err) != DEV_OK) {
+                    good = 0;
+                    break;
+                }
+                if (sysc::globaltimer() - t0 > (unsigned long long)timeout_ns) {
+                    atomicCAS(err, DEV_OK, DEV_ERR_TIMEOUT);
+                    good = 0;
+                    break;
+                }
+            }
+        }
+        ok = good;
+    }
+    ++gen;
+    __syncthreads();
+    return ok != 0;
+}
+
+template <class S, bool LOSSY>
+__global__ void __launch_bounds__(COOP_NT, 1)
+naive_coop_kernel(typename S::T *f, long long fs, const float *__restrict__ ce_, const float *__restrict__ ca_, int nx,
+                  int ny, int nz, int pitch, int kz, float ndt, long long step0, int nsteps, const SrcSet src,
+                  const Scales sc, bool back, int *bar, int *err, long long timeout_ns)
+{
+    using T = typename S::T;
+    T *const ex_ = f, *const ey_ = f + fs, *const ez_ = f + 2 * fs, *const hx_ = f + 3 * fs, *const hy_ = f + 4 * fs,
+             *const hz_ = f + 5 * fs;
+    unsigned gen = 0;
+    if (threadIdx.x == 0) gen = sysc::ld_acquire(reinterpret_cast<unsigned *>(bar + 4));
+    const int lane = threadIdx.x & 31;
+    const int nxc = (nx + 31) / 32, nzc = (nz + kz - 1) / kz;
+    const long long items = (long long)nxc * ny * nzc, stride = (long long)gridDim.x * (COOP_NT / 32);
+    const long long first = (long long)blockIdx.x * (COOP_NT / 32) + (threadIdx.x >> 5);
+    const long long last = first + (items - 1 - first) / stride * stride;  // of this warp (if it has any)
+    const long long sxy = (long long)pitch * ny;
+    auto place = [&](long long it, int &i, int &j, int &k0) {
+        j = (int)(it % ny);
+        const int r = (int)(it / ny);
+        i = (r % nxc) * 32 + lane;
+        k0 = (r / nxc) * kz;
+    };
+    for (int s = 0; s < nsteps; ++s) {
+        for (long long it = first; it < items; it += stride) {
+            int i, j, k0;
+            place(it, i, j, k0);
+            if (i >= nx) continue;
+            const int k1 = min(k0 + kz, nz);
+            const bool ip = i + 1 < nx, jp = j + 1 < ny;
+            long long p = i + (long long)pitch * (j + (long long)ny * k0);
+            float exc = S::dec(ex_[p], sc.s[0]), eyc = S::dec(ey_[p], sc.s[1]);
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k, p += sxy) {
+                const bool kp = k + 1 < nz;
+                const float exn = kp ? S::dec(ex_[p + sxy], sc.s[0]) : 0.f;
+                const float eyn = kp ? S::dec(ey_[p + sxy], sc.s[1]) : 0.f;
+                const float ez = S::dec(ez_[p], sc.s[2]);
+                const float ez_ip = ip ? S::dec(ez_[p + 1], sc.s[2]) : 0.f;
+                const float ey_ip = ip ? S::dec(ey_[p + 1], sc.s[1]) : 0.f;
+                const float ez_jp = jp ? S::dec(ez_[p + pitch], sc.s[2]) : 0.f;
+                const float ex_jp = jp ? S::dec(ex_[p + pitch], sc.s[0]) : 0.f;
+                const float hx = S::dec(hx_[p], sc.s[3]), hy = S::dec(hy_[p], sc.s[4]), hz = S::dec(hz_[p], sc.s[5]);
+                hx_[p] = S::enc(h_x(hx, ez_jp, ez, eyn, eyc, ndt), sc.is[3]);
+                hy_[p] = S::enc(h_y(hy, exn, exc, ez_ip, ez, ndt), sc.is[4]);
+                hz_[p] = S::enc(h_z(hz, ey_ip, eyc, ex_jp, exc, ndt), sc.is[5]);
+                exc = exn;
+                eyc = eyn;
+            }
+        }
+        if (!grid_barrier(bar, gen, err, timeout_ns)) return;
+        const long long step = step0 + s;
+        for (long long q = first; q < items; q += stride) {
+            const long long it = back ? last - (q - first) : q;
+            int i, j, k0;
+            place(it, i, j, k0);
+            if (i >= nx) continue;
+            const int k1 = min(k0 + kz, nz);
+            long long p = i + (long long)pitch * (j + (long long)ny * k0);
+            float hxm = k0 > 0 ? S::dec(hx_[p - sxy], sc.s[3]) : 0.f;
+            float hym = k0 > 0 ? S::dec(hy_[p - sxy], sc.s[4]) : 0.f;
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k, p += sxy) {
+                const float hx = S::dec(hx_[p], sc.s[3]), hy = S::dec(hy_[p], sc.s[4]), hz = S::dec(hz_[p], sc.s[5]);
+                const float hz_jm = j > 0 ? S::dec(hz_[p - pitch], sc.s[5]) : 0.f;
+                const float hx_jm = j > 0 ? S::dec(hx_[p - pitch], sc.s[3]) : 0.f;
+                const float hz_im = i > 0 ? S::dec(hz_[p - 1], sc.s[5]) : 0.f;
+                const float hy_im = i > 0 ? S::dec(hy_[p - 1], sc.s[4]) : 0.f;
+                const float ce = __ldg(ce_ + p);
+                const float ca = LOSSY ? __ldg(ca_ + p) : 1.f;
+                float ex = S::dec(ex_[p], sc.s[0]), ey = S::dec(ey_[p], sc.s[1]), ez = S::dec(ez_[p], sc.s[2]);
+                if (j > 0 && k > 0) ex = e_x(decay<LOSSY>(ca, ex), hz, hz_jm, hy, hym, ce);
+                if (i > 0 && k > 0) ey = e_y(decay<LOSSY>(ca, ey), hx, hxm, hz, hz_im, ce);
+                if (i > 0 && j > 0) ez = e_z(decay<LOSSY>(ca, ez), hy, hy_im, hx, hx_jm, ce);
+                for (int q = 0; q < src.n; ++q) {
+                    const SrcDesc &d = src.s[q];
+                    if (d.idx == p && step < d.n_amp) {
+                        const float a = S::src_amp(d.amp[step], sc.src);
+                        if (d.comp == 0) ex = add_source(ex, a);
+                        else if (d.comp == 1) ey = add_source(ey, a);
+                        else ez = add_source(ez, a);
+                    }
+                }
+                ex_[p] = S::enc(ex, sc.is[0]);
+                ey_[p] = S::enc(ey, sc.is[1]);
+                ez_[p] = S::enc(ez, sc.is[2]);
+                hxm = hx;
+                hym = hy;
+            }
+        }
+        if (s + 1 < nsteps && !grid_barrier(bar, gen, err, timeout_ns)) return;
+    }
+}
+
 dim3 naive_grid(int nx, int ny, int nz)
 {
     return dim3((nx + NAIVE_BX - 1) / NAIVE_BX, (ny + NAIVE_BY - 1) / NAIVE_BY,
                 (nz + NAIVE_KZ - 1) / NAIVE_KZ);
+}
+
+// Does the E half-step sweep the grid backwards, from what the H half-step
+// touched last?  It finds that part in L2 when the state does not fit there:
+// measured, FP32 (the pair of kernels) 160^3 64 -> 57 us a step, 256^3
+// 232 -> 222, 384^3 742 -> 738; FP16 256^3 197 -> 182.  A state of less than
+// 96 MB (six components and dt/eps) is in L2 either way, and the forward
+// sweep is then as fast or faster (FP16 160^3 33 us against 37).
+bool e_backwards(size_t eb, int nx, int ny, int nz)
+{
+    return (double)nx * ny * nz * (6.0 * eb + 4.0) > 96e6;
 }
 
 template <class S>
@@ -186,11 +337,11 @@ cudaError_t launch_e(void *const f[6], const float *ce, const float *ca, int nx,
     if (ca)
         naive_e_kernel<S, true><<<naive_grid(nx, ny, nz), dim3(NAIVE_BX, NAIVE_BY), 0, st>>>(
             (T *)f[0], (T *)f[1], (T *)f[2], (T *)f[3], (T *)f[4], (T *)f[5], ce, ca, nx, ny, nz, pitch, step, src,
-            sc);
+            sc, e_backwards(sizeof(T), nx, ny, nz));
     else
         naive_e_kernel<S, false><<<naive_grid(nx, ny, nz), dim3(NAIVE_BX, NAIVE_BY), 0, st>>>(
             (T *)f[0], (T *)f[1], (T *)f[2], (T *)f[3], (T *)f[4], (T *)f[5], ce, ca, nx, ny, nz, pitch, step, src,
-            sc);
+            sc, e_backwards(sizeof(T), nx, ny, nz));
     return cudaGetLastError();
 }
 
@@ -212,7 +363,52 @@ cudaError_t launch_block(void *const f[6], const float *ce, const float *ca, int
     return cudaGetLastError();
 }
 
+template <class S, bool LOSSY>
+cudaError_t launch_coop(void *f, long long fs, const float *ce, const float *ca, int nx, int ny, int nz, int pitch,
+                        float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc, int *bar, int *err,
+                        long long timeout_ns, int sms, cudaStream_t st)
+{
+    using T = typename S::T;
+    // rows in z per warp: the fewest row steps on the busiest warp, a column's
+    // start (its two z-neighbour loads) counted as half a row; a remainder
+    // round of full-height columns would double a half-step
+    const long long rows = (long long)((nx + 31) / 32) * ny, warps = (long long)sms * (COOP_NT / 32);
+    int kz = 1;
+    double least = 0.0;
+    for (int k = 1; k <= std::min(nz, 24); ++k) {
+        const double cost = (double)((rows * ((nz + k - 1) / k) + warps - 1) / warps) * (k + 0.5);
+        if (k == 1 || cost < least) {
+            least = cost;
+            kz = k;
+        }
+    }
+    const long long items = rows * ((nz + kz - 1) / kz);
+    const int grid = (int)std::min<long long>(sms, (items + COOP_NT / 32 - 1) / (COOP_NT / 32));
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(COOP_NT);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, naive_coop_kernel<S, LOSSY>, (T *)f, fs, ce, ca, nx, ny, nz, pitch, kz, neg_dt, step0,
+                              nsteps, src, sc, e_backwards(sizeof(T), nx, ny, nz), bar, err, timeout_ns);
+}
+
 } // namespace
+
+cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, const float *ca, int nx, int ny, int nz,
+                              int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc,
+                              int *bar, int *err, long long timeout_ns, int sms, cudaStream_t st)
+{
+    if (ca)
+        DISPATCH_FORMAT(fmt, S, launch_coop<S, true>(f, fs, ce, ca, nx, ny, nz, pitch, neg_dt, step0, nsteps, src, sc, bar,
+                                                     err, timeout_ns, sms, st));
+    DISPATCH_FORMAT(fmt, S, launch_coop<S, false>(f, fs, ce, ca, nx, ny, nz, pitch, neg_dt, step0, nsteps, src, sc, bar, err,
+                                                  timeout_ns, sms, st));
+}
 
 int naive_block_max_cells() { return NAIVE_BLOCK_CELLS; }
 
