@@ -1094,14 +1094,37 @@ fdtd_status fdtd_learned_record(fdtd_handle h, const int32_t lo[3], const int32_
                                std::min(z - lo[2], hi[2] - 1 - z));
         return d < thickness;
     };
-    std::vector<int> pick(3 * (size_t)per_step);
-    CK(cudaMemcpyAsync(prev, f0, 6 * arr, cudaMemcpyDeviceToDevice, h->stream));
+    // the box of S^{n-1} and S^n, taken in turn: a step copies the new box
+    // over the oldest one (the whole state, copied twice a step, was 6x
+    // the traffic of the box at its usual size)
+    const size_t per = 3 * (size_t)per_step;
+    CK(mlp_record_box(f0, fs, h->L.pitch, h->g.ny, ilo, ihi, prev, h->stream));
     fdtd_status st = fdtd_step(h, 1);
     if (st != FDTD_OK) return st;
-    CK(cudaMemcpyAsync(cur, f0, 6 * arr, cudaMemcpyDeviceToDevice, h->stream));
+    CK(mlp_record_box(f0, fs, h->L.pitch, h->g.ny, ilo, ihi, cur, h->stream));
+    // the cells of a step are drawn while the GPU runs the steps before it:
+    // a ring of host lists, one taken again once its copy is done
+    constexpr int RING = 4;
+    struct Ring {
+        std::vector<int> pick[RING];
+        cudaEvent_t copied[RING] = {};
+        cudaStream_t stream;
+        ~Ring()
+        {
+            cudaStreamSynchronize(stream);  // no copy out of `pick` is in flight any more
+            for (cudaEvent_t e : copied)
+                if (e) cudaEventDestroy(e);
+        }
+    } ring;
+    ring.stream = h->stream;
     for (int s = 0; s < n_steps; ++s) {
         st = fdtd_step(h, 1);
         if (st != FDTD_OK) return st;
+        const int r = s % RING;
+        if (ring.copied[r]) CK(cudaEventSynchronize(ring.copied[r]));
+        else CK(cudaEventCreateWithFlags(&ring.copied[r], cudaEventDisableTiming));
+        std::vector<int> &pick = ring.pick[r];
+        pick.resize(per);
         for (int q = 0; q < per_step; ++q) {
             int x, y, z;
             do {
@@ -1109,17 +1132,17 @@ fdtd_status fdtd_learned_record(fdtd_handle h, const int32_t lo[3], const int32_
                 y = lo[1] + (int)(rng() % (unsigned long long)(hi[1] - lo[1]));
                 z = lo[2] + (int)(rng() % (unsigned long long)(hi[2] - lo[2]));
             } while (!in_layer(x, y, z));
-            pick[3 * q] = x;
-            pick[3 * q + 1] = y;
-            pick[3 * q + 2] = z;
+            pick[3 * (size_t)q] = x;
+            pick[3 * (size_t)q + 1] = y;
+            pick[3 * (size_t)q + 2] = z;
         }
-        CK(cudaMemcpyAsync(cells, pick.data(), sizeof(int) * pick.size(), cudaMemcpyHostToDevice, h->stream));
+        CK(cudaMemcpyAsync(cells, pick.data(), sizeof(int) * per, cudaMemcpyHostToDevice, h->stream));
+        CK(cudaEventRecord(ring.copied[r], h->stream));
         CK(mlp_record(prev, cur, f0, fs, h->L.pitch, h->g.ny, ilo, ihi, cells, per_step, h->ce, h->ca,
                       -(float)h->c.dt, d_x + (size_t)s * per_step * mlpnet::NI,
                       d_y + (size_t)s * per_step * mlpnet::NO, h->stream));
-        CK(cudaMemcpyAsync(prev, cur, 6 * arr, cudaMemcpyDeviceToDevice, h->stream));
-        CK(cudaMemcpyAsync(cur, f0, 6 * arr, cudaMemcpyDeviceToDevice, h->stream));
-        CK(cudaStreamSynchronize(h->stream));  // the host cell list is reused next step
+        CK(mlp_record_box(f0, fs, h->L.pitch, h->g.ny, ilo, ihi, prev, h->stream));
+        std::swap(prev, cur);
     }
     return fdtd_sync(h);
 }

@@ -497,45 +497,78 @@ __device__ void yee_centre(const float *v, float ndt, float cb, float ca, bool l
     out[5] = hz;
 }
 
+// The six components of the box [lo, hi) into dst [6][box cells] (x fastest).
+__global__ void __launch_bounds__(256) record_box_kernel(const float *__restrict__ f, long long fstride, int pitch,
+                                                         int ny, int3 lo, int3 hi, float *__restrict__ dst)
+{
+    const int bx = hi.x - lo.x, by = hi.y - lo.y;
+    const long long bc = (long long)bx * by * (hi.z - lo.z);
+    const long long q = blockIdx.x * 256ll + threadIdx.x;
+    if (q >= bc) return;
+    const int i = lo.x + (int)(q % bx), j = lo.y + (int)((q / bx) % by), k = lo.z + (int)(q / ((long long)bx * by));
+    const long long p = i + (long long)pitch * (j + (long long)ny * k);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) dst[c * bc + q] = f[c * fstride + p];
+}
+
 // Training pairs from a reference run: for cells (x,y,z) of the layer region
 // (inside the box [lo, hi) of the reference grid), the normalised stencil of
 // (S^n, S^{n-1}) -- cells outside the box read 0, as they would at a wall --
 // and the normalised correction (S^{n+1} - Yee_box(S^n))(centre) / r that
-// takes the box's own Yee step to the reference's next state.
-__global__ void __launch_bounds__(256) record_kernel(const float *__restrict__ prev, const float *__restrict__ cur,
-                                                     const float *__restrict__ nxt, long long fstride, int pitch,
-                                                     int ny, int3 lo, int3 hi, const int *__restrict__ cells, int n,
-                                                     const float *__restrict__ ce, const float *__restrict__ ca,
-                                                     float ndt, float *__restrict__ X, float *__restrict__ Y)
+// takes the box's own Yee step to the reference's next state.  cur and prev
+// hold the box alone ([6][box cells]), nxt the whole reference state.
+// One warp per sample: a thread per sample left 4 CTAs to write 1.3 kB rows
+// 32 rows apart (267 us for 1000 samples); a warp writes its row in whole
+// lines and sums the squares with shuffles.  Bounded by the latency of the
+// gather (the box is in L2).
+constexpr int RW = 8;  // samples (warps) per CTA
+__global__ void __launch_bounds__(32 * RW) record_kernel(const float *__restrict__ prev, const float *__restrict__ cur,
+                                                         const float *__restrict__ nxt, long long fstride, int pitch,
+                                                         int ny, int3 lo, int3 hi, const int *__restrict__ cells, int n,
+                                                         const float *__restrict__ ce, const float *__restrict__ ca,
+                                                         float ndt, float *__restrict__ X, float *__restrict__ Y)
 {
-    const int q = blockIdx.x * 256 + threadIdx.x;
+    __shared__ float raw[RW][NI];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int q = blockIdx.x * RW + w;
     if (q >= n) return;
     const int x = cells[3 * q], y = cells[3 * q + 1], z = cells[3 * q + 2];
-    float *xo = X + (long long)q * NI;
+    const int bx = hi.x - lo.x, by = hi.y - lo.y;
+    const long long bc = (long long)bx * by * (hi.z - lo.z);
     double ss = 0.0;
-    for (int s = 0; s < 2; ++s) {
-        const float *F = s == 0 ? cur : prev;
-        for (int c = 0; c < 6; ++c)
-            for (int d = 0; d < 27; ++d) {
-                const int xx = x + d % 3 - 1, yy = y + (d / 3) % 3 - 1, zz = z + d / 9 - 1;
-                float v = 0.f;
-                if (xx >= lo.x && xx < hi.x && yy >= lo.y && yy < hi.y && zz >= lo.z && zz < hi.z)
-                    v = F[c * fstride + xx + (long long)pitch * (yy + (long long)ny * zz)];
-                xo[(s * 6 + c) * 27 + d] = v;
-                ss += (double)v * v;
-            }
+#pragma unroll
+    for (int u = 0; u < (NI + 31) / 32; ++u) {
+        const int k = lane + 32 * u;
+        if (k < NI) {
+            const int d = k % 27, c = (k / 27) % 6;
+            const int xx = x + d % 3 - 1, yy = y + (d / 3) % 3 - 1, zz = z + d / 9 - 1;
+            float v = 0.f;
+            if (xx >= lo.x && xx < hi.x && yy >= lo.y && yy < hi.y && zz >= lo.z && zz < hi.z)
+                v = (k < NI / 2 ? cur : prev)[c * bc + (xx - lo.x) + (long long)bx * ((yy - lo.y) + (long long)by * (zz - lo.z))];
+            raw[w][k] = v;
+            ss += (double)v * v;
+        }
     }
-    const long long p = x + (long long)pitch * (y + (long long)ny * z);
-    float yee[6];
-    yee_centre(xo, ndt, ce[p], ca ? ca[p] : 1.f, ca != nullptr, x == lo.x, y == lo.y, z == lo.z, yee);
+    for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
+    __syncwarp();
     // r below R_MIN counts as a zero stencil (its reciprocal would overflow
     // FP32): the pair is recorded as zeros
     const double r = sqrt(ss / NI);
     const double ir = r >= (double)R_MIN ? 1.0 / r : 0.0;
-    for (int k = 0; k < NI; ++k) xo[k] = (float)(xo[k] * ir);
+    float *xo = X + (long long)q * NI;
+#pragma unroll
+    for (int u = 0; u < (NI + 31) / 32; ++u) {
+        const int k = lane + 32 * u;
+        if (k < NI) xo[k] = (float)(raw[w][k] * ir);
+    }
+    const long long p = x + (long long)pitch * (y + (long long)ny * z);
+    float yee[6];  // every lane the same values; lane c writes component c
+    yee_centre(raw[w], ndt, ce[p], ca ? ca[p] : 1.f, ca != nullptr, x == lo.x, y == lo.y, z == lo.z, yee);
     const unsigned m = tangent_mask(x - lo.x, y - lo.y, z - lo.z, hi.x - lo.x, hi.y - lo.y, hi.z - lo.z);
+#pragma unroll
     for (int c = 0; c < 6; ++c)
-        Y[(long long)q * NO + c] = (m >> c) & 1u ? (float)(((double)nxt[c * fstride + p] - (double)yee[c]) * ir) : 0.f;
+        if (lane == c)
+            Y[(long long)q * NO + c] = (m >> c) & 1u ? (float)(((double)nxt[c * fstride + p] - (double)yee[c]) * ir) : 0.f;
 }
 
 // -------------------------------------------------- layer update (fused)
@@ -918,8 +951,18 @@ cudaError_t mlp_record(const float *prev, const float *cur, const float *nxt, lo
                        float neg_dt, float *X, float *Y, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    record_kernel<<<(n + 255) / 256, 256, 0, st>>>(prev, cur, nxt, fstride, pitch, ny, make_int3(lo[0], lo[1], lo[2]),
-                                                    make_int3(hi[0], hi[1], hi[2]), cells, n, ce, ca, neg_dt, X, Y);
+    record_kernel<<<(n + RW - 1) / RW, 32 * RW, 0, st>>>(prev, cur, nxt, fstride, pitch, ny,
+                                                         make_int3(lo[0], lo[1], lo[2]), make_int3(hi[0], hi[1], hi[2]),
+                                                         cells, n, ce, ca, neg_dt, X, Y);
+    return cudaGetLastError();
+}
+
+cudaError_t mlp_record_box(const float *f, long long fstride, int pitch, int ny, const int lo[3], const int hi[3],
+                           float *dst, cudaStream_t st)
+{
+    const long long bc = (long long)(hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2]);
+    record_box_kernel<<<(unsigned)((bc + 255) / 256), 256, 0, st>>>(f, fstride, pitch, ny, make_int3(lo[0], lo[1], lo[2]),
+                                                                     make_int3(hi[0], hi[1], hi[2]), dst);
     return cudaGetLastError();
 }
 

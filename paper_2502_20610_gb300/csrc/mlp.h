@@ -20,6 +20,11 @@ cudaError_t mlp_grad(const float *params, const float *X, const float *T, int n,
                      void *scratch, int batch, cudaStream_t st);
 cudaError_t mlp_train(float *params, const float *X, const float *T, long long n, int batch, int epochs, double lr,
                       unsigned long long seed, void *scratch, cudaStream_t st, double *last_epoch_loss);
+// The box [lo, hi) of a state (six components at f + c*fstride, rows of
+// `pitch`) into dst [6][box cells], and the pairs of `n` of its cells from two
+// such copies (S^{n-1}, S^n) and the whole state S^{n+1}.
+cudaError_t mlp_record_box(const float *f, long long fstride, int pitch, int ny, const int lo[3], const int hi[3],
+                           float *dst, cudaStream_t st);
 // ce, ca (nullable): the reference's E coefficients, for the box's own Yee
 // step of each recorded cell.
 cudaError_t mlp_record(const float *prev, const float *cur, const float *nxt, long long fstride, int pitch, int ny,
