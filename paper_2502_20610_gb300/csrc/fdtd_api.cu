@@ -141,7 +141,7 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     L.xface = L.yface = off;
     if (c.scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(c) >= 2) {
         const int tz = systolic_shape(pick_variant(c)).tz;
-        L.nzblk = ceil_div(g.nz, tz);
+        L.nzblk = ceil_div((long long)g.nz + tz - 1, tz);  // columns are stored whole: see the kernel
         L.nzb = L.nzblk * face_block(tz, L.eb);
         const size_t per = align_up((size_t)L.eb * (size_t)g.nx * g.ny * (size_t)L.nzb);
         L.fxs = L.fys = (long long)(per / L.eb);

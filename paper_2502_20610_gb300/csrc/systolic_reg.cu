@@ -36,18 +36,25 @@
 // a place that stays fixed for the whole life of the tile.  So the lane
 // leaving the box in x and the warp leaving it in y store their whole columns
 // with 16-byte stores, and the x lane and the y-shell warp refill theirs
-// with 16-byte shared loads.  The period is at least the grid's z extent, so
-// a wrapped position is next written only by a tile downwind of every reader
-// of the value there; rows outside the domain are neither stored nor kept
-// from a refill.
+// with 16-byte shared loads.  Columns are stored and read whole, rows outside
+// the grid in z included (their E is 0, see below): the period is a tile's z
+// extent longer than the grid, so that no tile's rows share a block with
+// another's that are still to be read, and a wrapped position is next written
+// only by a tile downwind of every reader of the value there (the CPU model
+// checks both).
 //
-// The warp whose y slot is outside the box sits out both half-steps, so it
-// carries the tile's bookkeeping: after the second barrier it publishes the
-// tile's own level t-1, then polls the upwind tiles' progress once for level
-// t+1 and, if they have published it, fetches those shells into the second
-// staging buffer.  Only when that poll failed (or on a tile's first
-// step) does warp 0 wait for the upwind tiles at the start of the step, and
-// thread 0 fetch the shells then.
+// Bookkeeping: a warp of its own polls the upwind tiles, fetches the next
+// step's shells as soon as their staging buffer is free, and publishes the
+// tile's levels.  While the warp whose y slot is outside the box did this
+// between its refills, its chain of stores, release, poll and copies (3100 of
+// 9500 cycles) was as long as the other warps' half-steps and stores.
+//
+// Code size: the step is some 3500 instructions long, and what lies between
+// is fetched with it.  Taking the cold paths out of the loop (row-by-row
+// stores and clearing at the grid's ends in z, masks of the H half-step, the
+// launch's last step, the capture box, a search for a source's row) gave
+// 172.8 -> 193 GCUPS at 256^3 and 180 -> 196 at 512^3 before the bookkeeping
+// warp, which gave 201 and 216 (FP16 at 256^3: 163 -> 188).
 //
 // Top faces: the z face goes to the field arrays at the end of each step;
 // the y face goes to the y-face buffer one step late, from the warp whose y
@@ -57,10 +64,12 @@
 // the E rows are exchanged for the H half-step, and after the H rows are
 // exchanged for the E half-step.
 //
-// Tile: 31 x 15 x NZ updated cells.  A step whose box lies inside the domain
-// and clear of the low walls (most steps of a large grid) runs both
-// half-steps with no per-cell masks.  Every arithmetic step is yee_cell.cuh,
-// so the result equals the naive schedule bit for bit.
+// Masks: none but the low walls'.  A cell outside the domain has dt/eps = 0
+// (the coefficient shells are zero-filled there), so its E stays 0; its H is
+// only read by such cells and by the tangential E of the low walls, which
+// stays as it is (the masked form of the E half-step, on steps whose box
+// touches a low wall).  Every arithmetic step is yee_cell.cuh, so the result
+// equals the naive schedule bit for bit.
 //
 // Storage: fields live in global memory as FP32, FP16 or BF16 (S, see
 // storage.cuh); registers hold FP32 values already rounded to the storage
@@ -78,10 +87,11 @@ namespace {
 
 using namespace sysc;
 
-template <int NZ_, class S_, bool LOSSY_, int TY_, int CL_ = 1>
+template <int NZ_, class S_, bool LOSSY_, int TY_, int CL_ = 1, bool CAP_ = false>
 struct RegTile {
     using S = S_;
     static constexpr bool LOSSY = LOSSY_;  // conducting cells: E <- ca E + cb curl H
+    static constexpr bool CAP = CAP_;      // the adjoint's launches: store the capture box's E every step
     // CTAs per thread-block cluster along x: 2 = pairs of x-adjacent tiles,
     // the upwind one sending its top x face through distributed shared memory
     static constexpr int CL = CL_;
@@ -89,7 +99,12 @@ struct RegTile {
     using T = typename S_::T;
     static constexpr int NZ = NZ_;        // updated z rows (registers 0..NZ-1)
     static constexpr int NR = NZ_ + 1;    // plus the shell row -1
-    static constexpr int RY = 16, NT = 32 * RY;
+    static constexpr int RY = 16, NTC = 32 * RY;  // y slots = compute warps
+    // and a warpgroup for the bookkeeping (one warp of it works), whose registers
+    // the compute warps take over: 640 * 96 = 512 * 112 + 128 * 32
+    static constexpr int NT = NTC + 128;
+    static constexpr int CREG = 112, BREG = 32;
+    static_assert(NTC * CREG + (NT - NTC) * BREG <= NT * 96, "within the launch's registers");
     // TY = RY - 1: one y slot outside the box, the y shell (its warp also
     // holds the previous step's top y row until its refill); TY = RY - 2:
     // the previous top row has a slot (and warp) of its own
@@ -128,21 +143,26 @@ struct RegTile {
     static constexpr int ZBC = RY * SWC, YBC = NR * SWC, XBC = NR * 16 * XAC;
     static constexpr int NCOEF = LOSSY ? 2 : 1;   // FP32 coefficient arrays: cb (dt/eps), ca
     static constexpr size_t r128(size_t b) { return (b + 127) / 128 * 128; }
-    // byte offsets of the shells within one staging buffer
+    // byte offsets of the shells within one staging buffer: of the fields, and of
+    // the coefficients
     static constexpr size_t OFF_Y = r128(6 * (size_t)ZB * EB);
     static constexpr size_t OFF_X = OFF_Y + r128(6 * (size_t)YB * EB);
-    static constexpr size_t OFF_ZC = OFF_X + r128(6 * (size_t)XB * EB);
-    static constexpr size_t OFF_YC = OFF_ZC + r128(NCOEF * 4 * (size_t)ZBC);
+    static constexpr size_t STG_B = OFF_X + r128(6 * (size_t)XB * EB);
+    static constexpr size_t OFF_YC = r128(NCOEF * 4 * (size_t)ZBC);
     static constexpr size_t OFF_XC = OFF_YC + r128(NCOEF * 4 * (size_t)YBC);
-    static constexpr unsigned TMA_BYTES =
-        6u * EB * (ZB + YB + XB) + NCOEF * 4u * (ZBC + YBC + XBC);
-    static constexpr int CR = 16;                 // coefficient ring rows (>= NR, power of 2)
+    static constexpr size_t COF_B = OFF_XC + r128(NCOEF * 4 * (size_t)XBC);
+    static constexpr unsigned FIELD_BYTES = 6u * EB * (ZB + YB + XB), COEF_BYTES = NCOEF * 4u * (ZBC + YBC + XBC);
+    // staging buffers: two, so that a step's shells are fetched during the step
+    // before.  The lossy form's second coefficient leaves room for one buffer of
+    // coefficients beside the two of fields, on a barrier of its own: coefficients
+    // are read before B2 only, so they are fetched from B2 on, and need no upwind
+    // tile.  (One buffer for everything, fetched from B1 on, left the copies'
+    // latency in every step: 224^3 FP32, 130 -> 162 GCUPS.)
+    static constexpr int NCBUF = LOSSY_ ? 1 : 2;
+    // coefficient ring rows: a power of two, or (lossy, for room) just a column
+    static constexpr int CR = LOSSY_ ? NR : 16;
     static constexpr int CE_F = RY * CR * 32;
     static_assert(CR >= NR, "coefficient ring holds the whole column");
-    // staging buffers: two (the next step's shells are fetched during this
-    // step) unless the lossy form's second coefficient set leaves no room
-    static constexpr int NBUF = LOSSY_ ? 1 : 2;
-    static constexpr size_t STG_B = OFF_XC + r128(NCOEF * 4 * (size_t)XBC);  // one buffer, bytes
     // x pairs: the downwind tile's receive ring of x faces, NSLOT slots of
     // [field][box row y][z-block] (rows 1..NZ of the x shell of one step)
     static constexpr int NSLOT = 6;
@@ -150,11 +170,16 @@ struct RegTile {
     static constexpr size_t RX_B = CL_ == 2 ? NSLOT * (size_t)RXS * EB : 0;
     static constexpr size_t smem_bytes()
     {
-        return NBUF * STG_B + sizeof(float) * (4 * (size_t)XE_F + NCOEF * (size_t)CE_F) + RX_B;
+        return 2 * STG_B + NCBUF * COF_B + sizeof(float) * (4 * (size_t)XE_F + NCOEF * (size_t)CE_F) + RX_B;
     }
 };
 
 __device__ __forceinline__ float shfl_from(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// Named barriers: the compute warps among themselves (16 warps), and with the
+// bookkeeping warp at a tile's start.
+__device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+__device__ __forceinline__ void bar_tile() { asm volatile("bar.sync 2, 544;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -186,10 +211,7 @@ __device__ __forceinline__ void st4(typename S::T *p, float is, float a, float b
     }
 }
 
-// Rows 1..NZ of one field of a column: loaded from a z-block, and stored into
-// one.  A store writes only the rows whose physical z (z0 + i - 1) lies in
-// the domain: with whole 16-byte chunks when all of them do, else row by row
-// (face-buffer positions of rows outside the domain belong to other cells).
+// Rows 1..NZ of one field of a column, loaded from a z-block and stored into one.
 template <class S, int NR>
 __device__ __forceinline__ void ld_rows(const typename S::T *p, float s, float (&v)[NR])
 {
@@ -198,17 +220,11 @@ __device__ __forceinline__ void ld_rows(const typename S::T *p, float s, float (
 }
 
 template <class S, int NR>
-__device__ __forceinline__ void st_rows(typename S::T *p, float is, const float (&v)[NR], int z0, int nz)
+__device__ __forceinline__ void st_rows(typename S::T *p, float is, const float (&v)[NR])
 {
-    if (z0 >= 0 && z0 + NR - 1 <= nz) {
 #pragma unroll
-        for (int q = 0; q < (NR - 1) / 4; ++q)
-            st4<S>(p + 4 * q, is, v[4 * q + 1], v[4 * q + 2], v[4 * q + 3], v[4 * q + 4]);
-    } else {
-#pragma unroll
-        for (int i = 1; i < NR; ++i)
-            if ((unsigned)(z0 + i - 1) < (unsigned)nz) p[i - 1] = S::enc(v[i], is);
-    }
+    for (int q = 0; q < (NR - 1) / 4; ++q)
+        st4<S>(p + 4 * q, is, v[4 * q + 1], v[4 * q + 2], v[4 * q + 3], v[4 * q + 4]);
 }
 
 // Bulk tensor copy of one box of a 4D map (TMA: x, y, z, array) starting at
@@ -313,25 +329,49 @@ __device__ bool wait_cluster_bar(const SysLaunch &P, unsigned long long *bar, un
     }
 }
 
-// Bounded wait for phase `parity` of the staging barrier.  Returns false if
-// the wait ran past the launch's timeout (the error word is then set).
-__device__ bool wait_stage(const SysLaunch &P, unsigned long long *bar, unsigned parity, int ticket)
+// True once the wait that began at t0 (set on the first call) is past `ns`.
+__device__ __forceinline__ bool past(unsigned long long &t0, unsigned long long ns)
+{
+    const unsigned long long now = globaltimer();
+    if (t0 == 0) t0 = now;
+    return now - t0 > ns;
+}
+
+__device__ __noinline__ void timed_out(int *ctrl, int ticket, int what)
+{
+    if (atomicCAS(ctrl + 1, DEV_OK, DEV_ERR_TIMEOUT) == DEV_OK) {
+        ctrl[2] = ticket;
+        ctrl[3] = what;
+    }
+}
+
+// Release / acquire at CTA scope on a shared word: how the compute warps and
+// the bookkeeping warp tell each other where they are.
+__device__ __forceinline__ void st_rel_cta(unsigned *p, unsigned v)
+{
+    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned ld_acq_cta(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+
+// Bounded wait for phase `parity` of a staging barrier; gives up at once when
+// the bookkeeping warp has (*quit).  False: the error word is set.
+__device__ bool wait_stage(const SysLaunch &P, unsigned long long *bar, unsigned parity, const unsigned *quit, int ticket)
 {
     unsigned long long t0 = 0;
-    for (int it = 0;; ++it) {
+    for (;;) {
         unsigned done;
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;"
                      " selp.u32 %0, 1, 0, p; }"
                      : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
         if (done) return true;
-        const unsigned long long now = globaltimer();
-        if (it == 0) {
-            t0 = now;
-        } else if (now - t0 > (unsigned long long)P.timeout_ns) {
-            if (atomicCAS(P.ctrl + 1, DEV_OK, DEV_ERR_TIMEOUT) == DEV_OK) {
-                P.ctrl[2] = ticket;
-                P.ctrl[3] = -1;
-            }
+        if (quit && ld_acq_cta(quit)) return false;
+        if (past(t0, 2 * (unsigned long long)P.timeout_ns)) {
+            timed_out(P.ctrl, ticket, -1);
             return false;
         }
     }
@@ -346,13 +386,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     constexpr int SW = R::SW, XA = R::XA, SWC = R::SWC;
     extern __shared__ __align__(1024) float4 smem4[];
     // staging buffers first (the dynamic shared memory base is 1024-byte
-    // aligned), each: the lower z, y and x shells of the 6 fields, then those
-    // of dt/eps (and ca); the pointers below are buffer 0's, buffer b is
-    // R::STG_B bytes further
+    // aligned): the lower z, y and x shells of the 6 fields, twice, then those
+    // of dt/eps (and ca)
     char *const stg0 = reinterpret_cast<char *>(smem4);
     // y exchange (layout: RegTile::VX): E^t (level t-1) rows i = 0..NZ-1, and
     // the new H rows r = 1..NZ at row r-1
-    float *const XEx = reinterpret_cast<float *>(stg0 + R::NBUF * R::STG_B);
+    char *const cof0 = stg0 + 2 * R::STG_B;
+    float *const XEx = reinterpret_cast<float *>(cof0 + R::NCBUF * R::COF_B);
     float *const XEz = XEx + R::XE_F;
     float *const XHx = XEz + R::XE_F;
     float *const XHz = XHx + R::XE_F;
@@ -370,12 +410,14 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     // x pairs: a slot of the receive ring is full (the upwind CTA arrives
     // once its x lanes have written it) / free again (the downwind CTA arrives)
     __shared__ alignas(8) unsigned long long s_rxf[R::NSLOT], s_rxe[R::NSLOT];
-    __shared__ alignas(8) unsigned long long s_bar[2];  // staging barriers, one per buffer: one phase per fill
-    // state of the next step's shells, decided during this one: 0 = the
-    // upwind tiles have not published them yet, 1 = published and fetched
-    // into the other buffer, 2 = published, not yet fetched (one buffer)
-    __shared__ int s_pref;
-    __shared__ unsigned s_niss[2];                      // fills issued into each buffer
+    __shared__ alignas(8) unsigned long long s_bar[3];  // staging barriers, one per buffer (lossy: and the
+                                                        // coefficients'): one phase per fill
+    // the bookkeeping warp's view of the compute warps: B1 barriers passed over
+    // the CTA's life, and the current tile's last finished level (its progress
+    // value less the epoch); s_quit: it has given up waiting
+    __shared__ unsigned s_steps, s_level, s_quit;
+    __shared__ unsigned s_steps2;  // B2 barriers passed (lossy)
+    __shared__ int s_pfail;  // ... before the tile's first step
     __shared__ unsigned s_seen[3];
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -414,18 +456,19 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     T *const XF = reinterpret_cast<T *>(P.xf);
     T *const YF = reinterpret_cast<T *>(P.yf);
     constexpr int BZ = R::BZ;
-#define FACE_STORE(dst, fs, z0)                                                             \
-    do {                                                                                    \
-        st_rows<S>((dst), IS(0), ex, (z0), P.nz); st_rows<S>((dst) + (fs), IS(1), ey, (z0), P.nz);         \
-        st_rows<S>((dst) + 2 * (fs), IS(2), ez, (z0), P.nz); st_rows<S>((dst) + 3 * (fs), IS(3), hx, (z0), P.nz); \
-        st_rows<S>((dst) + 4 * (fs), IS(4), hy, (z0), P.nz); st_rows<S>((dst) + 5 * (fs), IS(5), hz, (z0), P.nz); \
+#define FACE_STORE(dst, fs)                                                              \
+    do {                                                                                \
+        st_rows<S>((dst), IS(0), ex); st_rows<S>((dst) + (fs), IS(1), ey);               \
+        st_rows<S>((dst) + 2 * (fs), IS(2), ez); st_rows<S>((dst) + 3 * (fs), IS(3), hx); \
+        st_rows<S>((dst) + 4 * (fs), IS(4), hy); st_rows<S>((dst) + 5 * (fs), IS(5), hz); \
     } while (0)
 
     constexpr int CR = R::CR;
     if (tid == 0) {
-        s_niss[0] = s_niss[1] = 0u;
+        s_steps = s_steps2 = s_quit = 0u;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[0])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[1])) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[2])) : "memory");
         if constexpr (R::CL == 2) {
 #pragma unroll
             for (int k = 0; k < R::NSLOT; ++k) {
@@ -444,6 +487,15 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     const unsigned rx_remote = R::CL == 2 ? mapa(smem_u32(RX), 1u) : 0u;        // rank 0 -> rank 1's ring
     const unsigned rxf_remote = R::CL == 2 ? mapa(smem_u32(&s_rxf[0]), 1u) : 0u;
     const unsigned rxe_remote = R::CL == 2 ? mapa(smem_u32(&s_rxe[0]), 0u) : 0u;  // rank 1 -> rank 0
+    // the tile of a ticket (x pairs: this CTA's half of it, I may be past the last)
+    auto tile_of = [&](int ticket, int &I, int &J, int &K) {
+        const int tl = P.tiles[ticket];
+        const int gxe = R::CL == 2 ? (P.gx + 1) / 2 : P.gx;
+        I = tl % gxe;
+        if (R::CL == 2) I = 2 * I + (int)rank;
+        J = (tl / gxe) % P.gy;
+        K = tl / (gxe * P.gy);
+    };
     // messages (x faces) sent / received over this CTA's life: message m
     // uses slot m % NSLOT, its (m / NSLOT)-th use of that slot
     int msg_base = 0;
@@ -451,30 +503,143 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     // rank 0, the slot its x lanes have just filled; rank 1, the slot its x
     // lane has just read
     int sig_slot = -1;
+    if (w >= R::RY) {
+        // ------------------------------------------------ bookkeeping warp
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R::BREG));
+        if (w > R::RY) {
+            // (x pairs: cluster barriers count every thread that has not left)
+            return;
+        }
+        // Polls the upwind tiles' progress and fetches a step's lower shells
+        // (six bulk tensor copies; x start rounded down to 16 bytes, zero fill
+        // off the domain) as soon as their staging buffer is free, and publishes
+        // the tile's own levels: the release of a flag waits for the CTA's stores
+        // to land (1000 to 1900 cycles), a poll and the copies take as long
+        // again, and none of it holds up a compute warp here.
+        unsigned steps0 = 0, n0 = 0, n1 = 0, n2 = 0;  // s_steps at the tile's start; fills of each buffer
+        auto fetch_coefs = [&](int t, int Ax, int Ay, int Az, char *sb, unsigned long long *bar) {
+            const int bx = Ax - t, by = Ay - t, bz = Az - t, x0c = (bx - 1) & ~(R::XAC - 1);
+            tma_box(sb, &P.tm[0][1], x0c, by - 1, bz - 1, bar);
+            tma_box(sb + R::OFF_YC, &P.tm[1][1], x0c, by - 1, bz - 1, bar);
+            tma_box(sb + R::OFF_XC, &P.tm[2][1], x0c, by, bz - 1, bar);
+        };
+        for (;;) {
+            if constexpr (R::CL == 2) cluster_sync_all(); else bar_tile();
+            if constexpr (R::CL == 2) cluster_sync_all(); else bar_tile();
+            const int ticket = s_ticket;
+            if (s_abort || ticket >= P.ntiles) break;
+            int I, J, K;
+            tile_of(ticket, I, J, K);
+            if (R::CL == 2 && I >= P.gx) continue;
+            const int tile = I + P.gx * (J + P.gy * K);
+            const int Ax = I * TX, Ay = J * TY, Az = K * TZ, kb = K % P.nzblk;
+            const Interval iv = tile_interval<TX, TY, TZ>(P, I, J, K);
+            Upwind U;
+            upwind_of<TX, TY, TZ>(P, I, J, K, U);
+            if (lane < 3) s_seen[lane] = 0u;
+            __syncwarp();
+            bool ok = iv.s == 0 || wait_level(P, U, s_seen, iv.s - 1, ticket);
+            if (lane == 0) s_pfail = !ok;
+            bar_tile();
+            if (!ok) continue;
+            // a tile that starts late (or, start > end, enters the domain only
+            // after this launch) carries its upwind tiles' guarantee on
+            if (iv.s > 0 && lane == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.s);
+            if (iv.s > iv.e) continue;
+            int t = iv.s, tc = iv.s;                 // the next step to fetch (tc: lossy, its coefficients)
+            unsigned pub = 0;                        // the last level published
+            unsigned long long t_up = 0, t_own = 0;  // waiting for the upwind tiles, for the compute warps
+            while (ok && (t <= iv.e || (R::LOSSY && tc <= iv.e) || pub != (unsigned)iv.e + 1u)) {
+                bool idle = true;
+                if (R::LOSSY && tc <= iv.e) {  // the coefficients' buffer: free once B2 of step tc - 1 has been passed
+                    const unsigned passed2 = __shfl_sync(0xffffffffu, ld_acq_cta(&s_steps2), 0);
+                    if (tc == iv.s || (int)(passed2 - (steps0 + (unsigned)(tc - iv.s))) >= 0) {
+                        idle = false;
+                        if (lane == 0) {
+                            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&s_bar[2])),
+                                         "r"(R::COEF_BYTES) : "memory");
+                            fetch_coefs(tc, Ax, Ay, Az, cof0, &s_bar[2]);
+                        }
+                        ++tc;
+                        ++n2;
+                    }
+                }
+                // step t's buffer: free at the tile's start, else once B1 of step
+                // t - 1 has been passed
+                const unsigned passed = __shfl_sync(0xffffffffu, ld_acq_cta(&s_steps), 0);
+                if (t <= iv.e && (t < iv.s + 2 || (int)(passed - (steps0 + (unsigned)(t - iv.s))) >= 0)) {
+                    idle = false;
+                    if (level_ready(P, U, s_seen, t)) {
+                        __syncwarp();  // orders lanes 1, 2's acquires before lane 0's copies
+                        if (lane == 0) {
+                            const int bx = Ax - t, by = Ay - t, bz = Az - t, b = t & 1;
+                            const int x0 = (bx - 1) & ~(XA - 1);
+                            char *const sb = stg0 + (size_t)b * R::STG_B;
+                            unsigned long long *const bar = &s_bar[b];
+                            // order this thread's view of the upwind tiles' global stores
+                            // (generic proxy, acquired through their progress flags)
+                            // before the bulk copies that read them
+                            asm volatile("fence.proxy.async.global;" ::: "memory");
+                            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                                         "r"(R::FIELD_BYTES + (R::LOSSY ? 0u : R::COEF_BYTES)) : "memory");
+                            tma_box(sb, &P.tm[0][0], x0, by - 1, bz - 1, bar);                 // z shell: field arrays
+                            tma_box5(sb + R::OFF_Y, &P.tm[1][0], 0, bx, by - 1, kb, bar);      // y shell: y-face buffer
+                            tma_box5(sb + R::OFF_X, &P.tm[2][0], 0, by - 1, bx - 1, kb, bar);  // x shell: x-face buffer
+                            if (!R::LOSSY) fetch_coefs(t, Ax, Ay, Az, cof0 + (size_t)b * R::COF_B, bar);
+                        }
+                        if (t & 1) ++n1;
+                        else ++n0;
+                        ++t;
+                        t_up = 0;
+                    } else {
+                        bool late = lane == 0 && past(t_up, (unsigned long long)P.timeout_ns);
+                        if (late) timed_out(P.ctrl, ticket, (int)(P.epoch + (unsigned)t + 1u));
+                        late |= ld_volatile(P.ctrl + 1) != DEV_OK;
+                        ok = !__any_sync(0xffffffffu, late);
+                    }
+                }
+                const unsigned lv = __shfl_sync(0xffffffffu, ld_acq_cta(&s_level), 0);
+                if (lv != pub) {
+                    if (lane == 0) publish(P, tile, ticket, P.epoch + lv);
+                    pub = lv;
+                    t_own = 0;
+                    idle = false;
+                }
+                if (idle) {
+                    __nanosleep(32);
+                    bool late = lane == 0 && past(t_own, 8 * (unsigned long long)P.timeout_ns);
+                    if (late) timed_out(P.ctrl, ticket, -3);
+                    late |= *(volatile int *)&s_abort != 0;
+                    ok = !__any_sync(0xffffffffu, late);
+                }
+            }
+            if (!ok && lane == 0) st_rel_cta(&s_quit, 1u);
+            steps0 += (unsigned)(iv.e - iv.s + 1);
+        }
+        // no copy may still be writing when the CTA's shared memory goes (after an
+        // abort some were never waited for)
+        if (lane == 0) {
+            if (n0) wait_stage(P, &s_bar[0], (n0 - 1) & 1u, nullptr, -1);
+            if (n1) wait_stage(P, &s_bar[1], (n1 - 1) & 1u, nullptr, -1);
+            if (n2) wait_stage(P, &s_bar[2], (n2 - 1) & 1u, nullptr, -1);
+        }
+        __syncwarp();
+        if constexpr (R::CL == 2) cluster_sync_all();
+        return;
+    }
+
+    // ------------------------------------------------------- compute warps
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R::CREG));
     // fills waited for on each buffer (every thread waits on every fill, so
-    // every thread keeps the same counts)
-    unsigned n_wait0 = 0, n_wait1 = 0;
-    // lower shells of level t into buffer b: six bulk tensor copies issued by
-    // one thread (x start rounded down to 16 bytes; zero fill off the domain),
-    // counted in s_niss for the final drain
-    auto issue_shells = [&](int t, int b, int Ax, int Ay, int Az, int kb) {
-        const int bx = Ax - t, by = Ay - t, bz = Az - t;
-        const int x0 = (bx - 1) & ~(XA - 1), x0c = (bx - 1) & ~(R::XAC - 1);
-        char *sb = stg0 + (size_t)b * R::STG_B;
-        unsigned long long *bar = &s_bar[b];
-        // order this thread's view of the upwind tiles' global stores (generic
-        // proxy, acquired through their progress flags) before the bulk copies
-        // that read them
-        asm volatile("fence.proxy.async.global;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                     "r"(R::TMA_BYTES) : "memory");
-        tma_box(sb, &P.tm[0][0], x0, by - 1, bz - 1, bar);              // z shell: field arrays
-        tma_box5(sb + R::OFF_Y, &P.tm[1][0], 0, bx, by - 1, kb, bar);        // y shell: y-face buffer
-        tma_box5(sb + R::OFF_X, &P.tm[2][0], 0, by - 1, bx - 1, kb, bar);    // x shell: x-face buffer
-        tma_box(sb + R::OFF_ZC, &P.tm[0][1], x0c, by - 1, bz - 1, bar);
-        tma_box(sb + R::OFF_YC, &P.tm[1][1], x0c, by - 1, bz - 1, bar);
-        tma_box(sb + R::OFF_XC, &P.tm[2][1], x0c, by, bz - 1, bar);
-        ++s_niss[b];
+    // every thread keeps the same counts), B1 barriers passed
+    unsigned n_wait0 = 0, n_wait1 = 0, nsteps = 0;
+    unsigned n_wait2 = 0, nsteps2 = 0;  // (lossy)
+    // the coefficient ring's row of physical z = bz - 1 + i, with zr the row of
+    // bz - 1 (lossless: any number congruent to it)
+    auto ring = [](int zr, int i) {
+        if (!R::LOSSY) return (zr + i) & (R::CR - 1);
+        const int q = zr + i;
+        return q >= R::CR ? q - R::CR : q;
     };
     // the tile column of this thread: registers row i <-> r = i-1
     float ex[NR], ey[NR], ez[NR], hx[NR], hy[NR], hz[NR];
@@ -494,36 +659,30 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 st_remote_u32(mapa(smem_u32(&s_ticket), 1u), (unsigned)tk);
                 st_remote_u32(mapa(smem_u32(&s_abort), 1u), (unsigned)ab);
             }
-            if (tid == 0) s_pref = 0;
-            if (tid < 3) s_seen[tid] = 0u;
+            if (tid == 0) s_level = 0u;
             cluster_sync_all();
         } else {
+            bar_tile();
             if (tid == 0) {
                 s_ticket = atomicAdd(P.ctrl, 1);
                 s_abort = ld_volatile(P.ctrl + 1) != DEV_OK;
-                s_pref = 0;
+                s_level = 0u;
             }
-            if (tid < 3) s_seen[tid] = 0u;
-            __syncthreads();
+            bar_tile();
         }
         const int ticket = s_ticket;
-        const bool stop = s_abort || ticket >= P.ntiles;
-        __syncthreads();
-        if (stop) break;
+        if (s_abort || ticket >= P.ntiles) break;
         bool abort = false;
         int nmsg = 0;
         do {  // one tile (`break` leaves it early: an abort, or a pair member without a tile)
         int I, J, K;
         int m_lo = 1, m_hi = 0;  // x pairs: steps whose x face goes through the ring
+        tile_of(ticket, I, J, K);
         if constexpr (R::CL == 2) {
-            const int gxp = (P.gx + 1) / 2, pr = P.tiles[ticket];
-            const int pp = pr % gxp;
-            J = (pr / gxp) % P.gy;
-            K = pr / (gxp * P.gy);
-            I = 2 * pp + (int)rank;
-            if (2 * pp + 1 < P.gx) {
-                const Interval i0 = tile_interval<TX, TY, TZ>(P, 2 * pp, J, K);
-                const Interval i1 = tile_interval<TX, TY, TZ>(P, 2 * pp + 1, J, K);
+            const int I0 = I - (int)rank;
+            if (I0 + 1 < P.gx) {
+                const Interval i0 = tile_interval<TX, TY, TZ>(P, I0, J, K);
+                const Interval i1 = tile_interval<TX, TY, TZ>(P, I0 + 1, J, K);
                 if (i0.s <= i0.e && i1.s <= i1.e) {
                     m_lo = i1.s;
                     m_hi = min(i0.e, i1.e);
@@ -531,35 +690,19 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             }
             nmsg = max(0, m_hi - m_lo + 1);
             if (I >= P.gx) break;  // the last pair of an odd tile row has one tile
-        } else {
-            const int tl = P.tiles[ticket];
-            I = tl % P.gx;
-            J = (tl / P.gx) % P.gy;
-            K = tl / (P.gx * P.gy);
         }
-        const int tile = I + P.gx * (J + P.gy * K);
         const int Ax = I * TX, Ay = J * TY, Az = K * TZ;
         const int kb = K % P.nzblk;  // this tile's z-block in the face buffers
         T *const XFk = XF + (long long)kb * P.nx * P.ny * BZ;
         T *const YFk = YF + (long long)kb * P.nx * P.ny * BZ;
         const Interval iv = tile_interval<TX, TY, TZ>(P, I, J, K);
-        Upwind U;
-        upwind_of<TX, TY, TZ>(P, I, J, K, U);
+        bar_tile();  // the bookkeeping warp has waited for level start - 1
+        if (s_pfail) break;
+        if (iv.s > iv.e) continue;  // enters the domain only after this launch: nothing to do
 
-        if (iv.s > 0) {
-            if (w == 0) {
-                const bool ok = wait_level(P, U, s_seen, iv.s - 1, ticket);
-                if (tid == 0) s_abort = !ok;
-            }
-            __syncthreads();
-            if (s_abort) { abort = true; break; }
-        }
-        if (iv.s > iv.e) {  // enters the domain only after this launch: relay only
-            if (tid == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.s);
-            __syncthreads();
-            continue;
-        }
-
+        // ring row of physical z = bz - 1 at the first step
+        int zl = R::LOSSY ? (((Az - iv.s - 1) % CR) + CR) % CR : 0;
+        const int zr0 = R::LOSSY ? zl : Az - iv.s - 1;
         // initial load: level start-1, rows sigma_z = Az + r at physical Az + r - start + 1
         {
             const int bx = Ax - iv.s, by = Ay - iv.s;
@@ -597,11 +740,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 } else {
                     ex[i] = ey[i] = ez[i] = hx[i] = hy[i] = hz[i] = 0.f;
                 }
-                CEs[(w * CR + (pz & (CR - 1))) * 32 + lane] = c;
-                if (R::LOSSY) CAs[(w * CR + (pz & (CR - 1))) * 32 + lane] = a;
+                CEs[(w * CR + ring(zr0, i == NR - 1 && R::LOSSY ? 0 : i + 1)) * 32 + lane] = c;
+                if (R::LOSSY) CAs[(w * CR + ring(zr0, i == NR - 1 ? 0 : i + 1)) * 32 + lane] = a;
             }
         }
-        if (iv.s > 0 && tid == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.s);
 
         // may a point source lie in the box during this tile's steps?  (per
         // axis, the box holds coordinate c at steps A - c .. A - c + n - 1)
@@ -612,16 +754,19 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const int hi = min(min(iv.e, Ax - s.i + TX - 1), min(Ay - s.j + TY - 1, Az - s.k + TZ - 1));
             tile_src |= lo <= hi;
         }
-        for (int t = iv.s; t <= iv.e; ++t) {
+        for (int t = iv.s;; ++t, zl = R::LOSSY ? (zl == 0 ? CR - 1 : zl - 1) : 0) {
+            // (one pass more than steps: the last step's top y face)
             const int bx = Ax - t, by = Ay - t, bz = Az - t;  // box low corner at step t
-            const int cur = R::NBUF == 2 ? (t & 1) : 0;
-            char *const sb = stg0 + (size_t)cur * R::STG_B;
+            const int zr = R::LOSSY ? zl : bz - 1;
+            const int cur = t & 1;
+            const char *const sb = stg0 + (size_t)cur * R::STG_B;
+            const char *const cb = cof0 + (R::LOSSY ? 0 : (size_t)cur * R::COF_B);
             const T *const ZST = reinterpret_cast<const T *>(sb);
             const T *const YST = reinterpret_cast<const T *>(sb + R::OFF_Y);
             const T *const XST = reinterpret_cast<const T *>(sb + R::OFF_X);
-            const float *const ZSC = reinterpret_cast<const float *>(sb + R::OFF_ZC), *const ZSA = ZSC + R::ZBC;
-            const float *const YSC = reinterpret_cast<const float *>(sb + R::OFF_YC), *const YSA = YSC + R::YBC;
-            const float *const XSC = reinterpret_cast<const float *>(sb + R::OFF_XC), *const XSA = XSC + R::XBC;
+            const float *const ZSC = reinterpret_cast<const float *>(cb), *const ZSA = ZSC + R::ZBC;
+            const float *const YSC = reinterpret_cast<const float *>(cb + R::OFF_YC), *const YSA = YSC + R::YBC;
+            const float *const XSC = reinterpret_cast<const float *>(cb + R::OFF_XC), *const XSA = XSC + R::XBC;
             const int dx = (lane - bx) & 31, dy = (w - by) & (R::RY - 1);
             const int px = bx + dx, py = by + dy;
             const bool xbox = dx < TX, ybox = dy < TY;
@@ -629,18 +774,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const int ey_w = (by - 1) & (R::RY - 1);  // warp holding the y shell this step
             const int yf_w = (by + TY) & (R::RY - 1);  // warp holding the top y row of step t-1
             const long long col = px + (long long)P.pitch * py;
-            // rows i with physical z = bz + i - 1 inside the domain
-            const int i_lo = max(1, 1 - bz), i_hi = min(NR, P.nz - bz + 1);
-            // the box is clear of the low walls: every box cell is updated
-            // with no mask.  (The x-shell lane and the y-shell warp compute
-            // values that their refills overwrite.)  Cells beyond the high
-            // walls need none either: their dt/eps (and c_a) is 0 (the
-            // coefficient shells are zero-filled off the domain), so their E
-            // stays 0, and their H, whose curl reads only such E, stays 0 too.
-            const bool inner = bx >= 1 && by >= 1 && bz >= 1;
-            // every row of the box's z range lies in the domain (rows refilled
-            // from the face buffers need no clearing)
-            const bool zin = bz >= 0 && bz + TZ <= P.nz;
+            // the box touches a low wall, whose tangential E is left alone.  (No
+            // other masks: cells outside the domain have dt/eps (and c_a) 0, as the
+            // coefficient shells are zero-filled there, so their E stays 0; their H
+            // is only read by such cells and by that tangential E; and the x-shell
+            // lane and the y-shell warp compute values that their refills
+            // overwrite.)
+            const bool walls = bx < 1 || by < 1 || bz < 1;
             // physical x of this lane's column after the refills (the x-shell
             // lane moves to bx - 1)
             const int xw = (bx - 1) + ((lane - bx + 1) & 31);
@@ -660,8 +800,8 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     XEz[xe_at(w, i, lane)] = ez[i];
                 }
             }
-            __syncthreads();  // B1
-            if (s_abort) { abort = true; break; }
+            bar_compute();  // B1
+            if (tid == 0 && t <= iv.e) st_rel_cta(&s_steps, ++nsteps);
             // x pairs: this step's x face travels through ring slot `slot`
             const bool msg = R::CL == 2 && t >= m_lo && t <= m_hi;
             const bool rx_msg = msg && rank == 1, tx_msg = msg && rank == 0;
@@ -678,30 +818,17 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     sig_slot = -1;
                 }
             }
-            // unless the previous step found this step's shells published,
-            // wait here for the upwind tiles' level t; fetch the shells now
-            // unless they were fetched during the previous step
-            const int pst = s_pref;
-            if (pst == 0) {
-                if (w == 0) {
-                    const bool ok = wait_level(P, U, s_seen, t, ticket);
-                    if (tid == 0) s_abort = !ok;
-                }
-                __syncthreads();
-                if (s_abort) { abort = true; break; }
-            }
-            if (pst != 1 && tid == 0) issue_shells(t, cur, Ax, Ay, Az, kb);
-
             // B. the warp whose y slot leaves the tile this step is idle during
             //    the H half-step: it stores last step's top y face, which its
             //    registers still hold, into the y-face buffer
             if (w == yf_w && t > iv.s) {
-                const int pbx = bx + 1, pby = by + 1, pbz = bz + 1;  // box corner of step t-1
+                const int pbx = bx + 1, pby = by + 1;  // box corner of step t-1
                 const int pdx = (lane - pbx) & 31;
                 const int qx = pbx + pdx, qy = pby + TY - 1;
                 if (pdx < TX && (unsigned)qx < (unsigned)P.nx && (unsigned)qy < (unsigned)P.ny)
-                    FACE_STORE(YFk + ((long long)qy * P.nx + qx) * BZ, P.fys, pbz);
+                    FACE_STORE(YFk + ((long long)qy * P.nx + qx) * BZ, P.fys);
             }
+            if (t > iv.e) break;
             // x start of the staged z shell (rounded down to 16 bytes)
             const int x0 = (bx - 1) & ~(XA - 1), x0c = (bx - 1) & ~(R::XAC - 1);
 
@@ -713,7 +840,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 // before either is written, so 16-bit storage rounds two new
                 // values with one packed conversion
                 const float *const qx = XEx + xe_at(wn, 0, lane), *const qz = XEz + xe_at(wn, 0, lane);
-                auto h_pass = [&](auto masked) {
+                {
                     float4 gx, gz;  // VX: the y+1 neighbour's E rows 4q .. 4q+3
 #pragma unroll
                     for (int i = NR - 1; i >= 2; i -= 2) {
@@ -739,42 +866,27 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                         RND2(nh[0][0], nh[1][0], 3);
                         RND2(nh[0][1], nh[1][1], 4);
                         RND2(nh[0][2], nh[1][2], 5);
-                        const bool u0 = !decltype(masked)::value || (colin && i >= i_lo && i < i_hi);
-                        const bool u1 = !decltype(masked)::value || (colin && i - 1 >= i_lo && i - 1 < i_hi);
-                        const float a0 = u0 ? nh[0][0] : hx[i - 1], b0 = u0 ? nh[0][1] : hy[i - 1],
-                                    c0 = u0 ? nh[0][2] : hz[i - 1];
-                        const float a1 = u1 ? nh[1][0] : hx[i - 2], b1 = u1 ? nh[1][1] : hy[i - 2],
-                                    c1 = u1 ? nh[1][2] : hz[i - 2];
-                        hx[i] = a0; hy[i] = b0; hz[i] = c0;
-                        hx[i - 1] = a1; hy[i - 1] = b1; hz[i - 1] = c1;
+                        hx[i] = nh[0][0]; hy[i] = nh[0][1]; hz[i] = nh[0][2];
+                        hx[i - 1] = nh[1][0]; hy[i - 1] = nh[1][1]; hz[i - 1] = nh[1][2];
                     }
-                };
-                if (inner)
-                    h_pass(std::false_type());
-                else
-                    h_pass(std::true_type());
+                }
             }
             // every thread waits on the staging barrier itself: its completion
             // makes the copied shells visible to that thread, so no block
             // barrier is needed here (a timeout is noticed after B2)
             {
                 unsigned &nw = cur ? n_wait1 : n_wait0;
-                if (!wait_stage(P, &s_bar[cur], nw & 1u, ticket)) s_abort = 1;
+                if (!wait_stage(P, &s_bar[cur], nw & 1u, &s_quit, ticket)) s_abort = 1;
                 ++nw;
+                if (R::LOSSY) {
+                    if (!wait_stage(P, &s_bar[2], n_wait2 & 1u, &s_quit, ticket)) s_abort = 1;
+                    ++n_wait2;
+                }
             }
 
             // D. refills from the staged shells, then publish new H rows for the
             //    warp above's E half-step
             const int xec = (bx - 1) - x0c;  // x offset of the coefficient shell column in its chunk
-            // rows of a refilled column whose physical z lies outside the
-            // domain: the face buffers hold other cells' values there
-#define CLEAR_OUT_ROWS(a, b, c)                                                          \
-    do {                                                                                 \
-        if (!zin) {                                                                      \
-            _Pragma("unroll") for (int i_ = 1; i_ < NR; ++i_) if (i_ < i_lo || i_ >= i_hi) \
-                a[i_] = b[i_] = c[i_] = 0.f;                                               \
-        }                                                                                \
-    } while (0)
             if (w == ey_w) {  // the y shell warp takes its whole column set (level t)
                 // row 0 from the lower z shell (its row y = by - 1); rows
                 // 1..NZ from the y-face shell (x = bx .. bx+30) or, in the
@@ -795,12 +907,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 ld_rows<S>(src + 3 * fst, SC(3), hx);
                 ld_rows<S>(src + 4 * fst, SC(4), hy);
                 ld_rows<S>(src + 5 * fst, SC(5), hz);
-                CLEAR_OUT_ROWS(ex, ey, ez);
-                CLEAR_OUT_ROWS(hx, hy, hz);
 #pragma unroll
                 for (int i = 0; i < NR; ++i) {
-                    CEs[(w * CR + ((bz - 1 + i) & (CR - 1))) * 32 + lane] = YSC[i * SWC + xlc];
-                    if (R::LOSSY) CAs[(w * CR + ((bz - 1 + i) & (CR - 1))) * 32 + lane] = YSA[i * SWC + xlc];
+                    CEs[(w * CR + ring(zr, i)) * 32 + lane] = YSC[i * SWC + xlc];
+                    if (R::LOSSY) CAs[(w * CR + ring(zr, i)) * 32 + lane] = YSA[i * SWC + xlc];
                 }
             } else if (!ybox) {  // the previous top y row (two outside slots): kept
             } else {  // every lane's row -1 takes the lower z shell's H and coefficient
@@ -808,8 +918,8 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 hx[0] = S::dec(ZST[3 * R::ZB + o], SC(3));
                 hy[0] = S::dec(ZST[4 * R::ZB + o], SC(4));
                 hz[0] = S::dec(ZST[5 * R::ZB + o], SC(5));
-                CEs[(w * CR + ((bz - 1) & (CR - 1))) * 32 + lane] = ZSC[oc];
-                if (R::LOSSY) CAs[(w * CR + ((bz - 1) & (CR - 1))) * 32 + lane] = ZSA[oc];
+                CEs[(w * CR + ring(zr, 0)) * 32 + lane] = ZSC[oc];
+                if (R::LOSSY) CAs[(w * CR + ring(zr, 0)) * 32 + lane] = ZSA[oc];
                 if (!xbox) {  // the lane leaving the tile in x: rows 1..NZ of H from the x-face shell
                     // (x pairs: from the ring, once the upwind CTA's lanes have arrived)
                     const T *xs = XST + (dy + 1) * BZ;
@@ -822,13 +932,12 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     ld_rows<S>(xs + 3 * xst, SC(3), hx);
                     ld_rows<S>(xs + 4 * xst, SC(4), hy);
                     ld_rows<S>(xs + 5 * xst, SC(5), hz);
-                    CLEAR_OUT_ROWS(hx, hy, hz);
                     const float *xsc = XSC + dy * R::XAC + xec;
                     const float *xsa = XSA + dy * R::XAC + xec;
 #pragma unroll
                     for (int i = 1; i < NR; ++i) {
-                        CEs[(w * CR + ((bz - 1 + i) & (CR - 1))) * 32 + lane] = xsc[i * 16 * R::XAC];
-                        if (R::LOSSY) CAs[(w * CR + ((bz - 1 + i) & (CR - 1))) * 32 + lane] = xsa[i * 16 * R::XAC];
+                        CEs[(w * CR + ring(zr, i)) * 32 + lane] = xsc[i * 16 * R::XAC];
+                        if (R::LOSSY) CAs[(w * CR + ring(zr, i)) * 32 + lane] = xsa[i * 16 * R::XAC];
                     }
                 }
             }
@@ -846,23 +955,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     XHz[xe_at(w, i - 1, lane)] = hz[i];
                 }
             }
-            __syncthreads();  // B2
+            bar_compute();  // B2
             if (s_abort) { abort = true; break; }
-            // the warps outside the box in y sit out the E half-step: the one
-            // holding the previous top y row (the y shell's when the box leaves
-            // one y slot) publishes level t-1; the y shell's then checks (one
-            // poll) whether the upwind tiles have published level t+1 and
-            // fetches those shells into the other buffer if so (two buffers).
-            // (The release first: the poll after it is cheaper than before it.)
-            if (w == yf_w && lane == 0 && t > iv.s) publish(P, tile, ticket, P.epoch + (unsigned)t);  // level t-1 done
-            if (w == ey_w) {
-                const bool nxt = t + 1 <= iv.e && level_ready(P, U, s_seen, t + 1);
-                __syncwarp();  // orders lanes 1, 2's acquires before lane 0's copies
-                if (lane == 0) {
-                    if (R::NBUF == 2 && nxt) issue_shells(t + 1, cur ^ 1, Ax, Ay, Az, kb);
-                    s_pref = nxt ? (R::NBUF == 2 ? 1 : 2) : 0;
-                }
-            }
+            if (tid == 0 && t > iv.s) st_rel_cta(&s_level, (unsigned)t);  // level t-1 is stored
+            if (R::LOSSY && tid == 0) st_rel_cta(&s_steps2, ++nsteps2);
 
             // does this thread own a point source this step?  (16-bit storage:
             // its E rows are rounded after the source is added, not before)
@@ -874,6 +970,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     srcthr |= step < s.n_amp && s.i >= bx && s.i < bx + TX && s.j >= by && s.j < by + TY &&
                               s.k >= bz && s.k < bz + TZ && lane == (s.i & 31) && w == (s.j & (R::RY - 1));
                 }
+                srcthr = __any_sync(0xffffffffu, srcthr);  // its whole warp rounds late (shuffles in the E half-step)
             }
 
             if (ybox) {
@@ -901,8 +998,8 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                                                 : m == 0 ? gx.x : m == 1 ? gx.y : m == 2 ? gx.z : gx.w;
                             const float hz_ym = !R::VX ? qz[(r - 1) * 32]
                                                 : m == 0 ? gz.x : m == 1 ? gz.y : m == 2 ? gz.z : gz.w;
-                            const float c = CEs[(w * CR + ((bz + r - 1) & (CR - 1))) * 32 + lane];
-                            const float a = R::LOSSY ? CAs[(w * CR + ((bz + r - 1) & (CR - 1))) * 32 + lane] : 1.f;
+                            const float c = CEs[(w * CR + ring(zr, r)) * 32 + lane];
+                            const float a = R::LOSSY ? CAs[(w * CR + ring(zr, r)) * 32 + lane] : 1.f;
                             ne[k][0] = e_x(decay<R::LOSSY>(a, ex[r - 1]), hz[r], hz_ym, hy[r], hy[r - 1], c);
                             ne[k][1] = e_y(decay<R::LOSSY>(a, ey[r - 1]), hx[r], hx[r - 1], hz[r], hz_xm, c);
                             ne[k][2] = e_z(decay<R::LOSSY>(a, ez[r - 1]), hy[r], hy_xm, hx[r], hx_ym, c);
@@ -917,11 +1014,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                         for (int k = 0; k < 2; ++k) {
                             const int r = i - k;
                             if (decltype(masked)::value) {
-                                const bool in = colin && r >= i_lo && r < i_hi;
                                 const bool kz = bz + r - 1 > 0;
-                                o[k][0] = (in && ux && kz) ? ne[k][0] : ex[r - 1];
-                                o[k][1] = (in && uy && kz) ? ne[k][1] : ey[r - 1];
-                                o[k][2] = (in && uz) ? ne[k][2] : ez[r - 1];
+                                o[k][0] = (ux && kz) ? ne[k][0] : ex[r - 1];
+                                o[k][1] = (uy && kz) ? ne[k][1] : ey[r - 1];
+                                o[k][2] = uz ? ne[k][2] : ez[r - 1];
                             } else {
                                 o[k][0] = ne[k][0];
                                 o[k][1] = ne[k][1];
@@ -932,15 +1028,15 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                         ex[i - 1] = o[1][0]; ey[i - 1] = o[1][1]; ez[i - 1] = o[1][2];
                     }
                 };
-                // 16-bit storage rounds each new E value here, except in the
-                // (rare) thread that adds a point source this step: it rounds
-                // after the source, below (masked form)
+                // 16-bit storage rounds each new E value here, except in the (rare)
+                // warp that adds a point source this step: it rounds after the
+                // source, below
                 if (S::narrow && srcthr)
                     e_pass(std::false_type(), std::true_type());
-                else if (inner)
-                    e_pass(std::bool_constant<S::narrow>(), std::false_type());
-                else
+                else if (walls)
                     e_pass(std::bool_constant<S::narrow>(), std::true_type());
+                else
+                    e_pass(std::bool_constant<S::narrow>(), std::false_type());
                 {  // every lane's row -1 takes the lower z shell's E (level t)
                     const int o = (dy + 1) * SW + (xw - x0);
                     ex[0] = S::dec(ZST[0 * R::ZB + o], SC(0));
@@ -954,7 +1050,6 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     ld_rows<S>(xs, SC(0), ex);
                     ld_rows<S>(xs + xst, SC(1), ey);
                     ld_rows<S>(xs + 2 * xst, SC(2), ez);
-                    CLEAR_OUT_ROWS(ex, ey, ez);
                 }
             }
 
@@ -964,15 +1059,17 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 if (step < s.n_amp && s.i >= bx && s.i < bx + TX && s.j >= by && s.j < by + TY &&
                     s.k >= bz && s.k < bz + TZ && lane == (s.i & 31) && w == (s.j & (R::RY - 1))) {
                     const float a = S::src_amp(s.amp[step], P.sc.src);
+                    // added to the whole column, with -0 (which changes no value) in
+                    // the other rows: a select and an add a row is less code than
+                    // finding the row
                     const int ri = s.k - bz + 1;
+                    auto add = [&](float (&e)[NR]) {
 #pragma unroll
-                    for (int i = 1; i < NR; ++i) {
-                        if (i == ri) {
-                            if (s.comp == 0) ex[i] = add_source(ex[i], a);
-                            else if (s.comp == 1) ey[i] = add_source(ey[i], a);
-                            else ez[i] = add_source(ez[i], a);
-                        }
-                    }
+                        for (int i = 1; i < NR; ++i) e[i] = add_source(e[i], i == ri ? a : -0.f);
+                    };
+                    if (s.comp == 0) add(ex);
+                    else if (s.comp == 1) add(ey);
+                    else add(ez);
                 }
             }
             if (S::narrow && srcthr) {  // one rounding per value, as the naive schedule stores it
@@ -986,7 +1083,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 
             // the adjoint's recompute: this step's E of the cells of the
             // capture box (tiles that meet it only)
-            if (P.cap && colin && bx < P.cap_hi[0] && bx + TX > P.cap_lo[0] && by < P.cap_hi[1] &&
+            if (R::CAP && colin && bx < P.cap_hi[0] && bx + TX > P.cap_lo[0] && by < P.cap_hi[1] &&
                 by + TY > P.cap_lo[1] && bz < P.cap_hi[2] && bz + TZ > P.cap_lo[2] && px >= P.cap_lo[0] &&
                 px < P.cap_hi[0] && py >= P.cap_lo[1] && py < P.cap_hi[1]) {
                 float *cp = P.cap + 3 * P.cap_bc * (long long)t;
@@ -1003,23 +1100,11 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
                 }
             }
-            // G. stores: the whole box on the launch's last step, else the top faces
-            if (t == P.T - 1) {
-                if (colin) {
-#pragma unroll
-                    for (int i = 1; i < NR; ++i) {
-                        if (i >= i_lo && i < i_hi) {
-                            const long long g = col + sxy * (bz + i - 1);
-                            STORE6(g, i);
-                        }
-                    }
-                }
-            } else if (colin) {
-                // (the top y face is stored next step by the warp holding it)
-                if (NR - 1 >= i_lo && NR - 1 < i_hi) {  // top z face
-                    const long long g = col + sxy * (bz + NR - 2);
-                    STORE6(g, NR - 1);
-                }
+            // G. the top faces (the top y face is stored next step by the warp
+            // holding it; the launch's last step is stored whole, below)
+            if (colin && t < P.T - 1 && (unsigned)(bz + NR - 2) < (unsigned)P.nz) {  // top z face
+                const long long g = col + sxy * (bz + NR - 2);
+                STORE6(g, NR - 1);
             }
             // top x face (all rows of the lane leaving the box in x) into the
             // x-face buffer, where the downwind tile's x shell is fetched.
@@ -1044,37 +1129,31 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 }
                 if ((!(R::CL == 2 && tx_msg) || dy == TY - 1) && (unsigned)px < (unsigned)P.nx &&
                     (unsigned)py < (unsigned)P.ny)
-                    FACE_STORE(XFk + ((long long)px * P.ny + py) * BZ, P.fxs, bz);
+                    FACE_STORE(XFk + ((long long)px * P.ny + py) * BZ, P.fxs);
             }
             if (R::CL == 2 && msg) sig_slot = slot;
         }
         if (abort) break;
-        // the last step's top y face (the launch's last one included: the
-        // downwind tile reads it from the y-face buffer), then its progress
-        __syncthreads();
-        if (R::CL == 2 && sig_slot >= 0) {  // the tile's last message: filled / read
-            if (tid == 0) arrive_remote((rank == 0 ? rxf_remote : rxe_remote) + 8u * (unsigned)sig_slot);
-            sig_slot = -1;
+        if (iv.e == P.T - 1) {  // the launch's last step: the whole box
+            const int bx = Ax - iv.e, by = Ay - iv.e, bz = Az - iv.e;
+            const int dx = (lane - bx) & 31, dy = (w - by) & (R::RY - 1);
+            const int px = bx + dx, py = by + dy;
+            if (dx < TX && dy < TY && (unsigned)px < (unsigned)P.nx && (unsigned)py < (unsigned)P.ny) {
+                const long long col = px + (long long)P.pitch * py;
+#pragma unroll
+                for (int i = 1; i < NR; ++i)
+                    if ((unsigned)(bz + i - 1) < (unsigned)P.nz) {
+                        const long long g = col + sxy * (bz + i - 1);
+                        STORE6(g, i);
+                    }
+            }
         }
-        {
-            const int pbx = Ax - iv.e, pby = Ay - iv.e, pbz = Az - iv.e;
-            const int pdx = (lane - pbx) & 31, pdy = (w - pby) & (R::RY - 1);
-            const int qx = pbx + pdx, qy = pby + pdy;
-            if (pdy == TY - 1 && pdx < TX && (unsigned)qx < (unsigned)P.nx && (unsigned)qy < (unsigned)P.ny)
-                FACE_STORE(YFk + ((long long)qy * P.nx + qx) * BZ, P.fys, pbz);
-        }
-        __syncthreads();
-        if (tid == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.e + 1u);
+        bar_compute();
+        if (tid == 0) st_rel_cta(&s_level, (unsigned)iv.e + 1u);
         } while (false);
         msg_base += nmsg;
         sig_slot = -1;
-        if (R::CL == 1 && abort) break;  // a pair leaves together, at the next ticket
-    }
-    // after an abort, bulk copies may still be writing into the staging
-    // buffers: wait for them (bounded) before the CTA's shared memory goes
-    if (tid == 0) {
-        while (n_wait0 < s_niss[0] && wait_stage(P, &s_bar[0], n_wait0 & 1u, -1)) ++n_wait0;
-        while (n_wait1 < s_niss[1] && wait_stage(P, &s_bar[1], n_wait1 & 1u, -1)) ++n_wait1;
+        // (after an abort the CTA, or a pair together, leaves at the next ticket)
     }
     // x pairs: neither CTA leaves while its partner may still write into its
     // shared memory
@@ -1095,7 +1174,6 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 #undef RND2
 #undef STORE6
 #undef FACE_STORE
-#undef CLEAR_OUT_ROWS
 
 // 31 x 15 x 12 and 31 x 15 x 8 tiles, each for every kernel format; the
 // lossy (absorber) form for the 31 x 15 x 12 tile
@@ -1115,6 +1193,10 @@ struct RegShape {
         if (cl == 2) {
             if constexpr (HAS_PAIRS) DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, false, REG_TY, 2>>());
             return cudaErrorInvalidValue;
+        }
+        if (fmt == FDTD_STORAGE_F32) {  // and its capturing form, for the adjoint
+            const cudaError_t e = set<RegTile<NZ, StoreF32, false, REG_TY, 1, true>>();
+            if (e != cudaSuccess) return e;
         }
         DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, false, REG_TY>>());
     }
@@ -1140,6 +1222,10 @@ struct RegShape {
         if (cl == 2) {
             if constexpr (HAS_PAIRS) DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, false, REG_TY, 2>>(p, grid, st));
             return cudaErrorInvalidValue;
+        }
+        if (p.cap) {
+            if (fmt != FDTD_STORAGE_F32) return cudaErrorInvalidValue;
+            return go<RegTile<NZ, StoreF32, false, REG_TY, 1, true>>(p, grid, st);
         }
         DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, false, REG_TY>>(p, grid, st));
     }
