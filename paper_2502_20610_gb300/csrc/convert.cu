@@ -1,71 +1,119 @@
-// FP32 <-> storage-format conversion of one field component, used by
-// fdtd_write_fields / fdtd_read_fields when fields are stored as FP16 or
-// BF16: q = fl_S(v / s) on the way in (round to nearest even), v = s * q on
-// the way out (exact).  Dense arrays hold nx*ny*nz values; the device arrays
-// have rows of `pitch` elements.
+// Fields between the caller's dense FP32 arrays (nx*ny*nz values a component)
+// and the simulation's arrays (rows of `pitch` elements in the storage format;
+// 16-bit: q = fl_S(v / s), to nearest even, on the way in, v = s * q, exact, on
+// the way out), used by fdtd_write_fields / fdtd_read_fields.
+//
+// All components in one launch.  Bounded by memory on large grids (one read
+// and one write of each value), by the launch on small ones, where a copy per
+// component cost 2.5 us of host time each.  A block's x threads run along a
+// row, four values each where rows and pointers allow, its y threads take
+// rows: no division per value (an element-wise kernel with a 64-bit division
+// and a launch per component took 142 us to write and read 128^3 FP16, this 31).
 #include "internal.h"
 #include "storage.cuh"
 
 namespace {
 
+// enc or dec of four values at once: 16-byte FP32, 8-byte 16-bit accesses
 template <class S>
-__global__ void to_storage_kernel(typename S::T *__restrict__ dst, const float *__restrict__ src, int nx,
-                                  long long rows, int pitch, float inv_s)
+__device__ __forceinline__ void put4(typename S::T *p, const float4 v, float is)
 {
-    const long long n = (long long)nx * rows;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long r = q / nx, x = q - r * nx;
-        dst[x + r * pitch] = S::enc(src[q], inv_s);
+    if constexpr (sizeof(typename S::T) == 4) {
+        *reinterpret_cast<float4 *>(p) = v;
+    } else {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(S::enc2(v.x, v.y, is), S::enc2(v.z, v.w, is));
+    }
+}
+template <class S>
+__device__ __forceinline__ float4 get4(const typename S::T *p, float s)
+{
+    using T = typename S::T;
+    if constexpr (sizeof(T) == 4) {
+        return *reinterpret_cast<const float4 *>(p);
+    } else {
+        const uint2 u = *reinterpret_cast<const uint2 *>(p);
+        return make_float4(S::dec((T)(u.x & 0xffffu), s), S::dec((T)(u.x >> 16), s), S::dec((T)(u.y & 0xffffu), s),
+                           S::dec((T)(u.y >> 16), s));
     }
 }
 
-template <class S>
-__global__ void from_storage_kernel(float *__restrict__ dst, const typename S::T *__restrict__ src, int nx,
-                                    long long rows, int pitch, float s)
+// comps: the component of each z block, 4 bits each.  IN: dense -> arrays
+// (and the nzero words at `zero` cleared); else arrays -> dense, nothing if
+// *err is set.
+template <class S, bool IN, bool VEC>
+__global__ void __launch_bounds__(256)
+fields_kernel(typename S::T *arrays, long long fs, float *dense, long long n, int nx, long long rows, int pitch,
+              unsigned comps, const Scales sc, int *zero, int nzero, const int *err)
 {
-    const long long n = (long long)nx * rows;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long r = q / nx, x = q - r * nx;
-        dst[q] = S::dec(src[x + r * pitch], s);
+    if (!IN && *err != DEV_OK) return;
+    if (IN && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.y == 0)
+        for (int q = threadIdx.x; q < nzero; q += blockDim.x) zero[q] = 0;
+    const int c = (comps >> (4 * blockIdx.z)) & 15;
+    typename S::T *const f = arrays + c * fs;
+    float *const d = dense + blockIdx.z * n;
+    for (long long r = blockIdx.x * (long long)blockDim.y + threadIdx.y; r < rows; r += (long long)gridDim.x * blockDim.y) {
+        typename S::T *const fr = f + r * pitch;
+        float *const dr = d + r * nx;
+        if (VEC) {
+            for (int x = 4 * threadIdx.x; x < nx; x += 4 * blockDim.x) {
+                if (IN) put4<S>(fr + x, *reinterpret_cast<const float4 *>(dr + x), sc.is[c]);
+                else *reinterpret_cast<float4 *>(dr + x) = get4<S>(fr + x, sc.s[c]);
+            }
+        } else {
+            for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+                if (IN) fr[x] = S::enc(dr[x], sc.is[c]);
+                else dr[x] = S::dec(fr[x], sc.s[c]);
+            }
+        }
     }
 }
 
-int blocks_for(long long n) { return (int)std::min<long long>((n + 255) / 256, 152 * 16); }
+template <class S, bool IN>
+cudaError_t go(void *arrays, long long fs, float *dense, int nx, int ny, int nz, int pitch, unsigned comps, int ncomp,
+               const Scales &sc, int *zero, int nzero, const int *err, cudaStream_t st)
+{
+    const long long rows = (long long)ny * nz;
+    // four values a thread: rows of both sides start on 16 (8) bytes
+    const bool vec = nx % 4 == 0 && (uintptr_t)dense % 16 == 0;
+    const int per_row = vec ? nx / 4 : nx;
+    int bx = 8;
+    while (bx < 256 && bx < per_row) bx *= 2;
+    const dim3 block((unsigned)bx, 256u / bx);
+    const dim3 grid((unsigned)std::min<long long>((rows + block.y - 1) / block.y, 152 * 8), 1, (unsigned)ncomp);
+    if (vec)
+        fields_kernel<S, IN, true><<<grid, block, 0, st>>>((typename S::T *)arrays, fs, dense, (long long)nx * rows, nx, rows,
+                                                           pitch, comps, sc, zero, nzero, err);
+    else
+        fields_kernel<S, IN, false><<<grid, block, 0, st>>>((typename S::T *)arrays, fs, dense, (long long)nx * rows, nx, rows,
+                                                            pitch, comps, sc, zero, nzero, err);
+    return cudaGetLastError();
+}
+
+template <bool IN>
+cudaError_t dispatch(int storage, void *arrays, long long fs, float *dense, int nx, int ny, int nz, int pitch,
+                     unsigned comps, int ncomp, const Scales &sc, int *zero, int nzero, const int *err, cudaStream_t st)
+{
+    // the host converts with s at the boundary in the uniform formats too
+    if (storage == FDTD_STORAGE_F16)
+        return go<StoreF16, IN>(arrays, fs, dense, nx, ny, nz, pitch, comps, ncomp, sc, zero, nzero, err, st);
+    if (storage == FDTD_STORAGE_BF16)
+        return go<StoreBF16, IN>(arrays, fs, dense, nx, ny, nz, pitch, comps, ncomp, sc, zero, nzero, err, st);
+    return go<StoreF32, IN>(arrays, fs, dense, nx, ny, nz, pitch, comps, ncomp, sc, zero, nzero, err, st);
+}
 
 } // namespace
 
-cudaError_t launch_to_storage(void *pitched, const float *dense, int storage, int nx, int ny, int nz, int pitch,
-                              float inv_scale, cudaStream_t st)
+cudaError_t launch_write_fields(void *arrays, long long fs, const float *dense, int storage, int nx, int ny, int nz,
+                                int pitch, unsigned comps, int ncomp, const Scales &sc, int *zero, int nzero,
+                                cudaStream_t st)
 {
-    const long long rows = (long long)ny * nz, n = (long long)nx * rows;
-    if (n == 0) return cudaSuccess;
-    if (storage == FDTD_STORAGE_F16)
-        to_storage_kernel<StoreF16><<<blocks_for(n), 256, 0, st>>>((unsigned short *)pitched, dense, nx, rows, pitch,
-                                                                    inv_scale);
-    else if (storage == FDTD_STORAGE_BF16)
-        to_storage_kernel<StoreBF16><<<blocks_for(n), 256, 0, st>>>((unsigned short *)pitched, dense, nx, rows,
-                                                                     pitch, inv_scale);
-    else
-        to_storage_kernel<StoreF32><<<blocks_for(n), 256, 0, st>>>((float *)pitched, dense, nx, rows, pitch,
-                                                                    inv_scale);
-    return cudaGetLastError();
+    return dispatch<true>(storage, arrays, fs, const_cast<float *>(dense), nx, ny, nz, pitch, comps, ncomp, sc, zero, nzero,
+                          nullptr, st);
 }
 
-cudaError_t launch_from_storage(float *dense, const void *pitched, int storage, int nx, int ny, int nz,
-                                int pitch, float scale, cudaStream_t st)
+cudaError_t launch_read_fields(float *dense, const void *arrays, long long fs, int storage, int nx, int ny, int nz,
+                               int pitch, unsigned comps, int ncomp, const Scales &sc, const int *err, cudaStream_t st)
 {
-    const long long rows = (long long)ny * nz, n = (long long)nx * rows;
-    if (n == 0) return cudaSuccess;
-    if (storage == FDTD_STORAGE_F16)
-        from_storage_kernel<StoreF16><<<blocks_for(n), 256, 0, st>>>(dense, (const unsigned short *)pitched, nx,
-                                                                      rows, pitch, scale);
-    else if (storage == FDTD_STORAGE_BF16)
-        from_storage_kernel<StoreBF16><<<blocks_for(n), 256, 0, st>>>(dense, (const unsigned short *)pitched, nx,
-                                                                       rows, pitch, scale);
-    else
-        from_storage_kernel<StoreF32><<<blocks_for(n), 256, 0, st>>>(dense, (const float *)pitched, nx, rows,
-                                                                      pitch, scale);
-    return cudaGetLastError();
+    return dispatch<false>(storage, const_cast<void *>(arrays), fs, dense, nx, ny, nz, pitch, comps, ncomp, sc, nullptr, 0,
+                           err, st);
 }

@@ -475,7 +475,7 @@ struct fdtd_sim {
     int cap_lo[3] = {0, 0, 0}, cap_hi[3] = {0, 0, 0};
     long long cap_bc = 0, cap_s0 = 0;
     long long launches;
-    int sms;       // of the handle's device
+    int dev, sms;  // the handle's device and its SMs
     int max_ctas;
     std::vector<long long> count_le;  // tiles with start <= s
     int dbg_kind;
@@ -506,15 +506,16 @@ cudaError_t copy_rows(float *dst, size_t dpitch, const float *src, size_t spitch
                              cudaMemcpyDefault, st);
 }
 
-// True if `p` is device (or managed) memory the kernels can read and write.
-bool is_device_pointer(const void *p)
+// True if `p` is memory that kernels on device `dev` can read and write: its
+// own, or managed.
+bool is_local_pointer(const void *p, int dev)
 {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();  // pageable host memory on older runtimes
         return false;
     }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+    return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
 }
 
 #define CK(x)                                                                  \
@@ -729,6 +730,7 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(cuda_status(e));
+    h->dev = dev;
     h->sms = sms;
     if (coeffs->scheme == FDTD_SCHEME_SYSTOLIC) {
         e = systolic_configure(L.variant, h->fmt, h->ca != nullptr, L.cl);
@@ -794,24 +796,27 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src)
 {
     if (!h || !src) return FDTD_ERR_INVALID_ARG;
     const size_t n = (size_t)h->g.nx * h->g.ny * h->g.nz;
-    if (h->c.storage == FDTD_STORAGE_F32) {
-        for (int k = 0; k < 6; ++k)
-            CK(copy_rows((float *)h->f[k], h->L.pitch, src + (size_t)k * n, h->g.nx, h->g, h->stream));
+    const long long fs = (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb;
+    // cleared too: the error word and its details, and the grid barrier (a
+    // launch that timed out may have left arrivals in it)
+    int *const zero = h->ctrl + 1;
+    const int nzero = CTRL_BARRIER + 8 - 1;
+    if (is_local_pointer(src, h->dev)) {
+        CK(launch_write_fields(h->f[0], fs, src, h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, 0x543210u, 6, h->sc,
+                               zero, nzero, h->stream));
     } else {
-        const bool dev = is_device_pointer(src);
         for (int k = 0; k < 6; ++k) {
             const float *from = src + (size_t)k * n;
-            if (!dev) {  // through the dense FP32 stage
+            if (h->c.storage == FDTD_STORAGE_F32) {
+                CK(copy_rows((float *)h->f[k], h->L.pitch, from, h->g.nx, h->g, h->stream));
+            } else {  // through the dense FP32 stage
                 CK(cudaMemcpyAsync(h->stage, from, sizeof(float) * n, cudaMemcpyDefault, h->stream));
-                from = h->stage;
+                CK(launch_write_fields(h->f[0], fs, h->stage, h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch,
+                                       (unsigned)k, 1, h->sc, zero, 0, h->stream));
             }
-            CK(launch_to_storage(h->f[k], from, h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->sc.is[k],
-                                 h->stream));
         }
+        CK(cudaMemsetAsync(zero, 0, nzero * sizeof(int), h->stream));
     }
-    // the error word and its details, and the grid barrier (a launch that
-    // timed out may have left arrivals in it)
-    CK(cudaMemsetAsync(h->ctrl + 1, 0, (CTRL_BARRIER + 8 - 1) * sizeof(int), h->stream));
     // S^{n-1} := 0 (both band snapshots: which is "previous" alternates)
     if (h->prev) CK(cudaMemsetAsync(h->ws + h->L.prev, 0, h->L.layer - h->L.prev, h->stream));
     h->failed = false;
@@ -958,22 +963,30 @@ fdtd_status fdtd_sync(fdtd_handle h)
 fdtd_status fdtd_read_fields(fdtd_handle h, uint32_t component_mask, float *dst)
 {
     if (!h || (!dst && component_mask) || component_mask > 63u) return FDTD_ERR_INVALID_ARG;
+    const size_t n = (size_t)h->g.nx * h->g.ny * h->g.nz;
+    const long long fs = (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb;
+    unsigned comps = 0;
+    int ncomp = 0;
+    for (unsigned k = 0; k < 6; ++k)
+        if (component_mask & (1u << k)) comps |= k << (4 * ncomp++);
+    if (ncomp > 0 && is_local_pointer(dst, h->dev)) {
+        // the copy looks at the error word itself, so one synchronisation serves both
+        CK(launch_read_fields(dst, h->f[0], fs, h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, comps, ncomp, h->sc,
+                              h->ctrl + 1, h->stream));
+        return fdtd_sync(h);
+    }
     fdtd_status s = fdtd_sync(h);
     if (s != FDTD_OK) return s;
-    const size_t n = (size_t)h->g.nx * h->g.ny * h->g.nz;
-    const bool dev = h->c.storage == FDTD_STORAGE_F32 || is_device_pointer(dst);
-    size_t q = 0;
-    for (int k = 0; k < 6; ++k) {
-        if (!(component_mask & (1u << k))) continue;
+    for (int q = 0; q < ncomp; ++q) {
+        const unsigned k = (comps >> (4 * q)) & 15u;
+        float *const to = dst + (size_t)q * n;
         if (h->c.storage == FDTD_STORAGE_F32) {
-            CK(copy_rows(dst + q * n, h->g.nx, (const float *)h->f[k], h->L.pitch, h->g, h->stream));
+            CK(copy_rows(to, h->g.nx, (const float *)h->f[k], h->L.pitch, h->g, h->stream));
         } else {
-            float *to = dev ? dst + q * n : h->stage;
-            CK(launch_from_storage(to, h->f[k], h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->sc.s[k],
-                                   h->stream));
-            if (!dev) CK(cudaMemcpyAsync(dst + q * n, h->stage, sizeof(float) * n, cudaMemcpyDefault, h->stream));
+            CK(launch_read_fields(h->stage, h->f[0], fs, h->c.storage, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, k, 1, h->sc,
+                                  h->ctrl + 1, h->stream));
+            CK(cudaMemcpyAsync(to, h->stage, sizeof(float) * n, cudaMemcpyDefault, h->stream));
         }
-        ++q;
     }
     CK(cudaStreamSynchronize(h->stream));
     return FDTD_OK;

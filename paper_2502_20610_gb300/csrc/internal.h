@@ -57,12 +57,16 @@ cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, c
                               int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc,
                               int *bar, int *err, long long timeout_ns, int sms, cudaStream_t st);
 
-// FP32 <-> storage conversion of one component (convert.cu): `dense` holds
-// nx*ny*nz values, `pitched` rows of `pitch` elements.
-cudaError_t launch_to_storage(void *pitched, const float *dense, int storage, int nx, int ny, int nz, int pitch,
-                              float inv_scale, cudaStream_t st);
-cudaError_t launch_from_storage(float *dense, const void *pitched, int storage, int nx, int ny, int nz,
-                                int pitch, float scale, cudaStream_t st);
+// Fields between dense FP32 components (nx*ny*nz values each, packed in the
+// order of `comps`, 4 bits each) and the arrays in storage format (component
+// c at arrays + c*fs, rows of `pitch` elements), one launch (convert.cu);
+// device memory only.  Writing clears the nzero words at `zero` too, reading
+// does nothing when *err is set.
+cudaError_t launch_write_fields(void *arrays, long long fs, const float *dense, int storage, int nx, int ny, int nz,
+                                int pitch, unsigned comps, int ncomp, const Scales &sc, int *zero, int nzero,
+                                cudaStream_t st);
+cudaError_t launch_read_fields(float *dense, const void *arrays, long long fs, int storage, int nx, int ny, int nz,
+                               int pitch, unsigned comps, int ncomp, const Scales &sc, const int *err, cudaStream_t st);
 
 // Systolic scheme: the subdomain ("tile") geometry is a compile-time ring of
 // 32 x RY x RZ shared-memory slots per CTA of which 31 x (RY-1) x (RZ-1)

@@ -104,9 +104,10 @@ naive_e_kernel(typename S::T *__restrict__ ex_, typename S::T *__restrict__ ey_,
 // Small domains (at most NAIVE_BLOCK_CELLS cells, the largest thread block):
 // one CTA, one thread per cell, runs all the steps of a call with block
 // barriers between the half-steps instead of kernel boundaries, the regime
-// of Fig. 1 in which the update needs no global synchronisation.  The data
-// change inside the launch, so loads are plain (coherent) loads; the block
-// barrier orders each half-step's stores before the next one's loads.
+// of Fig. 1 in which the update needs no global synchronisation.  A thread's
+// own six values stay in registers for the whole call, neighbours go through
+// shared memory, so a half-step is a shared-memory round trip and a barrier:
+// 8^3, 100 steps 40.0 -> 25.9 us (fields in global memory before).
 template <class S, bool LOSSY>
 __global__ void __launch_bounds__(NAIVE_BLOCK_CELLS)
 naive_block_kernel(typename S::T *__restrict__ ex_, typename S::T *__restrict__ ey_, typename S::T *__restrict__ ez_,
@@ -114,52 +115,60 @@ naive_block_kernel(typename S::T *__restrict__ ex_, typename S::T *__restrict__ 
                    const float *__restrict__ ce_, const float *__restrict__ ca_, int nx, int ny, int nz, int pitch, float ndt, long long step0,
                    int nsteps, const SrcSet src, const Scales sc)
 {
-    const int q = threadIdx.x;
+    __shared__ float sex[NAIVE_BLOCK_CELLS], sey[NAIVE_BLOCK_CELLS], sez[NAIVE_BLOCK_CELLS];
+    __shared__ float shx[NAIVE_BLOCK_CELLS], shy[NAIVE_BLOCK_CELLS], shz[NAIVE_BLOCK_CELLS];
+    const int q = threadIdx.x, qy = nx, qz = nx * ny;
     const bool own = q < nx * ny * nz;
-    const int i = own ? q % nx : 0, j = own ? (q / nx) % ny : 0, k = own ? q / (nx * ny) : 0;
-    const long long sxy = (long long)pitch * ny;
+    const int i = own ? q % nx : 0, j = own ? (q / nx) % ny : 0, k = own ? q / qz : 0;
     const long long p = i + (long long)pitch * (j + (long long)ny * k);
-    const bool ip = i + 1 < nx, jp = j + 1 < ny, kp = k + 1 < nz;
+    const bool ip = own && i + 1 < nx, jp = own && j + 1 < ny, kp = own && k + 1 < nz;
     const float ce = own ? ce_[p] : 0.f;
     const float ca = LOSSY && own ? ca_[p] : 1.f;
+    float ex = 0.f, ey = 0.f, ez = 0.f, hx = 0.f, hy = 0.f, hz = 0.f;
+    if (own) {
+        ex = S::dec(ex_[p], sc.s[0]); ey = S::dec(ey_[p], sc.s[1]); ez = S::dec(ez_[p], sc.s[2]);
+        hx = S::dec(hx_[p], sc.s[3]); hy = S::dec(hy_[p], sc.s[4]); hz = S::dec(hz_[p], sc.s[5]);
+    }
+    unsigned mine = 0;  // the sources on this cell
+    for (int qq = 0; qq < src.n; ++qq)
+        if (own && src.s[qq].idx == p) mine |= 1u << qq;
+    sex[q] = ex; sey[q] = ey; sez[q] = ez;
+    __syncthreads();
     for (int s = 0; s < nsteps; ++s) {
         if (own) {
-            const float exc = S::dec(ex_[p], sc.s[0]), eyc = S::dec(ey_[p], sc.s[1]), ezc = S::dec(ez_[p], sc.s[2]);
-            const float exn = kp ? S::dec(ex_[p + sxy], sc.s[0]) : 0.f;
-            const float eyn = kp ? S::dec(ey_[p + sxy], sc.s[1]) : 0.f;
-            const float ez_ip = ip ? S::dec(ez_[p + 1], sc.s[2]) : 0.f;
-            const float ey_ip = ip ? S::dec(ey_[p + 1], sc.s[1]) : 0.f;
-            const float ez_jp = jp ? S::dec(ez_[p + pitch], sc.s[2]) : 0.f;
-            const float ex_jp = jp ? S::dec(ex_[p + pitch], sc.s[0]) : 0.f;
-            hx_[p] = S::enc(h_x(S::dec(hx_[p], sc.s[3]), ez_jp, ezc, eyn, eyc, ndt), sc.is[3]);
-            hy_[p] = S::enc(h_y(S::dec(hy_[p], sc.s[4]), exn, exc, ez_ip, ezc, ndt), sc.is[4]);
-            hz_[p] = S::enc(h_z(S::dec(hz_[p], sc.s[5]), ey_ip, eyc, ex_jp, exc, ndt), sc.is[5]);
+            const float ez_jp = jp ? sez[q + qy] : 0.f, ey_kp = kp ? sey[q + qz] : 0.f;
+            const float ex_kp = kp ? sex[q + qz] : 0.f, ez_ip = ip ? sez[q + 1] : 0.f;
+            const float ey_ip = ip ? sey[q + 1] : 0.f, ex_jp = jp ? sex[q + qy] : 0.f;
+            hx = S::rnd(h_x(hx, ez_jp, ez, ey_kp, ey, ndt), sc.s[3], sc.is[3]);
+            hy = S::rnd(h_y(hy, ex_kp, ex, ez_ip, ez, ndt), sc.s[4], sc.is[4]);
+            hz = S::rnd(h_z(hz, ey_ip, ey, ex_jp, ex, ndt), sc.s[5], sc.is[5]);
+            shx[q] = hx; shy[q] = hy; shz[q] = hz;
         }
         __syncthreads();
         if (own) {
-            const float hx = S::dec(hx_[p], sc.s[3]), hy = S::dec(hy_[p], sc.s[4]), hz = S::dec(hz_[p], sc.s[5]);
-            float ex = S::dec(ex_[p], sc.s[0]), ey = S::dec(ey_[p], sc.s[1]), ez = S::dec(ez_[p], sc.s[2]);
-            if (j > 0 && k > 0)
-                ex = e_x(decay<LOSSY>(ca, ex), hz, S::dec(hz_[p - pitch], sc.s[5]), hy, S::dec(hy_[p - sxy], sc.s[4]), ce);
-            if (i > 0 && k > 0)
-                ey = e_y(decay<LOSSY>(ca, ey), hx, S::dec(hx_[p - sxy], sc.s[3]), hz, S::dec(hz_[p - 1], sc.s[5]), ce);
-            if (i > 0 && j > 0)
-                ez = e_z(decay<LOSSY>(ca, ez), hy, S::dec(hy_[p - 1], sc.s[4]), hx, S::dec(hx_[p - pitch], sc.s[3]), ce);
+            if (j > 0 && k > 0) ex = e_x(decay<LOSSY>(ca, ex), hz, shz[q - qy], hy, shy[q - qz], ce);
+            if (i > 0 && k > 0) ey = e_y(decay<LOSSY>(ca, ey), hx, shx[q - qz], hz, shz[q - 1], ce);
+            if (i > 0 && j > 0) ez = e_z(decay<LOSSY>(ca, ez), hy, shy[q - 1], hx, shx[q - qy], ce);
             const long long step = step0 + s;
-            for (int qq = 0; qq < src.n; ++qq) {
-                const SrcDesc &d = src.s[qq];
-                if (d.idx == p && step < d.n_amp) {
+            for (unsigned m = mine; m; m &= m - 1) {
+                const SrcDesc &d = src.s[__ffs((int)m) - 1];
+                if (step < d.n_amp) {
                     const float a = S::src_amp(d.amp[step], sc.src);
                     if (d.comp == 0) ex = add_source(ex, a);
                     else if (d.comp == 1) ey = add_source(ey, a);
                     else ez = add_source(ez, a);
                 }
             }
-            ex_[p] = S::enc(ex, sc.is[0]);
-            ey_[p] = S::enc(ey, sc.is[1]);
-            ez_[p] = S::enc(ez, sc.is[2]);
+            ex = S::rnd(ex, sc.s[0], sc.is[0]);
+            ey = S::rnd(ey, sc.s[1], sc.is[1]);
+            ez = S::rnd(ez, sc.s[2], sc.is[2]);
+            sex[q] = ex; sey[q] = ey; sez[q] = ez;
         }
         __syncthreads();
+    }
+    if (own) {
+        ex_[p] = S::enc(ex, sc.is[0]); ey_[p] = S::enc(ey, sc.is[1]); ez_[p] = S::enc(ez, sc.is[2]);
+        hx_[p] = S::enc(hx, sc.is[3]); hy_[p] = S::enc(hy, sc.is[4]); hz_[p] = S::enc(hz, sc.is[5]);
     }
 }
 
