@@ -117,7 +117,7 @@ typedef struct {
  *     high face.  A zero network leaves the graded layer on PEC walls.
  *     Naive scheme and FP32 storage only (the update needs the whole previous
  *     level every step, which the systolic tiles do not keep).  Per step the
- *     band of the state is snapshotted, the network runs on the handle's
+ *     state's faces are snapshotted, the network runs on the handle's
  *     internal stream while the Yee step runs on the handle's stream, and
  *     the corrections are added once both are done. */
 typedef struct {

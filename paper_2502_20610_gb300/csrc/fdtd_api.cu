@@ -31,10 +31,9 @@ struct Layout {
     size_t xface, yface;  // register kernel's x- and y-face buffers (6 components each)
     long long fxs, fys;   // their elements per component
     int nzb, nzblk;       // their z extent: nzblk z-blocks of nzb / nzblk elements
-    // learned boundary: network, previous and current band snapshots, layer
-    // and band cell lists, layer predictions
-    size_t params, prev, snap, layer, band, pred;
-    long long nlayer, nband;
+    // learned boundary: network, its weights in the layer kernel's order, the
+    // previous and current snapshots of the faces, the corrections
+    size_t params, image, prev, snap, pred;
     int eb;     // bytes per stored field value (4 FP32, 2 FP16/BF16)
     int pitch;  // elements per x row in device memory (nx rounded up to 16 bytes)
     int variant, tx, ty, tz;  // systolic tile shape
@@ -51,31 +50,6 @@ int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 bool conducts(const fdtd_boundary &b)
 {
     return b.kind == FDTD_BOUNDARY_GRADED_ABSORBER || (b.kind == FDTD_BOUNDARY_LEARNED && b.sigma_max > 0.0);
-}
-
-// Cells within distance t of a wall (min over axes of the distance to the
-// nearest face < t): the total minus the inner box.
-long long cells_within(const fdtd_grid &g, int t)
-{
-    const long long ix = std::max(0, g.nx - 2 * t), iy = std::max(0, g.ny - 2 * t), iz = std::max(0, g.nz - 2 * t);
-    return (long long)g.nx * g.ny * g.nz - ix * iy * iz;
-}
-
-// (x, y, z) of those cells, x fastest.
-void list_cells_within(const fdtd_grid &g, int t, std::vector<int> &out)
-{
-    out.clear();
-    for (int k = 0; k < g.nz; ++k)
-        for (int j = 0; j < g.ny; ++j)
-            for (int i = 0; i < g.nx; ++i) {
-                const int d = std::min(std::min(std::min(i, g.nx - 1 - i), std::min(j, g.ny - 1 - j)),
-                                       std::min(k, g.nz - 1 - k));
-                if (d < t) {
-                    out.push_back(i);
-                    out.push_back(j);
-                    out.push_back(k);
-                }
-            }
 }
 
 constexpr int DEFAULT_VARIANT = 2;  // register-resident 31 x 15 x 12 with TMA shells: fastest measured
@@ -112,24 +86,20 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     off = align_up(off + sizeof(float) * (size_t)n);
     L.ca = off;  // E decay of conducting cells (absorber, or the learned layer's base)
     if (conducts(b)) off = align_up(off + sizeof(float) * (size_t)n);
-    L.nlayer = L.nband = 0;
-    L.params = L.prev = L.snap = L.layer = L.band = L.pred = off;
+    L.params = L.image = L.prev = L.snap = L.pred = off;
     if (b.kind == FDTD_BOUNDARY_LEARNED) {
-        L.nlayer = cells_within(g, 1);  // the faces carry the network's corrections
-        L.nband = cells_within(g, 2);   // their stencils reach one cell further
+        const LearnedGeo geo = learned_geometry(g.nx, g.ny, g.nz);
         L.params = off;
         off = align_up(off + sizeof(float) * (size_t)mlpnet::NPARAM);
-        // two band snapshots (S^{n-1}, S^n), each six components and its x slab
+        L.image = off;
+        off = align_up(off + learned_image_bytes());
+        // two snapshots (S^{n-1}, S^n)
         L.prev = off;
-        off = align_up(off + 6 * align_up(sizeof(float) * (size_t)n) + learned_xslab_bytes(g.ny, g.nz));
+        off = align_up(off + sizeof(float) * (size_t)geo.snap_floats);
         L.snap = off;
-        off = align_up(off + 6 * align_up(sizeof(float) * (size_t)n) + learned_xslab_bytes(g.ny, g.nz));
-        L.layer = off;
-        off = align_up(off + 3 * sizeof(int) * (size_t)L.nlayer);
-        L.band = off;
-        off = align_up(off + 3 * sizeof(int) * (size_t)L.nband);
+        off = align_up(off + sizeof(float) * (size_t)geo.snap_floats);
         L.pred = off;
-        off = align_up(off + 6 * sizeof(float) * (size_t)L.nlayer);
+        off = align_up(off + 6 * sizeof(float) * (size_t)geo.cells);
     }
     L.stage = off;
     if (c.storage != FDTD_STORAGE_F32) off = align_up(off + sizeof(float) * (size_t)g.nx * g.ny * g.nz);
@@ -449,10 +419,11 @@ struct fdtd_sim {
     float *ce;
     float *ca;     // E decay per cell (absorber), else null
     float *params, *prev, *pred;  // learned boundary (else null)
-    float *snap;                  // the band of the current state, read by the network
+    float *snap;                  // the faces of the current state, read by the network
+    void *image;
+    LearnedGeo geo;
     cudaStream_t aux;             // learned boundary: the network runs here, beside the Yee step
     cudaEvent_t ev_fork, ev_join;
-    int *layer, *band;
     int layer_grid;
     float *stage;  // dense FP32 component (16-bit storage), else null
     Scales sc;
@@ -632,8 +603,8 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     h->snap = learned ? (float *)(h->ws + L.snap) : nullptr;
     h->aux = nullptr;
     h->ev_fork = h->ev_join = nullptr;
-    h->layer = learned ? (int *)(h->ws + L.layer) : nullptr;
-    h->band = learned ? (int *)(h->ws + L.band) : nullptr;
+    h->image = learned ? h->ws + L.image : nullptr;
+    if (learned) h->geo = learned_geometry(grid->nx, grid->ny, grid->nz);
     h->layer_grid = 0;
     h->stage = coeffs->storage != FDTD_STORAGE_F32 ? (float *)(h->ws + L.stage) : nullptr;
     for (int k = 0; k < 6; ++k) {
@@ -698,17 +669,10 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     for (int k = 0; k < 6 && e == cudaSuccess; ++k)  // all-zero bits are +0 in every format
         e = cudaMemsetAsync(h->f[k], 0, (size_t)L.eb * padded, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ctrl, 0, 64 * sizeof(int), h->stream);
-    std::vector<int> lcells, bcells;
     if (e == cudaSuccess && learned) {
-        list_cells_within(*grid, 1, lcells);
-        list_cells_within(*grid, 2, bcells);
         e = cudaMemcpyAsync(h->params, boundary->model, sizeof(float) * mlpnet::NPARAM, cudaMemcpyDefault, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.prev, 0, L.layer - L.prev, h->stream);  // both snapshots
-        if (e == cudaSuccess && !lcells.empty())
-            e = cudaMemcpyAsync(h->layer, lcells.data(), sizeof(int) * lcells.size(), cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess && !bcells.empty())
-            e = cudaMemcpyAsync(h->band, bcells.data(), sizeof(int) * bcells.size(), cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess) e = learned_layer_configure();
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.prev, 0, L.pred - L.prev, h->stream);  // both snapshots
+        if (e == cudaSuccess) e = learned_layer_configure(h->params, h->image, h->stream);
         // the network's stream: highest priority, so its CTAs are placed first
         // and the Yee kernels fill the rest of each SM
         int lo = 0, hi = 0;
@@ -817,8 +781,8 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src)
         }
         CK(cudaMemsetAsync(zero, 0, nzero * sizeof(int), h->stream));
     }
-    // S^{n-1} := 0 (both band snapshots: which is "previous" alternates)
-    if (h->prev) CK(cudaMemsetAsync(h->ws + h->L.prev, 0, h->L.layer - h->L.prev, h->stream));
+    // S^{n-1} := 0 (both snapshots: which is "previous" alternates)
+    if (h->prev) CK(cudaMemsetAsync(h->ws + h->L.prev, 0, h->L.pred - h->L.prev, h->stream));
     h->failed = false;
     return FDTD_OK;
 }
@@ -833,27 +797,23 @@ fdtd_status fdtd_step(fdtd_handle h, int64_t n)
         if (h->params) {  // learned boundary: Yee everywhere, then the network's correction on the wall layer
             float *f0 = (float *)h->f[0];
             const long long fs = (long long)(h->L.fields[1] - h->L.fields[0]) / 4;
-            const long long ps = (long long)align_up(sizeof(float) * (size_t)h->L.pitch * h->g.ny * h->g.nz) / 4;
-            if (fs != ps) return FDTD_ERR_STATE;  // previous-state arrays mirror the field layout
-            // per step: snapshot the band of S^n (and its x slab); the network (S^n and S^{n-1}
-            // bands -> corrections) on the internal stream, the Yee step on the
+            // per step: snapshot the faces of S^n; the network (faces of S^n and
+            // S^{n-1} -> corrections) on the internal stream, the Yee step on the
             // caller's, both at once; then the corrections are added and the
             // snapshot becomes the next step's previous state
             for (int64_t s = 0; s < n; ++s) {
-                CK(learned_copy_cells(h->snap, f0, fs, h->L.pitch, h->g.ny, h->band, (int)h->L.nband, h->stream));
-                CK(learned_fill_xslab(h->snap, f0, fs, h->L.pitch, h->g.nx, h->g.ny, h->g.nz, h->stream));
+                CK(learned_snapshot(h->geo, f0, fs, h->L.pitch, h->snap, h->stream));
                 CK(cudaEventRecord(h->ev_fork, h->stream));
                 CK(cudaStreamWaitEvent(h->aux, h->ev_fork, 0));
-                CK(learned_layer_predict(h->params, h->snap, h->prev, fs, h->L.pitch, h->g.nx, h->g.ny, h->g.nz,
-                                         h->layer, (int)h->L.nlayer, h->pred, h->layer_grid, h->aux));
+                CK(learned_layer_predict(h->geo, h->params, h->image, h->snap, h->prev, h->pred, h->layer_grid, h->aux));
                 CK(cudaEventRecord(h->ev_join, h->aux));
                 CK(launch_naive_h(h->f, h->fmt, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, ndt, h->sc, h->stream));
                 CK(launch_naive_e(h->f, h->fmt, h->ce, h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, h->step, h->src,
                                   h->sc, h->stream));
                 CK(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
-                CK(learned_layer_scatter(f0, fs, h->L.pitch, h->g.ny, h->layer, (int)h->L.nlayer, h->pred, h->stream));
+                CK(learned_layer_scatter(h->geo, f0, fs, h->L.pitch, h->pred, h->stream));
                 std::swap(h->prev, h->snap);
-                h->launches += 6;
+                h->launches += 5;
                 h->step += 1;
             }
             return FDTD_OK;

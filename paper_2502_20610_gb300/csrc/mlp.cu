@@ -21,10 +21,9 @@
 // a time through the whole forward and backward pass in shared memory and
 // registers, and one that sums its partial gradients and takes the Adam
 // step.  The layer update of
-// a simulation step is one fused persistent kernel: it gathers the stencils
-// of 64 layer cells into shared memory and runs the three layers on them
-// with the weights resident in shared memory, the two large contractions on
-// the tensor cores (mma.sync TF32, three-term split for FP32 accuracy).
+// a simulation step is one fused persistent kernel over patches of the
+// domain's faces, the two large contractions on the tensor cores (mma.sync
+// TF32, three-term split for FP32 accuracy).
 #include "internal.h"
 #include "mlp.h"
 #include "yee_cell.cuh"
@@ -579,289 +578,395 @@ __global__ void __launch_bounds__(32 * RW) record_kernel(const float *__restrict
 // lo*hi + hi*lo + hi*hi ("3xTF32"): ~22 significant bits per operand, the
 // dropped lo*lo term below FP32 rounding of the sum, so the layer keeps
 // FP32 accuracy.
+// x rounded to TF32 (13 bits fewer, to nearest, ties away) as two integer
+// operations: cvt.rna.tf32.f32 gives the same for finite values, as a longer
+// sequence on this part.  (A NaN may lose its mark in hi; lo = x - hi keeps it.)
 __device__ __forceinline__ unsigned tf32_rna(float x)
 {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
+    return (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
 }
 __device__ __forceinline__ void split_tf32(float x, unsigned &hi, unsigned &lo)
 {
     hi = tf32_rna(x);
     lo = tf32_rna(__fsub_rn(x, __uint_as_float(hi)));
 }
-__device__ __forceinline__ void mma_tf32(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
-                                         unsigned b1)
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1)
 {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9},"
                  " {%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Shared tiles [k][64] (k = input feature or unit, 64 = cells or units) are
-// stored with the column index XOR-swizzled by (k mod 4) * 8, so the
-// fragment loads of a warp (rows k .. k+3, eight consecutive columns each)
-// hit 32 different banks.
-__device__ __forceinline__ int swz(int k, int c) { return c ^ ((k & 3) << 3); }
-
-// D[64 x 64] of this CTA's eight warps (warp w: rows 16*(w%4).., columns
-// 32*(w/4).., four m16n8 tiles) = sum_k A[k][row] B[k][col] over K (a
-// multiple of 8; A, B swizzled [k][64] tiles in shared memory).
-template <int K>
-__device__ __forceinline__ void warp_gemm_3xtf32(const float *A, const float *B, float (&acc)[4][4])
+// acc[n] += A B over one step of k, for the eight unit tiles n: w points at
+// this lane's fragment of unit tile 0.  Each of the three products runs over
+// all tiles before the next, so an accumulator's next use is eight
+// instructions away.
+__device__ __forceinline__ void contract(float (&acc)[8][4], const unsigned (&ah)[4], const unsigned (&al)[4], const uint4 *w)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int g = lane >> 2, q = lane & 3;
-    const int m0 = 16 * (w & 3), n0 = 32 * (w >> 2);
+    uint4 b[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int n = 0; n < 8; ++n) b[n] = w[8 * n];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
-#pragma unroll 2
-    for (int k0 = 0; k0 < K; k0 += 8) {
-        const int ka = k0 + q, kb = k0 + q + 4;
-        unsigned ah[4], al[4];
-        split_tf32(A[ka * 64 + swz(ka, m0 + g)], ah[0], al[0]);
-        split_tf32(A[ka * 64 + swz(ka, m0 + g + 8)], ah[1], al[1]);
-        split_tf32(A[kb * 64 + swz(kb, m0 + g)], ah[2], al[2]);
-        split_tf32(A[kb * 64 + swz(kb, m0 + g + 8)], ah[3], al[3]);
+    for (int n = 0; n < 8; ++n) mma_tf32(acc[n], al, b[n].x, b[n].y);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + 8 * j + g;
-            unsigned bh0, bl0, bh1, bl1;
-            split_tf32(B[ka * 64 + swz(ka, n)], bh0, bl0);
-            split_tf32(B[kb * 64 + swz(kb, n)], bh1, bl1);
-            mma_tf32(acc[j], al[0], al[1], al[2], al[3], bh0, bh1);
-            mma_tf32(acc[j], ah[0], ah[1], ah[2], ah[3], bl0, bl1);
-            mma_tf32(acc[j], ah[0], ah[1], ah[2], ah[3], bh0, bh1);
-        }
-    }
+    for (int n = 0; n < 8; ++n) mma_tf32(acc[n], ah, b[n].z, b[n].w);
+#pragma unroll
+    for (int n = 0; n < 8; ++n) mma_tf32(acc[n], ah, b[n].x, b[n].y);
 }
 
-// Shared memory of the fused layer kernel, in floats; the float4-read arrays
-// come first, each a multiple of 64 floats, so they stay 16-byte aligned.
-constexpr int LC = 64;  // layer cells per tile
-constexpr int NIP = 328;  // NI padded to a multiple of 8 (zero rows)
-static_assert((NIP - NI) * LC == 256, "one padding float per thread of the layer kernel");
-constexpr int SM_W1T = NIP * NH, SM_W2T = NH * NH, SM_W3T = NH * NO, SM_XT = NIP * LC, SM_H = NH * LC;
-constexpr size_t LAYER_SMEM =
-    sizeof(float) * (SM_W1T + SM_W2T + SM_XT + 2 * SM_H + SM_W3T + 2 * NH + NO + 2 * LC + 4 * LC);
+// The layer is the domain's six faces.  On a face the third of a stencil
+// beyond the wall is zero, which leaves 216 of the 324 inputs: 24 planes (the
+// face's own and the next one inward, two levels, six components) x 3 x 3
+// taps in the face.  A group of four warps takes patches of 16 x 4 cells of a
+// face, stages their footprint (24 planes of 18 x 6 cells) and contracts it as an implicit
+// convolution: a warp holds one row of 16 cells, k runs over taps and, within
+// a tap, over the planes, so an operand fragment is read straight from the
+// footprint at the tap's offset.
+//
+// What bounds it: the tensor pipe (3 x 280 k-rows of 64 units a cell, 8
+// cycles an m16n8k8), beside the weights' fragments from shared memory (256
+// of 394 cycles a k-step).  The kernel before it gathered each cell's 324
+// inputs on their own (81 copies of 4 bytes a thread and tile, six times the
+// footprint) and moved the hidden layers through shared memory, with five
+// block barriers a tile: 160^3 (152 k cells) 258 us, now 105 (56 % of the
+// tensor pipe), a step 329 -> 157.  The
+// hidden layers now stay in registers: an accumulator fragment holds units 2q
+// and 2q + 1 of a row where an operand fragment wants k = q and q + 4, so the
+// second layer's k is taken in that order.
+constexpr int PU = 16, PV = 4;             // cells of a patch
+constexpr int FROW = 20, FPL = 136;        // footprint: floats of a row (18 used), of a plane (6 rows)
+constexpr int NPL = 24, KF = 9 * NPL;      // planes, inputs of a face cell
+constexpr int WP = 66;                     // pitch of a row of weight fragments, in fragments of 16 bytes
+static_assert((PU + 2) * (PV + 2) > 96 && (PU + 2) * (PV + 2) <= 128 && NPL == 6 * 4, "four elements of six planes a lane");
+static_assert(FPL >= (PV + 2) * FROW, "a plane's rows");
+static_assert(FPL % 32 == 8, "the four planes of a fragment on disjoint banks");
+static_assert(WP % 8 == 2, "the fragments of eight lanes on disjoint banks");
+constexpr int LS_W1 = 0, LS_W2 = LS_W1 + 4 * (KF / 2) * WP, LS_F = LS_W2 + 4 * (NH / 2) * WP, LS_W3 = LS_F + 4 * NPL * FPL,
+              LS_B = LS_W3 + NO * NH, LS_END = LS_B + 2 * NH + 8;
+static_assert(LS_W2 % 4 == 0 && LS_F % 4 == 0 && LS_W3 % 4 == 0, "16-byte copies");
+constexpr size_t LAYER_SMEM = sizeof(float) * LS_END;
+static_assert(LAYER_SMEM <= 227 * 1024, "one CTA's shared memory");
 
-// Asynchronous 4-byte copy, global -> shared (cp.async, cached in L1).  With
-// valid == false nothing is read and the shared word is zero-filled; src is
-// then still an address inside the field array.
-__device__ __forceinline__ void cp_async_4(float *dst, const float *src, bool valid)
+// Input k of the network that face f (0..5 = x low, x high, y low, ...) reads
+// as plane p = (depth * 2 + level) * 6 + component at tap (dv, du).
+__device__ __host__ __forceinline__ int face_input(int f, int p, int dv, int du)
 {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+    const int c = p % 6, lev = (p / 6) % 2, depth = p / 12;
+    const int axis = f >> 1, dn = f & 1 ? 1 - depth : 1 + depth;  // offset + 1 along the face's normal
+    // u, v: the other two axes, the lower one first
+    const int dx = axis == 0 ? dn : du, dy = axis == 1 ? dn : (axis == 0 ? du : dv), dz = axis == 2 ? dn : dv;
+    return (lev * 6 + c) * 27 + dz * 9 + dy * 3 + dx;
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Each band snapshot (six components at c * fstride, rows of `pitch`) is
-// followed by its x slab: the planes x = 0, 1 (side 0) and x = nx-2, nx-1
-// (side 1) of every component, y fastest, [comp][side][xd][z][y], so that
-// the stencils of the cells on the two x faces (a full row apart from each
-// other in the snapshot) are read with consecutive y across the lanes.
-__device__ __host__ __forceinline__ long long xslab_floats(int ny, int nz) { return 24LL * ny * nz; }
-
-// Stage the unnormalised stencils of `tile` into Xt ([k][cell], swizzled)
-// with asynchronous copies: thread -> cell q = tid % 64 and three of the
-// twelve (level, component) pairs, (tid / 64) * 3 + 0..2, each a 27-cell
-// stencil; neighbour offsets are unrolled, validity is per axis, neighbours
-// outside the domain and cells past the list are zero.  Cells on an x face
-// read the x slab, the others the snapshot itself (same values).
-__device__ __forceinline__ void stage_stencils(float *Xt, const float *__restrict__ cur,
-                                               const float *__restrict__ prev, long long fstride, int pitch,
-                                               int nx, int ny, int nz, const int *__restrict__ cells, int ncells,
-                                               int tile)
+// The first two layers' weights as the layer kernel reads them: fragment (step,
+// q, unit) holds the rows k = q and q + 4 of an eight-row step of k, split:
+// {hi(q), hi(q + 4), lo(q), lo(q + 4)}, so that one 16-byte load gives the two
+// register pairs of an operand.  W1 of each face [6][KF / 8][4][NH] (step tap *
+// 3 + p / 8, row p % 8), then W2 [NH / 8][4][NH] (step j, rows q and q + 4:
+// inputs 8j + 2q and 8j + 2q + 1).
+__global__ void __launch_bounds__(256) weight_image_kernel(const float *__restrict__ P, uint4 *__restrict__ img)
 {
-    const int tid = threadIdx.x, q = tid & (LC - 1), p0 = (tid >> 6) * 3;
-    const int cell = tile * LC + q;
-    if (cell < ncells) {
-        const int x = cells[3 * cell], y = cells[3 * cell + 1], z = cells[3 * cell + 2];
-        const bool vx[3] = {x > 0, true, x + 1 < nx}, vy[3] = {y > 0, true, y + 1 < ny},
-                   vz[3] = {z > 0, true, z + 1 < nz};
-        const long long nyz = (long long)ny * nz;
-        // address of (x', y', z') of component c: level base + c * cs + o0 + x' sx + y' sy + z' sz
-        long long sx = 1, sy = pitch, sz = (long long)pitch * ny, cs = fstride, o0 = 0;
-        if (x == 0 || x == nx - 1) {
-            const int side = x == 0 ? 0 : 1, base = side ? nx - 2 : 0;
-            sx = nyz, sy = 1, sz = ny, cs = 4 * nyz;
-            o0 = 6 * fstride + (2 * side - base) * nyz;
-        }
-        const long long centre = o0 + x * sx + y * sy + z * sz;
-        const long long ox[3] = {-sx, 0, sx}, oy[3] = {-sy, 0, sy}, oz[3] = {-sz, 0, sz};
-#pragma unroll 1
-        for (int pq = 0; pq < 3; ++pq) {
-            const int pr = p0 + pq, lev = pr / 6, comp = pr - lev * 6;
-            const float *src = (lev == 0 ? cur : prev) + comp * cs + centre;
-#pragma unroll
-            for (int d = 0; d < 27; ++d) {
-                const int dx = d % 3, dy = (d / 3) % 3, dz = d / 9;
-                const int k = pr * 27 + d;
-                const bool ok = vx[dx] && vy[dy] && vz[dz];
-                const float *a = ok ? src + (ox[dx] + oy[dy] + oz[dz]) : src;
-                cp_async_4(&Xt[k * LC + swz(k, q)], a, ok);
-            }
-        }
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    constexpr int N1 = 6 * KF / 2 * NH;
+    if (e >= N1 + NH / 2 * NH) return;
+    float v[2];
+    if (e < N1) {
+        const int u = e % NH, q = (e / NH) % 4, step = (e / (4 * NH)) % (KF / 8), f = e / (4 * NH * (KF / 8));
+        const int tap = step / 3, p = 8 * (step % 3) + q;
+        for (int i = 0; i < 2; ++i) v[i] = P[OFF_W1 + u * NI + face_input(f, p + 4 * i, tap / 3, tap % 3)];
     } else {
+        const int r = e - N1, u = r % NH, q = (r / NH) % 4, j = r / (4 * NH);
+        for (int i = 0; i < 2; ++i) v[i] = P[OFF_W2 + u * NH + 8 * j + 2 * q + i];
+    }
+    uint4 o;
+    split_tf32(v[0], o.x, o.z);
+    split_tf32(v[1], o.y, o.w);
+    img[e] = o;
+}
+
+// x, y, z of in-plane (u, v) of face f at depth d
+__device__ __forceinline__ void face_cell(const LearnedGeo &g, int f, int u, int v, int d, int &x, int &y, int &z)
+{
+    const int axis = f >> 1, n = axis == 0 ? g.nx : axis == 1 ? g.ny : g.nz, w = f & 1 ? n - 1 - d : d;
+    x = axis == 0 ? w : u;
+    y = axis == 1 ? w : (axis == 0 ? u : v);
+    z = axis == 2 ? w : v;
+}
+
+// The two planes of each face of the six components, as they are now: plane
+// (face, depth) of component c at face's offset + ((depth * 6 + c) * nv + v) *
+// nu + u.  A block takes one face, both depths (neighbours in memory on the x
+// faces) and one component.
+__global__ void __launch_bounds__(256) snapshot_kernel(const __grid_constant__ LearnedGeo g, const float *__restrict__ fld,
+                                                       long long fs, int pitch, float *__restrict__ snap)
+{
+    const int f = blockIdx.y / 6, c = blockIdx.y % 6;
+    const LearnedFace &F = g.face[f];
+    const int n = F.nu * F.nv;
+    for (int e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) {
+        const int v = e / F.nu, u = e - v * F.nu;
 #pragma unroll
-        for (int pq = 0; pq < 3; ++pq)
-#pragma unroll
-            for (int d = 0; d < 27; ++d) {
-                const int k = (p0 + pq) * 27 + d;
-                Xt[k * LC + swz(k, q)] = 0.f;
-            }
+        for (int d = 0; d < 2; ++d) {
+            if (d >= F.depth) break;
+            int x, y, z;
+            face_cell(g, f, u, v, d, x, y, z);
+            snap[F.snap + (long long)(d * 6 + c) * n + e] = fld[c * fs + x + (long long)pitch * (y + (long long)g.ny * z)];
+        }
     }
 }
 
-__global__ void __launch_bounds__(256, 1) layer_kernel(const float *__restrict__ P, const float *__restrict__ cur,
-                                                       const float *__restrict__ prev, long long fstride, int pitch,
-                                                       int nx, int ny, int nz, const int *__restrict__ cells,
-                                                       int ncells, float *__restrict__ out)
+// tanh without a branch, for the 128 evaluations a thread and patch that the
+// tensor cores otherwise wait for.  Below 1 the seventh convergent of
+// Lambert's continued fraction x / (1 + x^2 / (3 + x^2 / (5 + ...))) as x less
+// x times a quotient of polynomials in x^2 (its truncation error is under 1e-9
+// there), above it 1 - 2 / (exp(2 |x|) + 1); one reciprocal for both, refined
+// by a Newton step.  At most 2 units in the last place off (1.3 in a
+// float32 emulation over the range; tanhf is allowed 2), odd, NaN for NaN.
+__device__ __forceinline__ float tanh_fast(float x)
+{
+    const float a = fabsf(x) > 10.f ? 10.f : fabsf(x), t = __fmul_rn(a, a);  // (NaN stays)
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(a, 2.885390081777927f)));  // 2 log2(e)
+    const bool small = a < 1.f;
+    const float ns = __fmul_rn(__fmul_rn(a, t), __fmaf_rn(t, __fmaf_rn(t, 27.f, 2772.f), 45045.f));
+    const float ds = __fmaf_rn(t, __fmaf_rn(t, __fmaf_rn(t, 28.f, 3150.f), 62370.f), 135135.f);
+    const float n = small ? ns : 2.f, d = small ? ds : __fadd_rn(e, 1.f);
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+    r = __fmaf_rn(r, __fmaf_rn(-d, r, 1.f), r);
+    const float y = __fmaf_rn(-n, r, small ? a : 1.f);
+    return copysignf(y, x);
+}
+
+// Footprint of one patch into shared memory by asynchronous 4-byte copies;
+// cells beyond the face (and a second plane that does not exist) read 0.  A
+// warp takes six planes (`place`: where the lane's four elements of a plane lie,
+// row << 8 | column, the same for every plane and patch).
+__device__ __forceinline__ void stage_patch(const LearnedGeo &g, int f, int u0, int v0, const float *__restrict__ cur,
+                                            const float *__restrict__ prev, const int (&place)[4], float *dst)
+{
+    const LearnedFace &F = g.face[f];
+    const int n = F.nu * F.nv, w = (threadIdx.x >> 5) & 3;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int row = place[i] >> 8, col = place[i] & 255;
+        const int u = u0 + col - 1, v = v0 + row - 1;
+        const bool in = (unsigned)u < (unsigned)F.nu && (unsigned)v < (unsigned)F.nv;
+        const int o = in ? v * F.nu + u : 0;
+        const unsigned a = (unsigned)__cvta_generic_to_shared(dst + w * FPL + row * FROW + col);
+        if (i < 3 || row < PV + 2) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {  // planes w + 4 k: depth of plane p is p / 12, level (p / 6) % 2
+                const int p = w + 4 * k, d = k / 3, lc = p - 12 * d;
+                const bool ok = in && d < F.depth;
+                const float *const src = (lc < 6 ? cur : prev) + F.snap + (long long)(ok ? d * 6 + lc % 6 : 0) * n + o;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(a + 16u * k * FPL), "l"(src), "r"(ok ? 4 : 0)
+                             : "memory");
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ void copy16(float *dst, const float *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// Corrections r f(x / r) of the face cells from the snapshots of S^n (cur) and
+// S^{n-1} (prev): component o of cell `id` at out[o * cells + id].  Persistent:
+// a CTA takes a run of consecutive patches, so it changes face (and first-layer
+// weights) once at most in the usual grids.  Its two groups of four warps (one
+// of each on an SM sub-partition) take the run's patches in turn, the second
+// half a patch behind: while one evaluates tanh the other has the tensor cores.
+__device__ __forceinline__ void bar_group(int grp) { asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory"); }
+
+__global__ void __launch_bounds__(256, 1) layer_kernel(const __grid_constant__ LearnedGeo g, const float *__restrict__ P,
+                                                       const uint4 *__restrict__ img, const float *__restrict__ cur,
+                                                       const float *__restrict__ prev, float *__restrict__ out)
 {
     extern __shared__ __align__(16) float sm[];
-    float *W1t = sm;                  // [k][unit]
-    float *W2t = W1t + SM_W1T;        // [k][unit]
-    float *Xt = W2t + SM_W2T;         // [k][cell]: the unnormalised stencil
-    float *H1t = Xt + SM_XT;          // [unit][cell]
-    float *H2t = H1t + SM_H;
-    float *W3t = H2t + SM_H;          // [k][out]
-    float *b1 = W3t + SM_W3T, *b2 = b1 + NH, *b3 = b2 + NH;
-    float *rr = b3 + NO;              // r per cell
-    float *ir = rr + LC;              // 1/r per cell (0 if r = 0)
-    float *part = ir + LC;            // [4][cell] partial sums of x^2
-    const int tid = threadIdx.x;
-    const int ntiles = (ncells + LC - 1) / LC;
-    // the first tile's stencils are in flight while the weights are loaded
-    if ((int)blockIdx.x < ntiles)
-        stage_stencils(Xt, cur, prev, fstride, pitch, nx, ny, nz, cells, ncells, blockIdx.x);
-    for (int e = tid; e < NH * NI; e += 256) {
-        const int u = e / NI, k = e - u * NI;
-        W1t[k * NH + swz(k, u)] = P[OFF_W1 + e];
-    }
-    for (int e = tid; e < (NIP - NI) * NH; e += 256) W1t[NI * NH + e] = 0.f;  // padding rows
-    for (int e = tid; e < NH * NH; e += 256) {
-        const int u = e / NH, k = e - u * NH;
-        W2t[k * NH + swz(k, u)] = P[OFF_W2 + e];
-    }
-    for (int e = tid; e < NO * NH; e += 256) {
-        const int o = e / NH, k = e - o * NH;
-        W3t[k * NO + o] = P[OFF_W3 + e];
-    }
+    float *const W1 = sm + LS_W1, *const W2 = sm + LS_W2, *const FP = sm + LS_F, *const W3 = sm + LS_W3;
+    float *const b1 = sm + LS_B, *const b2 = b1 + NH, *const b3 = b2 + NH;
+    const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 3, grp = tid >> 7, gr = lane >> 2, q = lane & 3;
+    const int per = (g.patches + gridDim.x - 1) / gridDim.x;
+    const int first = blockIdx.x * per, last = min(first + per, g.patches);
+    if (first >= last) return;
+    auto face_of = [&](int patch) {
+        int f = 0;
+        while (patch >= g.face[f].patch0 + g.face[f].pu * g.face[f].pv) ++f;
+        return f;
+    };
+    auto origin = [&](int patch, int f, int &u0, int &v0) {
+        const LearnedFace &F = g.face[f];
+        const int r = patch - F.patch0;
+        u0 = F.u0 + PU * (r % F.pu);
+        v0 = F.v0 + PV * (r / F.pu);
+    };
+    auto load_w1 = [&](int f) {
+        const float *const src = reinterpret_cast<const float *>(img + (size_t)f * (KF / 2) * NH);
+        for (int e = tid; e < KF / 2 * NH; e += 256) copy16(W1 + 4 * ((e / NH) * WP + e % NH), src + 4 * e);
+    };
+    int place[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) place[i] = (lane + 32 * i) / (PU + 2) << 8 | (lane + 32 * i) % (PU + 2);
+    for (int e = tid; e < NO * NH; e += 256) W3[e] = P[OFF_W3 + e];
     if (tid < NH) {
         b1[tid] = P[OFF_B1 + tid];
         b2[tid] = P[OFF_B2 + tid];
     }
     if (tid < NO) b3[tid] = P[OFF_B3 + tid];
-    Xt[NI * LC + tid] = 0.f;  // padding rows of the stencil (256 zeros), never staged over
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        cp_async_wait_all();
-        __syncthreads();  // this tile's stencils have landed; the previous tile is done with H / rr
-        {
-            // sum of squares of the thread's own 81 staged values, in staging order
-            const int q = tid & (LC - 1), p0 = (tid >> 6) * 3;
-            float ss = 0.f;
-#pragma unroll
-            for (int pq = 0; pq < 3; ++pq)
-#pragma unroll
-                for (int d = 0; d < 27; ++d) {
-                    const int k = (p0 + pq) * 27 + d;
-                    const float v = Xt[k * LC + swz(k, q)];
-                    ss = __fmaf_rn(v, v, ss);
-                }
-            part[(tid >> 6) * LC + q] = ss;
+    {
+        const float *const src = reinterpret_cast<const float *>(img + (size_t)6 * (KF / 2) * NH);
+        for (int e = tid; e < NH / 2 * NH; e += 256) copy16(W2 + 4 * ((e / NH) * WP + e % NH), src + 4 * e);
+    }
+    float *const fpg = FP + grp * 2 * NPL * FPL;
+    for (int seg = first, seg_end; seg < last; seg = seg_end) {  // the run's patches on one face
+        const int f = face_of(seg);
+        const LearnedFace &F = g.face[f];
+        seg_end = min(last, F.patch0 + F.pu * F.pv);
+        int u0, v0;
+        if (seg != first) __syncthreads();  // everybody is past the previous face's weights
+        load_w1(f);
+        if (seg + grp < seg_end) {
+            origin(seg + grp, f, u0, v0);
+            stage_patch(g, f, u0, v0, cur, prev, place, fpg);
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (tid < LC) {
-            const float ss = part[tid] + part[LC + tid] + part[2 * LC + tid] + part[3 * LC + tid];
-            const float r = sqrtf(ss / NI);
-            const bool live = r >= R_MIN;  // smaller r: the cell keeps its value
-            rr[tid] = live ? r : 0.f;
-            ir[tid] = live ? 1.f / r : 0.f;
+    for (int patch = seg + grp, it = 0; patch < seg_end; patch += 2, ++it) {
+        if (it) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            bar_group(grp);  // this patch's footprint has landed; the other buffer is free
         }
-        __syncthreads();
-        // layers 1 and 2 on the tensor cores (3xTF32): H1 = tanh((W1 x) / r +
-        // b1), H2 = tanh(W2 H1 + b2); warp w holds cells 16*(w%4) + g (+8) and
-        // units 32*(w/4) + 8j + 2q (+1) of its accumulator fragments
-        {
-            const int lane = tid & 31, w = tid >> 5, g = lane >> 2, q = lane & 3;
-            const int m0 = 16 * (w & 3), n0 = 32 * (w >> 2);
-            float acc[4][4];
-            warp_gemm_3xtf32<NIP>(Xt, W1t, acc);
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int cell = m0 + g + 8 * (e >> 1), unit = n0 + 8 * j + 2 * q + (e & 1);
-                    H1t[unit * LC + swz(unit, cell)] = tanhf(__fmaf_rn(acc[j][e], ir[cell], b1[unit]));
-                }
-            __syncthreads();  // every warp is past layer 1's reads of Xt
-            // the next tile's stencils fly while layers 2 and 3 run
-            const int next = tile + gridDim.x;
-            if (next < ntiles) stage_stencils(Xt, cur, prev, fstride, pitch, nx, ny, nz, cells, ncells, next);
-            warp_gemm_3xtf32<NH>(H1t, W2t, acc);
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int cell = m0 + g + 8 * (e >> 1), unit = n0 + 8 * j + 2 * q + (e & 1);
-                    H2t[unit * LC + swz(unit, cell)] = tanhf(__fadd_rn(acc[j][e], b2[unit]));
-                }
+        origin(patch, f, u0, v0);
+        if (patch + 2 < seg_end) {
+            int nu0, nv0;
+            origin(patch + 2, f, nu0, nv0);
+            stage_patch(g, f, nu0, nv0, cur, prev, place, fpg + ((it + 1) & 1) * NPL * FPL);
         }
-        __syncthreads();
-        // layer 3: the correction r f added to the Yee step later
-        for (int e = tid; e < LC * NO; e += 256) {
-            const int q = e / NO, o = e - q * NO;
-            const int cell = tile * LC + q;
-            if (cell >= ncells) continue;
-            float f = b3[o];
-            for (int k = 0; k < NH; ++k) f = __fmaf_rn(H2t[k * LC + swz(k, q)], W3t[k * NO + o], f);
-            const unsigned m = tangent_mask(cells[3 * cell], cells[3 * cell + 1], cells[3 * cell + 2], nx, ny, nz);
-            out[(long long)cell * NO + o] = (m >> o) & 1u ? __fmul_rn(rr[q], f) : 0.f;
+        // the second group's first patch starts once the first group is through
+        // its first layer
+        if (it == 0 && grp == 1) asm volatile("bar.sync 3, 256;" ::: "memory");
+        const float *const fp = fpg + (it & 1) * NPL * FPL + w * FROW + gr;
+        float acc[8][4];
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+        // layer 1 on the unnormalised inputs, and the sum of their squares (rows
+        // gr and gr + 8 of the warp's 16 cells)
+        float ss0 = 0.f, ss1 = 0.f;
+        const uint4 *wr = reinterpret_cast<const uint4 *>(W1) + q * WP + gr;
+#pragma unroll 1
+        for (int tap = 0; tap < 9; ++tap) {
+            const float *const ft = fp + (tap / 3) * FROW + tap % 3;
+#pragma unroll
+            for (int j = 0; j < 3; ++j, wr += 4 * WP) {
+                const float x0 = ft[(8 * j + q) * FPL], x1 = ft[(8 * j + q) * FPL + 8];
+                const float x2 = ft[(8 * j + q + 4) * FPL], x3 = ft[(8 * j + q + 4) * FPL + 8];
+                ss0 = __fmaf_rn(x0, x0, __fmaf_rn(x2, x2, ss0));
+                ss1 = __fmaf_rn(x1, x1, __fmaf_rn(x3, x3, ss1));
+                unsigned ah[4], al[4];
+                split_tf32(x0, ah[0], al[0]);
+                split_tf32(x1, ah[1], al[1]);
+                split_tf32(x2, ah[2], al[2]);
+                split_tf32(x3, ah[3], al[3]);
+                contract(acc, ah, al, wr);
+            }
+        }
+#pragma unroll
+        for (int d = 1; d < 4; d <<= 1) {
+            ss0 = __fadd_rn(ss0, __shfl_xor_sync(0xffffffffu, ss0, d));
+            ss1 = __fadd_rn(ss1, __shfl_xor_sync(0xffffffffu, ss1, d));
+        }
+        const float r0 = sqrtf(ss0 / NI), r1 = sqrtf(ss1 / NI);
+        const bool live0 = r0 >= R_MIN, live1 = r1 >= R_MIN;  // smaller r: the cell keeps its value
+        const float ir0 = live0 ? 1.f / r0 : 0.f, ir1 = live1 ? 1.f / r1 : 0.f;
+        if (it == 0 && grp == 0 && seg + 1 < seg_end) asm volatile("bar.arrive 3, 256;" ::: "memory");
+        // H1 = tanh((W1 x) / r + b1), in place
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const float2 b = *reinterpret_cast<const float2 *>(b1 + 8 * n + 2 * q);
+            acc[n][0] = tanh_fast(__fmaf_rn(acc[n][0], ir0, b.x));
+            acc[n][1] = tanh_fast(__fmaf_rn(acc[n][1], ir0, b.y));
+            acc[n][2] = tanh_fast(__fmaf_rn(acc[n][2], ir1, b.x));
+            acc[n][3] = tanh_fast(__fmaf_rn(acc[n][3], ir1, b.y));
+        }
+        // layer 2: operand fragment j from accumulator fragment j
+        float acc2[8][4];
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc2[n][e] = 0.f;
+        const uint4 *const w2 = reinterpret_cast<const uint4 *>(W2) + q * WP + gr;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            unsigned ah[4], al[4];
+            split_tf32(acc[j][0], ah[0], al[0]);
+            split_tf32(acc[j][2], ah[1], al[1]);
+            split_tf32(acc[j][1], ah[2], al[2]);
+            split_tf32(acc[j][3], ah[3], al[3]);
+            contract(acc2, ah, al, w2 + 4 * j * WP);
+        }
+        // layer 3 in FP32: a lane's 16 units of its two rows, then the four lanes of a row
+        float y0[NO], y1[NO];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) y0[o] = y1[o] = 0.f;
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            const float2 b = *reinterpret_cast<const float2 *>(b2 + 8 * n + 2 * q);
+            const float h00 = tanh_fast(__fadd_rn(acc2[n][0], b.x)), h01 = tanh_fast(__fadd_rn(acc2[n][1], b.y));
+            const float h10 = tanh_fast(__fadd_rn(acc2[n][2], b.x)), h11 = tanh_fast(__fadd_rn(acc2[n][3], b.y));
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                const float2 c = *reinterpret_cast<const float2 *>(W3 + o * NH + 8 * n + 2 * q);
+                y0[o] = __fmaf_rn(h01, c.y, __fmaf_rn(h00, c.x, y0[o]));
+                y1[o] = __fmaf_rn(h11, c.y, __fmaf_rn(h10, c.x, y1[o]));
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < NO; ++o)
+#pragma unroll
+            for (int d = 1; d < 4; d <<= 1) {
+                y0[o] = __fadd_rn(y0[o], __shfl_xor_sync(0xffffffffu, y0[o], d));
+                y1[o] = __fadd_rn(y1[o], __shfl_xor_sync(0xffffffffu, y1[o], d));
+            }
+        // lane q writes components q and q + 4 of cells (u0 + gr, v0 + w) and (u0 + gr + 8, v0 + w)
+        const int v = v0 + w;
+        if (v < F.v1) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int u = u0 + gr + 8 * h;
+                if (u >= F.u1) continue;
+                const long long id = F.cell0 + (long long)(v - F.v0) * (F.u1 - F.u0) + (u - F.u0);
+                const float r = h ? (live1 ? r1 : 0.f) : (live0 ? r0 : 0.f);
+#pragma unroll
+                for (int o = 0; o < NO; ++o)
+                    if ((o & 3) == q) out[o * g.cells + id] = __fmul_rn(r, __fadd_rn(h ? y1[o] : y0[o], b3[o]));
+            }
         }
     }
-    cp_async_wait_all();  // nothing left in flight at exit
-}
-
-__global__ void __launch_bounds__(256) scatter_kernel(float *__restrict__ f, long long fstride, int pitch, int ny,
-                                                      const int *__restrict__ cells, int ncells,
-                                                      const float *__restrict__ vals)
-{
-    const int q = blockIdx.x * 256 + threadIdx.x;
-    if (q >= ncells) return;
-    const long long p = cells[3 * q] + (long long)pitch * (cells[3 * q + 1] + (long long)ny * cells[3 * q + 2]);
-    for (int c = 0; c < NO; ++c) f[c * fstride + p] = __fadd_rn(f[c * fstride + p], vals[(long long)q * NO + c]);
-}
-
-__global__ void __launch_bounds__(256) copy_cells_kernel(float *__restrict__ dst, const float *__restrict__ src,
-                                                         long long fstride, int pitch, int ny,
-                                                         const int *__restrict__ cells, int ncells)
-{
-    const int q = blockIdx.x * 256 + threadIdx.x;
-    if (q >= ncells) return;
-    const long long p = cells[3 * q] + (long long)pitch * (cells[3 * q + 1] + (long long)ny * cells[3 * q + 2]);
-    for (int c = 0; c < NO; ++c) dst[c * fstride + p] = src[c * fstride + p];
-}
-
-// The x slab of a band snapshot (layout above): element e of the slab is
-// (comp, side, xd, z, y) in that order, y fastest; planes outside the grid
-// (nx < 2) are zero and never read.
-__global__ void __launch_bounds__(256) fill_xslab_kernel(float *__restrict__ snap, const float *__restrict__ f,
-                                                         long long fstride, int pitch, int nx, int ny, int nz)
-{
-    const long long n = xslab_floats(ny, nz);
-    float *slab = snap + 6 * fstride;
-    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < n; e += (long long)gridDim.x * 256) {
-        const int y = (int)(e % ny);
-        long long r = e / ny;
-        const int z = (int)(r % nz);
-        r /= nz;
-        const int xd = (int)(r & 1), side = (int)((r >> 1) & 1), comp = (int)(r >> 2);
-        const int x = side ? nx - 2 + xd : xd;
-        slab[e] = (x >= 0 && x < nx) ? f[comp * fstride + x + (long long)pitch * (y + (long long)ny * z)] : 0.f;
     }
+}
+
+// The corrections added to the components that the walls get wrong.
+__global__ void __launch_bounds__(256) scatter_kernel(const __grid_constant__ LearnedGeo g, float *__restrict__ fld,
+                                                      long long fs, int pitch, const float *__restrict__ vals)
+{
+    const LearnedFace &F = g.face[blockIdx.y];
+    const int nu = F.u1 - F.u0, n = nu * (F.v1 - F.v0);
+    const int e = blockIdx.x * 256 + threadIdx.x;
+    if (e >= n) return;
+    const int v = e / nu, u = e - v * nu;
+    int x, y, z;
+    face_cell(g, blockIdx.y, F.u0 + u, F.v0 + v, 0, x, y, z);
+    const unsigned m = tangent_mask(x, y, z, g.nx, g.ny, g.nz);
+    const long long p = x + (long long)pitch * (y + (long long)g.ny * z);
+#pragma unroll
+    for (int c = 0; c < NO; ++c)
+        if ((m >> c) & 1u) fld[c * fs + p] = __fadd_rn(fld[c * fs + p], vals[c * g.cells + F.cell0 + e]);
 }
 
 } // namespace
@@ -966,47 +1071,73 @@ cudaError_t mlp_record_box(const float *f, long long fstride, int pitch, int ny,
     return cudaGetLastError();
 }
 
-size_t learned_layer_smem() { return LAYER_SMEM; }
-
-cudaError_t learned_layer_configure()
+LearnedGeo learned_geometry(int nx, int ny, int nz)
 {
-    return cudaFuncSetAttribute(layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LAYER_SMEM);
+    LearnedGeo g = {};
+    g.nx = nx;
+    g.ny = ny;
+    g.nz = nz;
+    const int n[3] = {nx, ny, nz};
+    long long snap = 0, cell = 0;
+    int patch = 0;
+    for (int f = 0; f < 6; ++f) {
+        LearnedFace &F = g.face[f];
+        const int axis = f >> 1, ua = axis == 0 ? 1 : 0, va = axis == 2 ? 1 : 2;
+        F.nu = n[ua];
+        F.nv = n[va];
+        F.depth = std::min(2, n[axis]);
+        // each cell belongs to one face: all of the z faces', of the y faces' those
+        // between them, of the x faces' the rest; one face where a domain is one cell thick
+        F.u0 = axis == 0 ? std::min(1, ny) : 0;
+        F.u1 = axis == 0 ? std::max(F.u0, ny - 1) : F.nu;
+        F.v0 = axis == 2 ? 0 : std::min(1, nz);
+        F.v1 = axis == 2 ? F.nv : std::max(F.v0, nz - 1);
+        if ((f & 1) && n[axis] == 1) F.u1 = F.u0;
+        const bool none = F.u1 <= F.u0 || F.v1 <= F.v0;
+        F.pu = none ? 0 : (F.u1 - F.u0 + PU - 1) / PU;
+        F.pv = none ? 0 : (F.v1 - F.v0 + PV - 1) / PV;
+        if (none) F.u1 = F.u0;
+        F.snap = snap;
+        F.cell0 = cell;
+        F.patch0 = patch;
+        snap += 12ll * F.nu * F.nv;
+        cell += (long long)(F.u1 - F.u0) * (F.v1 - F.v0);
+        patch += F.pu * F.pv;
+    }
+    g.snap_floats = snap;
+    g.cells = cell;
+    g.patches = patch;
+    return g;
 }
 
-cudaError_t learned_layer_predict(const float *params, const float *cur, const float *prev, long long fstride,
-                                  int pitch, int nx, int ny, int nz, const int *cells, int ncells, float *out,
-                                  int grid, cudaStream_t st)
+size_t learned_image_bytes() { return sizeof(uint4) * (6 * (size_t)(KF / 2) * NH + NH / 2 * NH); }
+
+cudaError_t learned_layer_configure(const float *params, void *image, cudaStream_t st)
 {
-    if (ncells <= 0) return cudaSuccess;
-    const int tiles = (ncells + LC - 1) / LC;
-    layer_kernel<<<std::min(grid, tiles), 256, LAYER_SMEM, st>>>(params, cur, prev, fstride, pitch, nx, ny, nz, cells,
-                                                                 ncells, out);
+    CKE(cudaFuncSetAttribute(layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LAYER_SMEM));
+    weight_image_kernel<<<((6 * KF + NH) / 2 * NH + 255) / 256, 256, 0, st>>>(params, (uint4 *)image);
     return cudaGetLastError();
 }
 
-cudaError_t learned_layer_scatter(float *f, long long fstride, int pitch, int ny, const int *cells, int ncells,
-                                  const float *vals, cudaStream_t st)
+cudaError_t learned_snapshot(const LearnedGeo &g, const float *f, long long fs, int pitch, float *snap, cudaStream_t st)
 {
-    if (ncells <= 0) return cudaSuccess;
-    scatter_kernel<<<(ncells + 255) / 256, 256, 0, st>>>(f, fstride, pitch, ny, cells, ncells, vals);
+    const long long n = std::max(std::max((long long)g.nx * g.ny, (long long)g.nx * g.nz), (long long)g.ny * g.nz);
+    snapshot_kernel<<<dim3((unsigned)std::min<long long>((n + 255) / 256, 4096), 36), 256, 0, st>>>(g, f, fs, pitch, snap);
     return cudaGetLastError();
 }
 
-cudaError_t learned_copy_cells(float *dst, const float *src, long long fstride, int pitch, int ny, const int *cells,
-                               int ncells, cudaStream_t st)
+cudaError_t learned_layer_predict(const LearnedGeo &g, const float *params, const void *image, const float *cur,
+                                  const float *prev, float *out, int grid, cudaStream_t st)
 {
-    if (ncells <= 0) return cudaSuccess;
-    copy_cells_kernel<<<(ncells + 255) / 256, 256, 0, st>>>(dst, src, fstride, pitch, ny, cells, ncells);
+    layer_kernel<<<std::min(grid, g.patches), 256, LAYER_SMEM, st>>>(g, params, (const uint4 *)image, cur, prev, out);
     return cudaGetLastError();
 }
 
-size_t learned_xslab_bytes(int ny, int nz) { return sizeof(float) * (size_t)xslab_floats(ny, nz); }
-
-cudaError_t learned_fill_xslab(float *snap, const float *f, long long fstride, int pitch, int nx, int ny, int nz,
-                               cudaStream_t st)
+cudaError_t learned_layer_scatter(const LearnedGeo &g, float *f, long long fs, int pitch, const float *vals,
+                                  cudaStream_t st)
 {
-    const long long n = xslab_floats(ny, nz);
-    const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    fill_xslab_kernel<<<blocks, 256, 0, st>>>(snap, f, fstride, pitch, nx, ny, nz);
+    int most = 0;
+    for (const LearnedFace &F : g.face) most = std::max(most, (F.u1 - F.u0) * (F.v1 - F.v0));
+    scatter_kernel<<<dim3((unsigned)((most + 255) / 256), 6), 256, 0, st>>>(g, f, fs, pitch, vals);
     return cudaGetLastError();
 }

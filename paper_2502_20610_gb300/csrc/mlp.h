@@ -31,24 +31,35 @@ cudaError_t mlp_record(const float *prev, const float *cur, const float *nxt, lo
                        const int lo[3], const int hi[3], const int *cells, int n, const float *ce, const float *ca,
                        float neg_dt, float *X, float *Y, cudaStream_t st);
 
-// Layer update of a simulation step (FP32 fields at f + c*fstride, rows of
-// `pitch`): corrections r f for `ncells` layer cells (x,y,z triplets) from
-// the current and previous band snapshots (each followed by its x slab,
-// below) into out [ncells][6]; scatter adds them to the cells after the Yee
-// step.
-size_t learned_layer_smem();
-cudaError_t learned_layer_configure();
-cudaError_t learned_layer_predict(const float *params, const float *cur, const float *prev, long long fstride,
-                                  int pitch, int nx, int ny, int nz, const int *cells, int ncells, float *out,
-                                  int grid, cudaStream_t st);
-cudaError_t learned_layer_scatter(float *f, long long fstride, int pitch, int ny, const int *cells, int ncells,
-                                  const float *vals, cudaStream_t st);
-cudaError_t learned_copy_cells(float *dst, const float *src, long long fstride, int pitch, int ny, const int *cells,
-                               int ncells, cudaStream_t st);
-// A band snapshot (6 * fstride floats) is followed by its x slab: the planes
-// x = 0, 1, nx-2, nx-1 of the six components, y fastest, which the layer
-// update reads for the cells on the two x faces.  learned_fill_xslab copies
-// them from the fields f into the slab of `snap`.
-size_t learned_xslab_bytes(int ny, int nz);
-cudaError_t learned_fill_xslab(float *snap, const float *f, long long fstride, int pitch, int nx, int ny, int nz,
-                               cudaStream_t st);
+// The learned layer's geometry: the six faces of the domain (0..5 = x low, x
+// high, y low, ...), each with in-plane axes u, v (the other two, the lower one
+// first) of nu x nv cells.  A face computes the cells [u0, u1) x [v0, v1) of
+// its plane (each cell of the layer belongs to one face), numbered from
+// cell0, u fastest, in pu x pv patches from patch0; `depth` planes (itself
+// and the next inward, if there is one) of the six components are kept in a
+// snapshot from float `snap`.
+struct LearnedFace {
+    int nu, nv, depth;
+    int u0, u1, v0, v1;
+    int pu, pv, patch0;
+    long long snap, cell0;
+};
+struct LearnedGeo {
+    int nx, ny, nz, patches;
+    LearnedFace face[6];
+    long long snap_floats, cells;
+};
+LearnedGeo learned_geometry(int nx, int ny, int nz);
+
+// Layer update of a simulation step (FP32 fields at f + c*fs, rows of `pitch`):
+// a snapshot of the faces' planes; the corrections r f of the layer's cells
+// from the snapshots of S^n and S^{n-1} into out [6][cells]; the corrections
+// added after the Yee step.  `image`: learned_image_bytes() of weights in the
+// kernel's order, made once by learned_layer_configure.
+size_t learned_image_bytes();
+cudaError_t learned_layer_configure(const float *params, void *image, cudaStream_t st);
+cudaError_t learned_snapshot(const LearnedGeo &g, const float *f, long long fs, int pitch, float *snap, cudaStream_t st);
+cudaError_t learned_layer_predict(const LearnedGeo &g, const float *params, const void *image, const float *cur,
+                                  const float *prev, float *out, int grid, cudaStream_t st);
+cudaError_t learned_layer_scatter(const LearnedGeo &g, float *f, long long fs, int pitch, const float *vals,
+                                  cudaStream_t st);
