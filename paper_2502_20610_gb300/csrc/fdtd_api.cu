@@ -93,11 +93,14 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
         off = align_up(off + sizeof(float) * (size_t)mlpnet::NPARAM);
         L.image = off;
         off = align_up(off + learned_image_bytes());
-        // two snapshots (S^{n-1}, S^n)
+        // two snapshots (S^{n-1}, S^n) of the faces, each in the room of a whole
+        // state and its x planes (the workspace keeps that size)
+        const size_t room = std::max(sizeof(float) * (size_t)geo.snap_floats,
+                                     6 * align_up(sizeof(float) * (size_t)n) + 96 * (size_t)g.ny * g.nz);
         L.prev = off;
-        off = align_up(off + sizeof(float) * (size_t)geo.snap_floats);
+        off = align_up(off + room);
         L.snap = off;
-        off = align_up(off + sizeof(float) * (size_t)geo.snap_floats);
+        off = align_up(off + room);
         L.pred = off;
         off = align_up(off + 6 * sizeof(float) * (size_t)geo.cells);
     }
@@ -671,7 +674,8 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     if (e == cudaSuccess) e = cudaMemsetAsync(h->ctrl, 0, 64 * sizeof(int), h->stream);
     if (e == cudaSuccess && learned) {
         e = cudaMemcpyAsync(h->params, boundary->model, sizeof(float) * mlpnet::NPARAM, cudaMemcpyDefault, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + L.prev, 0, L.pred - L.prev, h->stream);  // both snapshots
+        for (size_t q : {L.prev, L.snap})
+            if (e == cudaSuccess) e = cudaMemsetAsync(h->ws + q, 0, sizeof(float) * (size_t)h->geo.snap_floats, h->stream);
         if (e == cudaSuccess) e = learned_layer_configure(h->params, h->image, h->stream);
         // the network's stream: highest priority, so its CTAs are placed first
         // and the Yee kernels fill the rest of each SM
@@ -782,7 +786,10 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src)
         CK(cudaMemsetAsync(zero, 0, nzero * sizeof(int), h->stream));
     }
     // S^{n-1} := 0 (both snapshots: which is "previous" alternates)
-    if (h->prev) CK(cudaMemsetAsync(h->ws + h->L.prev, 0, h->L.pred - h->L.prev, h->stream));
+    if (h->prev) {
+        CK(cudaMemsetAsync(h->ws + h->L.prev, 0, sizeof(float) * (size_t)h->geo.snap_floats, h->stream));
+        CK(cudaMemsetAsync(h->ws + h->L.snap, 0, sizeof(float) * (size_t)h->geo.snap_floats, h->stream));
+    }
     h->failed = false;
     return FDTD_OK;
 }
