@@ -60,9 +60,15 @@
 // the y face goes to the y-face buffer one step late, from the warp whose y
 // slot leaves, while it sits out the H half-step; the x face goes to the
 // x-face buffer at the end of each step.  A tile therefore publishes level
-// t-1 after the second barrier of step t.  Two block barriers per step: after
-// the E rows are exchanged for the H half-step, and after the H rows are
-// exchanged for the E half-step.
+// t-1 after the second barrier of step t.
+//
+// Two barriers per step: B1, after the E rows are exchanged for the H
+// half-step, and B2, after the H rows are exchanged for the E half-step.  A
+// warp arrives as soon as its rows are written (the H rows are written as they
+// are computed) and waits only when it needs its neighbour's: its z and x face
+// stores lie between arrival and wait of B1, its refills between those of B2.
+// With block barriers after the stores and refills: 201 GCUPS at 256^3, 216 at
+// 512^3, FP16 188 at 256^3, lossy 162 at 224^3; so 208, 223, 197 and 167.
 //
 // Masks: none but the low walls'.  A cell outside the domain has dt/eps = 0
 // (the coefficient shells are zero-filled there), so its E stays 0; its H is
@@ -176,9 +182,7 @@ struct RegTile {
 
 __device__ __forceinline__ float shfl_from(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-// Named barriers: the compute warps among themselves (16 warps), and with the
-// bookkeeping warp at a tile's start.
-__device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+// Named barrier of the compute warps with the bookkeeping warp at a tile's start.
 __device__ __forceinline__ void bar_tile() { asm volatile("bar.sync 2, 544;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -377,6 +381,33 @@ __device__ bool wait_stage(const SysLaunch &P, unsigned long long *bar, unsigned
     }
 }
 
+// The two barriers of a step, as an arrival of each compute warp (once its
+// lanes' shared-memory accesses before it are done) and a wait later: what a
+// warp does in between holds nobody up.  The wait is bounded and ends when the
+// CTA gives up (*quit); every lane gets the same answer.
+__device__ __forceinline__ void half_arrive(unsigned long long *bar)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ bool half_wait(const SysLaunch &P, unsigned long long *bar, unsigned parity, const int *quit,
+                                          int ticket)
+{
+    unsigned long long t0 = 0;
+    for (;;) {
+        unsigned done;
+        asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;"
+                     " selp.u32 %0, 1, 0, p; }"
+                     : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+        if (__all_sync(0xffffffffu, done)) return true;
+        bool late = past(t0, 4 * (unsigned long long)P.timeout_ns);
+        if (late) timed_out(P.ctrl, ticket, -4);
+        late |= *(const volatile int *)quit != 0;
+        if (__any_sync(0xffffffffu, late)) return false;
+    }
+}
+
 template <class R>
 __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_constant__ SysLaunch P)
 {
@@ -416,7 +447,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     // the CTA's life, and the current tile's last finished level (its progress
     // value less the epoch); s_quit: it has given up waiting
     __shared__ unsigned s_steps, s_level, s_quit;
-    __shared__ unsigned s_steps2;  // B2 barriers passed (lossy)
+    __shared__ alignas(8) unsigned long long s_half[3];  // B1 and B2 (lossy: and a step's coefficients read)
     __shared__ int s_pfail;  // ... before the tile's first step
     __shared__ unsigned s_seen[3];
 
@@ -465,10 +496,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 
     constexpr int CR = R::CR;
     if (tid == 0) {
-        s_steps = s_steps2 = s_quit = 0u;
+        s_steps = s_quit = 0u;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[0])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[1])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[2])) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_half[0])), "r"(R::RY) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_half[1])), "r"(R::RY) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_half[2])), "r"(R::RY) : "memory");
         if constexpr (R::CL == 2) {
 #pragma unroll
             for (int k = 0; k < R::NSLOT; ++k) {
@@ -551,9 +585,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             unsigned long long t_up = 0, t_own = 0;  // waiting for the upwind tiles, for the compute warps
             while (ok && (t <= iv.e || (R::LOSSY && tc <= iv.e) || pub != (unsigned)iv.e + 1u)) {
                 bool idle = true;
-                if (R::LOSSY && tc <= iv.e) {  // the coefficients' buffer: free once B2 of step tc - 1 has been passed
-                    const unsigned passed2 = __shfl_sync(0xffffffffu, ld_acq_cta(&s_steps2), 0);
-                    if (tc == iv.s || (int)(passed2 - (steps0 + (unsigned)(tc - iv.s))) >= 0) {
+                if (R::LOSSY && tc <= iv.e) {  // the coefficients' buffer: free once step tc - 1 has read it
+                    unsigned read = 1;
+                    if (n2 > 0)  // (reads of fill n2 - 1; the compute warps cannot be a phase ahead of it)
+                        asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;"
+                                     " selp.u32 %0, 1, 0, p; }"
+                                     : "=r"(read) : "r"(smem_u32(&s_half[2])), "r"((n2 - 1u) & 1u) : "memory");
+                    if (__all_sync(0xffffffffu, read)) {
                         idle = false;
                         if (lane == 0) {
                             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&s_bar[2])),
@@ -614,7 +652,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 }
             }
             if (!ok && lane == 0) st_rel_cta(&s_quit, 1u);
-            steps0 += (unsigned)(iv.e - iv.s + 1);
+            steps0 += (unsigned)(iv.e - iv.s + 2);  // (one pass more than steps)
         }
         // no copy may still be writing when the CTA's shared memory goes (after an
         // abort some were never waited for)
@@ -630,10 +668,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 
     // ------------------------------------------------------- compute warps
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R::CREG));
-    // fills waited for on each buffer (every thread waits on every fill, so
-    // every thread keeps the same counts), B1 barriers passed
-    unsigned n_wait0 = 0, n_wait1 = 0, nsteps = 0;
-    unsigned n_wait2 = 0, nsteps2 = 0;  // (lossy)
+    // passes over the step loop (phases of B1 and of B2), and the parities of the
+    // next fill of each staging buffer (bits 0, 1; lossy: 2, the coefficients):
+    // every thread waits for every phase and keeps the same counts
+    unsigned n_half = 0, fills = 0;
     // the coefficient ring's row of physical z = bz - 1 + i, with zr the row of
     // bz - 1 (lossless: any number congruent to it)
     auto ring = [](int zr, int i) {
@@ -754,6 +792,26 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const int hi = min(min(iv.e, Ax - s.i + TX - 1), min(Ay - s.j + TY - 1, Az - s.k + TZ - 1));
             tile_src |= lo <= hi;
         }
+        // A. publish E^t (old) rows for the warp below's H half-step, and arrive at
+        //    the barrier before it
+        auto publish_e = [&]() {
+            if constexpr (R::VX) {
+                float *const qx = XEx + xe_at(w, 0, lane), *const qz = XEz + xe_at(w, 0, lane);
+#pragma unroll
+                for (int i = 0; i < NZ; i += 4) {
+                    *reinterpret_cast<float4 *>(qx + i) = make_float4(ex[i], ex[i + 1], ex[i + 2], ex[i + 3]);
+                    *reinterpret_cast<float4 *>(qz + i) = make_float4(ez[i], ez[i + 1], ez[i + 2], ez[i + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < NZ; ++i) {
+                    XEx[xe_at(w, i, lane)] = ex[i];
+                    XEz[xe_at(w, i, lane)] = ez[i];
+                }
+            }
+            half_arrive(&s_half[0]);
+        };
+        publish_e();
         for (int t = iv.s;; ++t, zl = R::LOSSY ? (zl == 0 ? CR - 1 : zl - 1) : 0) {
             // (one pass more than steps: the last step's top y face)
             const int bx = Ax - t, by = Ay - t, bz = Az - t;  // box low corner at step t
@@ -785,23 +843,11 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             // lane moves to bx - 1)
             const int xw = (bx - 1) + ((lane - bx + 1) & 31);
 
-            // A. publish E^t (old) rows for the warp below's H half-step
-            if constexpr (R::VX) {
-                float *const qx = XEx + xe_at(w, 0, lane), *const qz = XEz + xe_at(w, 0, lane);
-#pragma unroll
-                for (int i = 0; i < NZ; i += 4) {
-                    *reinterpret_cast<float4 *>(qx + i) = make_float4(ex[i], ex[i + 1], ex[i + 2], ex[i + 3]);
-                    *reinterpret_cast<float4 *>(qz + i) = make_float4(ez[i], ez[i + 1], ez[i + 2], ez[i + 3]);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < NZ; ++i) {
-                    XEx[xe_at(w, i, lane)] = ex[i];
-                    XEz[xe_at(w, i, lane)] = ez[i];
-                }
-            }
-            bar_compute();  // B1
-            if (tid == 0 && t <= iv.e) st_rel_cta(&s_steps, ++nsteps);
+            if (!half_wait(P, &s_half[0], n_half & 1u, &s_abort, ticket)) s_abort = 1;  // B1
+            // (a wait of the step before may have run out: every warp sees it here)
+            if (s_abort) { abort = true; break; }
+            ++n_half;
+            if (tid == 0) st_rel_cta(&s_steps, n_half);
             // x pairs: this step's x face travels through ring slot `slot`
             const bool msg = R::CL == 2 && t >= m_lo && t <= m_hi;
             const bool rx_msg = msg && rank == 1, tx_msg = msg && rank == 0;
@@ -840,6 +886,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 // before either is written, so 16-bit storage rounds two new
                 // values with one packed conversion
                 const float *const qx = XEx + xe_at(wn, 0, lane), *const qz = XEz + xe_at(wn, 0, lane);
+                float *const hxo = XHx + xe_at(w, 0, lane), *const hzo = XHz + xe_at(w, 0, lane);
                 {
                     float4 gx, gz;  // VX: the y+1 neighbour's E rows 4q .. 4q+3
 #pragma unroll
@@ -868,19 +915,31 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                         RND2(nh[0][2], nh[1][2], 5);
                         hx[i] = nh[0][0]; hy[i] = nh[0][1]; hz[i] = nh[0][2];
                         hx[i - 1] = nh[1][0]; hy[i - 1] = nh[1][1]; hz[i - 1] = nh[1][2];
+                        // published for the warp above's E half-step as they come (the
+                        // last readers are behind B1; the x-shell lane's are not used)
+                        if (!R::VX) {
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                hxo[(i - k - 1) * 32] = hx[i - k];
+                                hzo[(i - k - 1) * 32] = hz[i - k];
+                            }
+                        } else if ((i - 2) % 4 == 0) {
+                            *reinterpret_cast<float4 *>(hxo + i - 2) = make_float4(hx[i - 1], hx[i], hx[i + 1], hx[i + 2]);
+                            *reinterpret_cast<float4 *>(hzo + i - 2) = make_float4(hz[i - 1], hz[i], hz[i + 1], hz[i + 2]);
+                        }
                     }
                 }
+                half_arrive(&s_half[1]);
             }
             // every thread waits on the staging barrier itself: its completion
             // makes the copied shells visible to that thread, so no block
             // barrier is needed here (a timeout is noticed after B2)
             {
-                unsigned &nw = cur ? n_wait1 : n_wait0;
-                if (!wait_stage(P, &s_bar[cur], nw & 1u, &s_quit, ticket)) s_abort = 1;
-                ++nw;
+                if (!wait_stage(P, &s_bar[cur], (fills >> cur) & 1u, &s_quit, ticket)) s_abort = 1;
+                fills ^= 1u << cur;
                 if (R::LOSSY) {
-                    if (!wait_stage(P, &s_bar[2], n_wait2 & 1u, &s_quit, ticket)) s_abort = 1;
-                    ++n_wait2;
+                    if (!wait_stage(P, &s_bar[2], (fills >> 2) & 1u, &s_quit, ticket)) s_abort = 1;
+                    fills ^= 4u;
                 }
             }
 
@@ -941,24 +1000,21 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
                 }
             }
-            if constexpr (R::VX) {
-                float *const qx = XHx + xe_at(w, 0, lane), *const qz = XHz + xe_at(w, 0, lane);
-#pragma unroll
-                for (int i = 1; i < NR; i += 4) {
-                    *reinterpret_cast<float4 *>(qx + i - 1) = make_float4(hx[i], hx[i + 1], hx[i + 2], hx[i + 3]);
-                    *reinterpret_cast<float4 *>(qz + i - 1) = make_float4(hz[i], hz[i + 1], hz[i + 2], hz[i + 3]);
-                }
-            } else {
+            if (!ybox) {  // the y-shell warp's H rows
 #pragma unroll
                 for (int i = 1; i < NR; ++i) {
                     XHx[xe_at(w, i - 1, lane)] = hx[i];
                     XHz[xe_at(w, i - 1, lane)] = hz[i];
                 }
             }
-            bar_compute();  // B2
-            if (s_abort) { abort = true; break; }
+            if (!ybox) half_arrive(&s_half[1]);
+            if (R::LOSSY) half_arrive(&s_half[2]);  // the coefficients are read
+            if (!half_wait(P, &s_half[1], (n_half - 1u) & 1u, &s_abort, ticket)) {  // B2
+                s_abort = 1;
+                abort = true;
+                break;
+            }
             if (tid == 0 && t > iv.s) st_rel_cta(&s_level, (unsigned)t);  // level t-1 is stored
-            if (R::LOSSY && tid == 0) st_rel_cta(&s_steps2, ++nsteps2);
 
             // does this thread own a point source this step?  (16-bit storage:
             // its E rows are rounded after the source is added, not before)
@@ -1081,6 +1137,9 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 }
             }
 
+            // what the warp below waits for first, then this warp's stores (x pairs:
+            // last, the stores into the partner's ring are signalled after B1)
+            if (R::CL == 1) publish_e();
             // the adjoint's recompute: this step's E of the cells of the
             // capture box (tiles that meet it only)
             if (R::CAP && colin && bx < P.cap_hi[0] && bx + TX > P.cap_lo[0] && by < P.cap_hi[1] &&
@@ -1131,6 +1190,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     (unsigned)py < (unsigned)P.ny)
                     FACE_STORE(XFk + ((long long)px * P.ny + py) * BZ, P.fxs);
             }
+            if (R::CL == 2) publish_e();
             if (R::CL == 2 && msg) sig_slot = slot;
         }
         if (abort) break;
@@ -1148,7 +1208,11 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
             }
         }
-        bar_compute();
+        half_arrive(&s_half[1]);  // every store of the tile is done
+        if (!half_wait(P, &s_half[1], (n_half - 1u) & 1u, &s_abort, ticket)) {
+            s_abort = 1;
+            break;
+        }
         if (tid == 0) st_rel_cta(&s_level, (unsigned)iv.e + 1u);
         } while (false);
         msg_base += nmsg;
