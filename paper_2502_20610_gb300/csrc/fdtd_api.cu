@@ -526,18 +526,34 @@ cudaError_t coop_steps(fdtd_sim *h, int n)
     return e;
 }
 
-// Does a systolic call of n steps run on the naive kernels instead?  A
-// systolic launch of few steps pays for filling and draining its pipeline of
-// tiles: measured (FP32, us, systolic / naive) for one step 101 / 15 at 64^3,
-// 168 / 22 at 112^3, 253 / 64 at 160^3, 558 / 232 at 256^3, 1562 / 742 at
-// 384^3; for two steps 109 / 29, 180 / 43, 277 / 127, 645 / 463, 2030 / 1482;
-// for three steps 384^3 is about equal (2374 / 2223) and 256^3 near it.  Not
-// under a test hook, while capturing or in cluster pairs, which are the
-// systolic kernel's own.
+// Does a systolic call of n steps run on the cooperative streaming kernel
+// instead (the same bits)?  A systolic launch first fills its pipeline of
+// tiles: some 7.6 us for each tile along the three axes, or 0.12 us for each
+// tile where they outnumber the SMs, and then takes about 4.7 us and 4.2 ns a
+// thousand cells a step; the streaming kernel takes 6 us (its barriers) and,
+// a thousand cells, 7.2 ns while the state is in L2, 11 to twice L2 and 13.2
+// beyond (16-bit storage: 7.8, 10, 11).  Measured crossings (steps; FP32, then
+// FP16 where it differs): 16^3 10, 32^3 22, 64^3 32, 112^3 25, 160^3 7 / 20,
+// 256^3 3 / 5, 384^3 3, 40 x 40 x 300 64, 40 x 200 x 300 20; the estimate has to
+// be 10 % ahead, which puts the lines at 11, 22, 29, 21, 6 / 12, 2, 2, 57 and 16.
+// A handle whose tile was chosen, or whose launches are kept short, gets that
+// for all but one or two steps (measured ahead everywhere: 64^3 109 -> 17 us,
+// 384^3 2030 -> 1530 for two).  Not under a test hook, while capturing or in
+// cluster pairs, which are the systolic kernel's own.
 bool short_call(const fdtd_sim *h, int64_t n)
 {
     if (h->cap || h->dbg_kind != FDTD_DEBUG_NONE || h->dbg_order != 0 || h->L.cl != 1) return false;
-    return n <= 2;
+    if (n <= 2) return true;
+    if (h->c.tile[0] != 0 || n > h->L.steps_per_launch) return false;
+    const double nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, cells = nx * ny * nz, k = cells * 1e-6;
+    const double state = cells * (6.0 * h->L.eb + 4.0);
+    const bool wide = h->L.eb == 4;
+    const double per = state <= 96e6 ? (wide ? 7.2 : 7.8) : state <= 256e6 ? (wide ? 11.0 : 10.0) : (wide ? 13.2 : 11.0);
+    const double hops = nx / h->L.tx + ny / h->L.ty + nz / h->L.tz;
+    const double tiles = std::ceil(nx / h->L.tx) * std::ceil(ny / h->L.ty) * std::ceil(nz / h->L.tz);
+    const double stream = (double)n * (6.0 + k * per);
+    const double systolic = std::max(7.6 * hops, 0.12 * tiles) + (double)n * (4.7 + 4.2 * k);
+    return stream < 0.9 * systolic;
 }
 
 fdtd_status upload_tiles(fdtd_sim *h, int order, unsigned seed)

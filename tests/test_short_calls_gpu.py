@@ -1,11 +1,11 @@
 """Short calls and the naive schedule's cooperative launch, bit for bit against
 the systolic kernel.
 
-A call of one or two steps on a systolic handle, and any call on a naive
-handle whose state is at most twice L2, run in one cooperative launch with
-grid barriers.  Every storage, lossy cells, sources, extents below a warp,
-and columns that do not divide into the launch's warps must give the bits of
-one long systolic launch (at least three steps a call).
+Few steps on a systolic handle (one or two where its tile was chosen), and any
+call on a naive handle whose state is at most twice L2, run in one
+cooperative launch with grid barriers.  Every storage, lossy cells, sources,
+extents below a warp, and columns that do not divide into the launch's warps
+must give the bits of one systolic launch.
 """
 import numpy as np
 import pytest
@@ -37,12 +37,14 @@ def run(shape, calls, scheme, sources, **kw):
 def test_bits_of_the_systolic_kernel(cuda_device, shape, kw):
     nz, ny, nx = shape
     src = [(2, nx // 2, ny // 2, nz // 2, wl.sine_source(64, DT)), (0, nx - 1, 0, nz - 1, wl.sine_source(5, DT, 7.0))]
-    long, at, n = run(shape, [9], "systolic", src, **kw)
+    long, at, n = run(shape, [9], "systolic", src, tile="31x15x12", **kw)
     assert (at, n) == (9, 1)
     short, at, n = run(shape, [1, 2, 2, 1, 1, 2], "systolic", src, **kw)
     assert (at, n) == (9, 6)
     assert torch.equal(long, short)
-    mixed, _, _ = run(shape, [1, 4, 2, 2], "systolic", src, **kw)
+    mixed, _, _ = run(shape, [1, 4, 2, 2], "systolic", src, tile="31x15x12", **kw)
+    default, _, n = run(shape, [9], "systolic", src, **kw)
+    assert n == 1 and torch.equal(long, default)
     assert torch.equal(long, mixed)
     naive, at, _ = run(shape, [5, 1, 3], "naive", src, **kw)
     assert at == 9 and torch.equal(long, naive)
@@ -51,7 +53,7 @@ def test_bits_of_the_systolic_kernel(cuda_device, shape, kw):
 def test_backward_sweep_of_a_state_beyond_l2(cuda_device):
     """Over 96 MB of state the E half-step sweeps the grid backwards."""
     shape = (150, 161, 170)
-    long, _, _ = run(shape, [4], "systolic", [])
+    long, _, _ = run(shape, [4], "systolic", [], tile="31x15x12")
     naive, _, launches = run(shape, [4], "naive", [])
     assert launches == 1 and torch.equal(long, naive)
 
@@ -79,7 +81,7 @@ def test_steps_replay_from_a_captured_graph(cuda_device):
 
 
 def run_plain(shape, f0, n):
-    sim = fdtd.Sim(shape, 2.0, DT, scheme="systolic")
+    sim = fdtd.Sim(shape, 2.0, DT, scheme="systolic", tile="31x15x12")
     sim.write_fields(f0)
     sim.step(n)
     out = sim.read_fields().view(torch.int32)
