@@ -1226,7 +1226,11 @@ fdtd_status fdtd_adjoint_gradient(fdtd_handle h, const fdtd_overlap_objective *o
     // step unless the register kernel can capture the box) use the naive
     // kernel pair, which the systolic schedule reproduces bit for bit
     const bool reg_kernel = h->c.scheme == FDTD_SCHEME_SYSTOLIC && h->L.variant >= 2;
-    auto one_step = [&]() -> cudaError_t { return naive_step(h); };
+    auto one_step = [&]() -> cudaError_t {
+        // one cooperative launch, as for a naive handle, unless the state is far
+        // beyond L2 (200 x 200 x 100: 57 -> 51 us a step)
+        return (double)h->g.nx * h->g.ny * h->g.nz * 28.0 <= 256e6 ? coop_steps(h, 1) : naive_step(h);
+    };
     // m steps of h, the box's E after step r (r = 1..m) into plane p0 + r of
     // buf: captured by the register kernel, or copied after single steps
     auto run_capture = [&](long long m, float *buf, long long p0) -> fdtd_status {
