@@ -43,11 +43,11 @@
 // only by a tile downwind of every reader of the value there (the CPU model
 // checks both).
 //
-// Bookkeeping: a warp of its own polls the upwind tiles, fetches the next
-// step's shells as soon as their staging buffer is free, and publishes the
-// tile's levels.  While the warp whose y slot is outside the box did this
-// between its refills, its chain of stores, release, poll and copies (3100 of
-// 9500 cycles) was as long as the other warps' half-steps and stores.
+// Bookkeeping: two warps of their own.  One polls the upwind tiles and fetches
+// the next step's shells as soon as their staging buffer is free, the other
+// publishes the tile's levels.  While the warp whose y slot is outside the box
+// did this between its refills, its chain of stores, release, poll and copies
+// (3100 of 9500 cycles) was as long as the other warps' half-steps and stores.
 //
 // Code size: the step is some 3500 instructions long, and what lies between
 // is fetched with it.  Taking the cold paths out of the loop (row-by-row
@@ -56,11 +56,16 @@
 // 172.8 -> 193 GCUPS at 256^3 and 180 -> 196 at 512^3 before the bookkeeping
 // warp, which gave 201 and 216 (FP16 at 256^3: 163 -> 188).
 //
-// Top faces: the z face goes to the field arrays at the end of each step;
-// the y face goes to the y-face buffer one step late, from the warp whose y
-// slot leaves, while it sits out the H half-step; the x face goes to the
-// x-face buffer at the end of each step.  A tile therefore publishes level
-// t-1 after the second barrier of step t.
+// Top faces: the z face goes to the field arrays and the y and x faces to
+// their buffers at the end of each step, each warp then arriving at that step's
+// barrier (of four in turn), which the publishing warp watches: a level is
+// published as soon as its last face is stored.  A cell's path through time
+// crosses into the next tile every 1 / (1/31 + 1/15 + 1/12) = 5.5 steps, so on
+// domains that do not fill the chip this delay is a part of every step: with
+// the y face stored a step late and a level published after B2 of the step
+// after, 64^3 x 200 steps took 1082 us, now 982 (128^3 FP16 146 -> 155 GCUPS,
+// 200 x 200 x 100 163 -> 169, 256^3 unchanged at 213).  An arrival costs least:
+// a release store a warp instead took 1.5 %, with a look at the abort word 3 %.
 //
 // Two barriers per step: B1, after the E rows are exchanged for the H
 // half-step, and B2, after the H rows are exchanged for the E half-step.  A
@@ -192,8 +197,8 @@ struct RegTile {
 
 __device__ __forceinline__ float shfl_from(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-// Named barrier of the compute warps with the bookkeeping warp at a tile's start.
-__device__ __forceinline__ void bar_tile() { asm volatile("bar.sync 2, 544;" ::: "memory"); }
+// Named barrier of the compute warps with the two bookkeeping warps at a tile's start.
+__device__ __forceinline__ void bar_tile() { asm volatile("bar.sync 2, 576;" ::: "memory"); }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -360,7 +365,7 @@ __device__ __noinline__ void timed_out(int *ctrl, int ticket, int what)
 }
 
 // Release / acquire at CTA scope on a shared word: how the compute warps and
-// the bookkeeping warp tell each other where they are.
+// the bookkeeping warps tell each other where they are.
 __device__ __forceinline__ void st_rel_cta(unsigned *p, unsigned v)
 {
     asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
@@ -373,7 +378,7 @@ __device__ __forceinline__ unsigned ld_acq_cta(const unsigned *p)
 }
 
 // Bounded wait for phase `parity` of a staging barrier; gives up at once when
-// the bookkeeping warp has (*quit).  False: the error word is set.
+// a bookkeeping warp has (*quit).  False: the error word is set.
 __device__ bool wait_stage(const SysLaunch &P, unsigned long long *bar, unsigned parity, const unsigned *quit, int ticket)
 {
     unsigned long long t0 = 0;
@@ -453,10 +458,12 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     __shared__ alignas(8) unsigned long long s_rxf[R::NSLOT], s_rxe[R::NSLOT];
     __shared__ alignas(8) unsigned long long s_bar[3];  // staging barriers, one per buffer (lossy: and the
                                                         // coefficients'): one phase per fill
-    // the bookkeeping warp's view of the compute warps: B1 barriers passed over
-    // the CTA's life, and the current tile's last finished level (its progress
-    // value less the epoch); s_quit: it has given up waiting
-    __shared__ unsigned s_steps, s_level, s_quit;
+    // the bookkeeping warps' view of the compute warps: B1 barriers passed over
+    // the CTA's life, and a barrier each for four steps in turn, which the compute
+    // warps arrive at once a step's faces are stored.  s_told: the steps that the
+    // publishing warp has seen there; s_quit: a bookkeeping warp has given up
+    __shared__ unsigned s_steps, s_told, s_quit;
+    __shared__ alignas(8) unsigned long long s_fin[4];
     __shared__ alignas(8) unsigned long long s_half[3];  // B1 and B2 (lossy: and a step's coefficients read)
     __shared__ int s_pfail;  // ... before the tile's first step
     __shared__ unsigned s_seen[3];
@@ -505,8 +512,10 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     } while (0)
 
     constexpr int CR = R::CR, CP = R::CP, CRM = R::CRM;
+    if (tid < 4)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_fin[tid])), "r"(R::RY) : "memory");
     if (tid == 0) {
-        s_steps = s_quit = 0u;
+        s_steps = s_told = s_quit = 0u;
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[0])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[1])) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bar[2])) : "memory");
@@ -520,8 +529,8 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_rxe[k])) : "memory");
             }
         }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (tid < 4) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
     // x pairs: rank 0 holds the upwind tile (I even), rank 1 the downwind one;
     // every CTA of the cluster must be running before distributed shared
@@ -548,19 +557,21 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     // lane has just read
     int sig_slot = -1;
     if (w >= R::RY) {
-        // ------------------------------------------------ bookkeeping warp
+        // ----------------------------------------------- bookkeeping warps
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R::BREG));
-        if (w > R::RY) {
+        if (w > R::RY + 1) {
             // (x pairs: cluster barriers count every thread that has not left)
             return;
         }
-        // Polls the upwind tiles' progress and fetches a step's lower shells
-        // (six bulk tensor copies; x start rounded down to 16 bytes, zero fill
-        // off the domain) as soon as their staging buffer is free, and publishes
-        // the tile's own levels: the release of a flag waits for the CTA's stores
-        // to land (1000 to 1900 cycles), a poll and the copies take as long
-        // again, and none of it holds up a compute warp here.
+        // The first polls the upwind tiles' progress and fetches a step's lower
+        // shells (six bulk tensor copies; x start rounded down to 16 bytes, zero
+        // fill off the domain) as soon as their staging buffer is free.  The
+        // second publishes the tile's own levels: the release of a flag waits for
+        // the CTA's stores to land (1000 to 1900 cycles), and a poll and the
+        // copies take as long again.
+        const bool publisher = w == R::RY + 1;
         unsigned steps0 = 0, n0 = 0, n1 = 0, n2 = 0;  // s_steps at the tile's start; fills of each buffer
+        unsigned n_fin = 0;  // steps before the tile's (fetch), steps seen finished (publisher)
         auto fetch_coefs = [&](int t, int Ax, int Ay, int Az, char *sb, unsigned long long *bar) {
             const int bx = Ax - t, by = Ay - t, bz = Az - t, x0c = (bx - 1) & ~(R::XAC - 1);
             tma_box(sb, &P.tm[0][1], x0c, by - 1, bz - 1, bar);
@@ -580,20 +591,49 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const Interval iv = tile_interval<TX, TY, TZ>(P, I, J, K);
             Upwind U;
             upwind_of<TX, TY, TZ>(P, I, J, K, U);
+            if (publisher) {
+                bar_tile();
+                if (s_pfail) continue;
+                // a tile that starts late (or, start > end, enters the domain only
+                // after this launch) carries its upwind tiles' guarantee on
+                if (iv.s > 0 && lane == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.s);
+                if (iv.s > iv.e) continue;
+                unsigned long long t_own = 0;
+                for (int t = iv.s; t <= iv.e;) {
+                    unsigned fin;
+                    asm volatile("{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;"
+                                 " selp.u32 %0, 1, 0, p; }"
+                                 : "=r"(fin) : "r"(smem_u32(&s_fin[n_fin & 3u])), "r"((n_fin >> 2) & 1u) : "memory");
+                    if (__all_sync(0xffffffffu, fin)) {
+                        ++t;
+                        ++n_fin;
+                        if (lane == 0) {
+                            *(volatile unsigned *)&s_told = n_fin;
+                            publish(P, tile, ticket, P.epoch + (unsigned)t);
+                        }
+                        t_own = 0;
+                        continue;
+                    }
+                    __nanosleep(32);
+                    bool late = lane == 0 && past(t_own, 8 * (unsigned long long)P.timeout_ns);
+                    if (late) {
+                        timed_out(P.ctrl, ticket, -3);
+                        st_rel_cta(&s_quit, 1u);
+                    }
+                    late |= *(volatile int *)&s_abort != 0;
+                    if (__any_sync(0xffffffffu, late)) break;
+                }
+                continue;
+            }
             if (lane < 3) s_seen[lane] = 0u;
             __syncwarp();
             bool ok = iv.s == 0 || wait_level(P, U, s_seen, iv.s - 1, ticket);
             if (lane == 0) s_pfail = !ok;
             bar_tile();
-            if (!ok) continue;
-            // a tile that starts late (or, start > end, enters the domain only
-            // after this launch) carries its upwind tiles' guarantee on
-            if (iv.s > 0 && lane == 0) publish(P, tile, ticket, P.epoch + (unsigned)iv.s);
-            if (iv.s > iv.e) continue;
+            if (!ok || iv.s > iv.e) continue;
             int t = iv.s, tc = iv.s;                 // the next step to fetch (tc: lossy, its coefficients)
-            unsigned pub = 0;                        // the last level published
             unsigned long long t_up = 0, t_own = 0;  // waiting for the upwind tiles, for the compute warps
-            while (ok && (t <= iv.e || (R::LOSSY && tc <= iv.e) || pub != (unsigned)iv.e + 1u)) {
+            while (ok && (t <= iv.e || (R::LOSSY && tc <= iv.e))) {
                 bool idle = true;
                 if (R::LOSSY && tc <= iv.e) {  // the coefficients' buffer: free once step tc - 1 has read it
                     unsigned read = 1;
@@ -613,9 +653,12 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
                 }
                 // step t's buffer: free at the tile's start, else once B1 of step
-                // t - 1 has been passed
+                // t - 1 has been passed.  (And no step may finish whose barrier has
+                // one that the publishing warp has not seen: four steps before it)
                 const unsigned passed = __shfl_sync(0xffffffffu, ld_acq_cta(&s_steps), 0);
-                if (t <= iv.e && (t < iv.s + 2 || (int)(passed - (steps0 + (unsigned)(t - iv.s))) >= 0)) {
+                const unsigned told = __shfl_sync(0xffffffffu, *(volatile unsigned *)&s_told, 0);
+                if (t <= iv.e && (t < iv.s + 2 || ((int)(passed - (steps0 + (unsigned)(t - iv.s))) >= 0 &&
+                                                   (int)(told + 3u - (n_fin + (unsigned)(t - iv.s))) >= 0))) {
                     idle = false;
                     if (level_ready(P, U, s_seen, t)) {
                         __syncwarp();  // orders lanes 1, 2's acquires before lane 0's copies
@@ -638,20 +681,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                         if (t & 1) ++n1;
                         else ++n0;
                         ++t;
-                        t_up = 0;
+                        t_up = t_own = 0;
                     } else {
                         bool late = lane == 0 && past(t_up, (unsigned long long)P.timeout_ns);
                         if (late) timed_out(P.ctrl, ticket, (int)(P.epoch + (unsigned)t + 1u));
                         late |= ld_volatile(P.ctrl + 1) != DEV_OK;
                         ok = !__any_sync(0xffffffffu, late);
                     }
-                }
-                const unsigned lv = __shfl_sync(0xffffffffu, ld_acq_cta(&s_level), 0);
-                if (lv != pub) {
-                    if (lane == 0) publish(P, tile, ticket, P.epoch + lv);
-                    pub = lv;
-                    t_own = 0;
-                    idle = false;
                 }
                 if (idle) {
                     __nanosleep(32);
@@ -662,11 +698,12 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 }
             }
             if (!ok && lane == 0) st_rel_cta(&s_quit, 1u);
-            steps0 += (unsigned)(iv.e - iv.s + 2);  // (one pass more than steps)
+            n_fin += (unsigned)(iv.e - iv.s + 1);
+            steps0 += (unsigned)(iv.e - iv.s + 1) + (R::CL == 2 ? 1u : 0u);  // (x pairs: one pass more than steps)
         }
         // no copy may still be writing when the CTA's shared memory goes (after an
         // abort some were never waited for)
-        if (lane == 0) {
+        if (lane == 0 && !publisher) {
             if (n0) wait_stage(P, &s_bar[0], (n0 - 1) & 1u, nullptr, -1);
             if (n1) wait_stage(P, &s_bar[1], (n1 - 1) & 1u, nullptr, -1);
             if (n2) wait_stage(P, &s_bar[2], (n2 - 1) & 1u, nullptr, -1);
@@ -681,7 +718,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
     // passes over the step loop (phases of B1 and of B2), and the parities of the
     // next fill of each staging buffer (bits 0, 1; lossy: 2, the coefficients):
     // every thread waits for every phase and keeps the same counts
-    unsigned n_half = 0, fills = 0;
+    unsigned n_half = 0, fills = 0, n_fin = 0;
     // the coefficient ring's row of physical z = bz - 1 + i, with zr the row of
     // bz - 1 (lossless: any number congruent to it)
     auto ring = [](int zr, int i) {
@@ -711,14 +748,12 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 st_remote_u32(mapa(smem_u32(&s_ticket), 1u), (unsigned)tk);
                 st_remote_u32(mapa(smem_u32(&s_abort), 1u), (unsigned)ab);
             }
-            if (tid == 0) s_level = 0u;
             cluster_sync_all();
         } else {
             bar_tile();
             if (tid == 0) {
                 s_ticket = atomicAdd(P.ctrl, 1);
                 s_abort = ld_volatile(P.ctrl + 1) != DEV_OK;
-                s_level = 0u;
             }
             bar_tile();
         }
@@ -827,7 +862,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
         };
         publish_e();
         for (int t = iv.s;; ++t, zl = R::LOSSY ? (zl == 0 ? CR - 1 : zl - 1) : 0) {
-            // (one pass more than steps: the last step's top y face)
+            // (x pairs: one pass more than steps, for the last slot's signal)
             const int bx = Ax - t, by = Ay - t, bz = Az - t;  // box low corner at step t
             const int zr = R::LOSSY ? zl : bz - 1;
             const int cur = t & 1;
@@ -844,7 +879,6 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const bool xbox = dx < TX, ybox = dy < TY;
             const bool colin = xbox && ybox && (unsigned)px < (unsigned)P.nx && (unsigned)py < (unsigned)P.ny;
             const int ey_w = (by - 1) & (R::RY - 1);  // warp holding the y shell this step
-            const int yf_w = (by + TY) & (R::RY - 1);  // warp holding the top y row of step t-1
             const long long col = px + (long long)P.pitch * py;
             // the box touches a low wall, whose tangential E is left alone.  (No
             // other masks: cells outside the domain have dt/eps (and c_a) 0, as the
@@ -878,17 +912,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     sig_slot = -1;
                 }
             }
-            // B. the warp whose y slot leaves the tile this step is idle during
-            //    the H half-step: it stores last step's top y face, which its
-            //    registers still hold, into the y-face buffer
-            if (w == yf_w && t > iv.s) {
-                const int pbx = bx + 1, pby = by + 1;  // box corner of step t-1
-                const int pdx = (lane - pbx) & 31;
-                const int qx = pbx + pdx, qy = pby + TY - 1;
-                if (pdx < TX && (unsigned)qx < (unsigned)P.nx && (unsigned)qy < (unsigned)P.ny)
-                    FACE_STORE(YFk + ((long long)qy * P.nx + qx) * BZ, P.fys);
-            }
-            if (t > iv.e) break;
+            if (R::CL == 2 && t > iv.e) break;
             // x start of the staged z shell (rounded down to 16 bytes)
             const int x0 = (bx - 1) & ~(XA - 1), x0c = (bx - 1) & ~(R::XAC - 1);
 
@@ -1027,7 +1051,6 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 abort = true;
                 break;
             }
-            if (tid == 0 && t > iv.s) st_rel_cta(&s_level, (unsigned)t);  // level t-1 is stored
 
             // does this thread own a point source this step?  (16-bit storage:
             // its E rows are rounded after the source is added, not before)
@@ -1153,7 +1176,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 
             // what the warp below waits for first, then this warp's stores (x pairs:
             // last, the stores into the partner's ring are signalled after B1)
-            if (R::CL == 1) publish_e();
+            if (R::CL == 1 && t < iv.e) publish_e();
             // the adjoint's recompute: this step's E of the cells of the
             // capture box (tiles that meet it only)
             if (R::CAP && colin && bx < P.cap_hi[0] && bx + TX > P.cap_lo[0] && by < P.cap_hi[1] &&
@@ -1173,9 +1196,16 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
                 }
             }
-            // G. the top faces (the top y face is stored next step by the warp
-            // holding it; the launch's last step is stored whole, below)
-            if (colin && t < P.T - 1 && (unsigned)(bz + NR - 2) < (unsigned)P.nz) {  // top z face
+            // G. the top faces (of the launch's last step too, which is stored whole
+            // below: the downwind tiles need not wait for that).  The top y face: its
+            // warp, which is idle in the next H half-step, has the most to store.
+            // Last, or with 16-bit storage first (FP32 256^3 213.4 and 211.8 GCUPS,
+            // FP16 201.3 and 203.1)
+            auto y_face = [&]() {
+                if (colin && dy == TY - 1) FACE_STORE(YFk + ((long long)py * P.nx + px) * BZ, P.fys);
+            };
+            if (S::narrow) y_face();
+            if (colin && (unsigned)(bz + NR - 2) < (unsigned)P.nz) {  // top z face
                 const long long g = col + sxy * (bz + NR - 2);
                 STORE6(g, NR - 1);
             }
@@ -1204,10 +1234,15 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     (unsigned)py < (unsigned)P.ny)
                     FACE_STORE(XFk + ((long long)px * P.ny + py) * BZ, P.fxs);
             }
+            if (!S::narrow) y_face();
+            // this warp's faces of level t are stored
+            half_arrive(&s_fin[n_fin & 3u]);
+            ++n_fin;
             if (R::CL == 2) publish_e();
             if (R::CL == 2 && msg) sig_slot = slot;
+            if (R::CL == 1 && t == iv.e) break;
         }
-        if (abort) break;
+        if (abort || *(volatile int *)&s_abort != 0) break;
         if (iv.e == P.T - 1) {  // the launch's last step: the whole box
             const int bx = Ax - iv.e, by = Ay - iv.e, bz = Az - iv.e;
             const int dx = (lane - bx) & 31, dy = (w - by) & (R::RY - 1);
@@ -1222,12 +1257,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     }
             }
         }
-        half_arrive(&s_half[1]);  // every store of the tile is done
-        if (!half_wait(P, &s_half[1], (n_half - 1u) & 1u, &s_abort, ticket)) {
-            s_abort = 1;
-            break;
+        if constexpr (R::CL == 2) {  // B2's phase of the pass more
+            half_arrive(&s_half[1]);
+            if (!half_wait(P, &s_half[1], (n_half - 1u) & 1u, &s_abort, ticket)) {
+                s_abort = 1;
+                break;
+            }
         }
-        if (tid == 0) st_rel_cta(&s_level, (unsigned)iv.e + 1u);
         } while (false);
         msg_base += nmsg;
         sig_slot = -1;
