@@ -877,6 +877,13 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const int dx = (lane - bx) & 31, dy = (w - by) & (R::RY - 1);
             const int px = bx + dx, py = by + dy;
             const bool xbox = dx < TX, ybox = dy < TY;
+            // a row of cells outside the domain in y stays as it is (E = 0, and its H is
+            // read by nobody): its warp skips the half-steps until it becomes the
+            // y shell, and leaves its share of the issue slots to the others (FP32
+            // 256^3 213.2 -> 216.9 GCUPS, 512^3 228.3 -> 230.5, FP16 256^3 203.0 ->
+            // 205.7, 128^3 155.3 -> 158.3).  The same for groups of four z rows
+            // cost more, in branches and spills, than it saved (209.0, FP16 173.2).
+            const bool act = ybox && (unsigned)py < (unsigned)P.ny;
             const bool colin = xbox && ybox && (unsigned)px < (unsigned)P.nx && (unsigned)py < (unsigned)P.ny;
             const int ey_w = (by - 1) & (R::RY - 1);  // warp holding the y shell this step
             const long long col = px + (long long)P.pitch * py;
@@ -917,7 +924,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             const int x0 = (bx - 1) & ~(XA - 1), x0c = (bx - 1) & ~(R::XAC - 1);
 
             // C. H half-step, top-down in place: H[i] <- H[i-1] - dt curl_f(E[i-1], E[i], ...)
-            if (ybox) {
+            if (act) {
                 const int wn = (w + 1) & (R::RY - 1);
                 const int src = (lane + 1) & 31;
                 // rows in pairs (i, i-1), both computed from the old values
@@ -1009,7 +1016,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     put_ce(ring(zr, i), lane, YSC[i * SWC + xlc]);
                     if (R::LOSSY) CAs[(w * CRM + ring(zr, i)) * CP + lane] = YSA[i * SWC + xlc];
                 }
-            } else if (!ybox) {  // the previous top y row (two outside slots): kept
+            } else if (!act) {  // outside the domain, or the previous top y row (two outside slots): kept
             } else {  // every lane's row -1 takes the lower z shell's H and coefficient
                 const int o = (dy + 1) * SW + (xw - x0), oc = (dy + 1) * SWC + (xw - x0c);
                 hx[0] = S::dec(ZST[3 * R::ZB + o], SC(3));
@@ -1044,7 +1051,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                     XHz[xe_at(w, i - 1, lane)] = hz[i];
                 }
             }
-            if (!ybox) half_arrive(&s_half[1]);
+            if (!act) half_arrive(&s_half[1]);
             if (R::LOSSY) half_arrive(&s_half[2]);  // the coefficients are read
             if (!half_wait(P, &s_half[1], (n_half - 1u) & 1u, &s_abort, ticket)) {  // B2
                 s_abort = 1;
@@ -1065,7 +1072,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
                 srcthr = __any_sync(0xffffffffu, srcthr);  // its whole warp rounds late (shuffles in the E half-step)
             }
 
-            if (ybox) {
+            if (act) {
                 // F. E half-step, top-down in place: E[i] <- E[i-1] + ce curl_b(H[i], H[i-1], ...)
                 const int wm = (w - 1) & (R::RY - 1);
                 const int src = (lane - 1) & 31;
