@@ -1062,6 +1062,31 @@ fdtd_status fdtd_learned_record_scratch_size(fdtd_handle h, int32_t per_step, si
     return FDTD_OK;
 }
 
+namespace {
+
+// One axis of the recorder's random cells: numbers modulo a box width w, and
+// whether such a coordinate lies further than t from both faces.
+struct Drawn {
+    unsigned w, t, in;
+    unsigned long long m;
+    Drawn(int width, int thickness)
+        : w((unsigned)width), t((unsigned)thickness), in(width - 2ll * thickness > 0 ? (unsigned)(width - 2ll * thickness) : 0u),
+          m(w > 1 ? (unsigned long long)(((unsigned __int128)1 << 64) / w) : 0ull)
+    {
+    }
+    unsigned mod(unsigned long long v) const
+    {
+        unsigned long long r = v - (unsigned long long)(((unsigned __int128)v * m) >> 64) * w;
+        if (w == 1) return 0u;
+        r -= r >= w ? w : 0u;
+        r -= r >= w ? w : 0u;
+        return (unsigned)r;
+    }
+    unsigned inner(unsigned c) const { return c - t < in; }
+};
+
+} // namespace
+
 fdtd_status fdtd_learned_record(fdtd_handle h, const int32_t lo[3], const int32_t hi[3], int32_t thickness,
                                 int32_t n_steps, int32_t per_step, uint64_t seed, float *d_x, float *d_y,
                                 void *d_scratch, size_t scratch_bytes)
@@ -1085,11 +1110,13 @@ fdtd_status fdtd_learned_record(fdtd_handle h, const int32_t lo[3], const int32_
     const int ilo[3] = {lo[0], lo[1], lo[2]}, ihi[3] = {hi[0], hi[1], hi[2]};
     // layer region of the box: cells within `thickness` of one of its faces
     std::mt19937_64 rng(seed);
-    auto in_layer = [&](int x, int y, int z) {
-        const int d = std::min(std::min(std::min(x - lo[0], hi[0] - 1 - x), std::min(y - lo[1], hi[1] - 1 - y)),
-                               std::min(z - lo[2], hi[2] - 1 - z));
-        return d < thickness;
-    };
+    // A cell's draw is three numbers modulo the box's widths, taken again until
+    // the cell is in the layer.  The draws of a step (7000 of them for 1000
+    // cells of a 48^3 box) are what a short step waits for, so: remainders by a
+    // multiplication with floor(2^64 / width) (its quotient is at most two too
+    // small) instead of 64-bit divisions, and no branch on the layer, which the
+    // processor would guess wrong every other time.
+    const Drawn axis[3] = {Drawn(hi[0] - lo[0], thickness), Drawn(hi[1] - lo[1], thickness), Drawn(hi[2] - lo[2], thickness)};
     // the box of S^{n-1} and S^n, taken in turn: a step copies the new box
     // over the oldest one (the whole state, copied twice a step, was 6x
     // the traffic of the box at its usual size)
@@ -1120,17 +1147,14 @@ fdtd_status fdtd_learned_record(fdtd_handle h, const int32_t lo[3], const int32_
         if (ring.copied[r]) CK(cudaEventSynchronize(ring.copied[r]));
         else CK(cudaEventCreateWithFlags(&ring.copied[r], cudaEventDisableTiming));
         std::vector<int> &pick = ring.pick[r];
-        pick.resize(per);
-        for (int q = 0; q < per_step; ++q) {
-            int x, y, z;
-            do {
-                x = lo[0] + (int)(rng() % (unsigned long long)(hi[0] - lo[0]));
-                y = lo[1] + (int)(rng() % (unsigned long long)(hi[1] - lo[1]));
-                z = lo[2] + (int)(rng() % (unsigned long long)(hi[2] - lo[2]));
-            } while (!in_layer(x, y, z));
-            pick[3 * (size_t)q] = x;
-            pick[3 * (size_t)q + 1] = y;
-            pick[3 * (size_t)q + 2] = z;
+        pick.resize(per + 3);  // (a rejected cell after the last one)
+        for (int q = 0; q < per_step;) {
+            int *const c = pick.data() + 3 * (size_t)q;
+            const unsigned x = axis[0].mod(rng()), y = axis[1].mod(rng()), z = axis[2].mod(rng());
+            c[0] = lo[0] + (int)x;
+            c[1] = lo[1] + (int)y;
+            c[2] = lo[2] + (int)z;
+            q += 1 - (int)(axis[0].inner(x) & axis[1].inner(y) & axis[2].inner(z));
         }
         CK(cudaMemcpyAsync(cells, pick.data(), sizeof(int) * per, cudaMemcpyHostToDevice, h->stream));
         CK(cudaEventRecord(ring.copied[r], h->stream));
