@@ -79,7 +79,8 @@ typedef struct {
     int32_t storage;          /* FDTD_STORAGE_*; the systolic 31x15x15 and 31x7x15 tiles take F32 only */
     float field_scale[6];     /* 16-bit storage: s_c, a power of two in [2^-100, 2^100], 0 = 1;
                                  unused for F32.  Equal scales are fastest. */
-    int32_t tile[3];          /* systolic subdomain (updated cells per axis); 0 = default */
+    int32_t tile[3];          /* systolic subdomain (updated cells per axis); 0 = 31x15x12,
+                                 or 31x15x8 on domains too small to give every SM a tile */
     int32_t cluster[3];       /* systolic thread-block cluster shape in tiles; 0 = 1.
                                  (1,1,1): every tile in its own CTA, all faces between
                                  tiles through global memory (Sec. 3, Sec. 4).

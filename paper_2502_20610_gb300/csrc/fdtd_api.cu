@@ -52,12 +52,31 @@ bool conducts(const fdtd_boundary &b)
     return b.kind == FDTD_BOUNDARY_GRADED_ABSORBER || (b.kind == FDTD_BOUNDARY_LEARNED && b.sigma_max > 0.0);
 }
 
-constexpr int DEFAULT_VARIANT = 2;  // register-resident 31 x 15 x 12 with TMA shells: fastest measured
+// Tile shape requested in coeffs.tile -> variant, or -1.  (0,0,0) is the
+// register-resident 31 x 15 x 12, which updates most cells a second, or
+// 31 x 15 x 8 where the tiles inside the domain at a time are no more than the
+// SMs (152): every tile then has an SM, and a step takes what one tile's step
+// and its waits for the upwind tiles take, which is less for 8 rows.  Measured,
+// 12 and 8 rows, 400 steps FP32: 16^3 1456 and 1166 us, 64^3 (140 tiles of 8
+// rows at a time) 1860 and 1504, 400 x 24 x 24 (136) 1845 and 1568, 72^3 (186)
+// 1883 and 1566, 80^3 (242) 1913 and 1870, 96^3 (384) 2557 and 2746.  Long
+// columns hand tiles on more often, and the line lies lower: 40 x 40 x 150 (160)
+// 1893 and 1671, 24 x 24 x 270 (153) 1815 and 2038.  Cluster pairs and
+// conducting cells take the 12-row form only, and very long launches keep it
+// (their tile order would be half as long again).
+constexpr int FEW_TILES = 152, FEW_TILES_COLUMN = 100, FEW_TILES_STEPS = 4096;
 
-// Tile shape requested in coeffs.tile (0,0,0 = default) -> variant, or -1.
-int pick_variant(const fdtd_coeffs &c)
+int pick_variant(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &b)
 {
-    if (c.tile[0] == 0 && c.tile[1] == 0 && c.tile[2] == 0) return DEFAULT_VARIANT;
+    if (c.tile[0] == 0 && c.tile[1] == 0 && c.tile[2] == 0) {
+        constexpr int ROWS12 = 2, ROWS8 = 3;
+        const SysShape sh = systolic_shape(ROWS8);
+        const double at_a_time = ((double)g.nx + sh.tx - 1) / sh.tx * (((double)g.ny + sh.ty - 1) / sh.ty) *
+                                 (((double)g.nz + sh.tz - 1) / sh.tz);
+        const bool few = c.cluster[0] != 2 && !conducts(b) && c.steps_per_launch <= FEW_TILES_STEPS &&
+                         at_a_time <= (g.nz > 4 * std::max(g.nx, g.ny) ? FEW_TILES_COLUMN : FEW_TILES);
+        return few ? ROWS8 : ROWS12;
+    }
     for (int v = 0; v < SYS_NSHAPES; ++v) {
         const SysShape sh = systolic_shape(v);
         if (c.tile[0] == sh.tx && c.tile[1] == sh.ty && c.tile[2] == sh.tz) return v;
@@ -112,8 +131,8 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     L.fxs = L.fys = 0;
     L.nzb = L.nzblk = 0;
     L.xface = L.yface = off;
-    if (c.scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(c) >= 2) {
-        const int tz = systolic_shape(pick_variant(c)).tz;
+    if (c.scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(g, c, b) >= 2) {
+        const int tz = systolic_shape(pick_variant(g, c, b)).tz;
         L.nzblk = ceil_div((long long)g.nz + tz - 1, tz);  // columns are stored whole: see the kernel
         L.nzb = L.nzblk * face_block(tz, L.eb);
         const size_t per = align_up((size_t)L.eb * (size_t)g.nx * g.ny * (size_t)L.nzb);
@@ -129,7 +148,7 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     L.steps_per_launch = c.steps_per_launch > 0 ? c.steps_per_launch : DEFAULT_STEPS_PER_LAUNCH;
     L.gx = L.gy = L.gz = 0;
     L.ntiles_max = 0;
-    L.variant = pick_variant(c);
+    L.variant = pick_variant(g, c, b);
     if (L.variant < 0) return false;
     L.cl = c.scheme == FDTD_SCHEME_SYSTOLIC && c.cluster[0] == 2 ? 2 : 1;
     const SysShape sh = systolic_shape(L.variant);
@@ -174,14 +193,14 @@ fdtd_status check_args(const fdtd_grid *g, const fdtd_coeffs *c, const fdtd_boun
     for (int a = 0; a < 3; ++a) {
         if (c->tile[a] < 0 || c->cluster[a] < 0) return FDTD_ERR_INVALID_ARG;
     }
-    if (pick_variant(*c) < 0) return FDTD_ERR_UNSUPPORTED;
+    if (pick_variant(*g, *c, *b) < 0) return FDTD_ERR_UNSUPPORTED;
     // the shared-memory systolic kernels (tiles 31x15x15, 31x7x15) hold FP32 only
-    if (c->scheme == FDTD_SCHEME_SYSTOLIC && c->storage != FDTD_STORAGE_F32 && pick_variant(*c) < 2)
+    if (c->scheme == FDTD_SCHEME_SYSTOLIC && c->storage != FDTD_STORAGE_F32 && pick_variant(*g, *c, *b) < 2)
         return FDTD_ERR_UNSUPPORTED;
     // clusters: one CTA, or x pairs {2,1,1} of the lossless 31 x 15 x 12
     // register tile under the systolic scheme
     if (c->cluster[1] > 1 || c->cluster[2] > 1 || c->cluster[0] > 2) return FDTD_ERR_UNSUPPORTED;
-    if (c->cluster[0] == 2 && (c->scheme != FDTD_SCHEME_SYSTOLIC || pick_variant(*c) != 2 || conducts(*b)))
+    if (c->cluster[0] == 2 && (c->scheme != FDTD_SCHEME_SYSTOLIC || pick_variant(*g, *c, *b) != 2 || conducts(*b)))
         return FDTD_ERR_UNSUPPORTED;
     if (b->kind < FDTD_BOUNDARY_PEC || b->kind > FDTD_BOUNDARY_LEARNED) return FDTD_ERR_INVALID_ARG;
     if (b->kind == FDTD_BOUNDARY_GRADED_ABSORBER && !b->model) {
@@ -191,7 +210,7 @@ fdtd_status check_args(const fdtd_grid *g, const fdtd_coeffs *c, const fdtd_boun
     }
     if (b->kind == FDTD_BOUNDARY_GRADED_ABSORBER) {
         // the register kernel's 31 x 15 x 12 tile is the one built with the lossy update
-        if (c->scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(*c) != 2) return FDTD_ERR_UNSUPPORTED;
+        if (c->scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(*g, *c, *b) != 2) return FDTD_ERR_UNSUPPORTED;
     }
     if (b->kind == FDTD_BOUNDARY_LEARNED) {
         if (b->thickness < 1 || !b->model || !(b->sigma_max >= 0.0) || !std::isfinite(b->sigma_max) ||
@@ -528,14 +547,14 @@ cudaError_t coop_steps(fdtd_sim *h, int n)
 
 // Does a systolic call of n steps run on the cooperative streaming kernel
 // instead (the same bits)?  A systolic launch first fills its pipeline of
-// tiles: some 7.6 us for each tile along the three axes, or 0.12 us for each
-// tile where they outnumber the SMs, and then takes about 4.7 us and 4.2 ns a
-// thousand cells a step; the streaming kernel takes 6 us (its barriers) and,
-// a thousand cells, 7.2 ns while the state is in L2, 11 to twice L2 and 13.2
-// beyond (16-bit storage: 7.8, 10, 11).  Measured crossings (steps; FP32, then
-// FP16 where it differs): 16^3 10, 32^3 22, 64^3 32, 112^3 25, 160^3 7 / 20,
-// 256^3 3 / 5, 384^3 3, 40 x 40 x 300 64, 40 x 200 x 300 20; the estimate has to
-// be 10 % ahead, which puts the lines at 11, 22, 29, 21, 6 / 12, 2, 2, 57 and 16.
+// tiles: some 5.2 us for each tile along the three axes and 0.06 us for each
+// tile there is; it then takes 4.5 us a step (3.5 with 8-row tiles), or 2.2 us
+// and 4.7 ns a thousand cells where that is more.  The streaming kernel takes
+// 6 us (its barriers) and, a thousand cells, 7.2 ns while the state is in L2,
+// 11 to twice L2 and 13.2 beyond (16-bit storage: 7.8, 10, 11).  Measured
+// crossings (steps; FP32, then FP16 where it differs): 16^3 8, 32^3 14, 64^3 17,
+// 112^3 17, 160^3 8 / 14, 256^3 3, 40 x 40 x 300 49; the estimate has to be 10 %
+// ahead, which puts the lines at 5, 11, 15, 13, 5 / 9, 2 and 26.
 // A handle whose tile was chosen, or whose launches are kept short, gets that
 // for all but one or two steps (measured ahead everywhere: 64^3 109 -> 17 us,
 // 384^3 2030 -> 1530 for two).  Not under a test hook, while capturing or in
@@ -552,7 +571,8 @@ bool short_call(const fdtd_sim *h, int64_t n)
     const double hops = nx / h->L.tx + ny / h->L.ty + nz / h->L.tz;
     const double tiles = std::ceil(nx / h->L.tx) * std::ceil(ny / h->L.ty) * std::ceil(nz / h->L.tz);
     const double stream = (double)n * (6.0 + k * per);
-    const double systolic = std::max(7.6 * hops, 0.12 * tiles) + (double)n * (4.7 + 4.2 * k);
+    const double step = std::max(h->L.tz < 12 ? 3.5 : 4.5, 2.2 + 4.7 * k);
+    const double systolic = 5.2 * hops + 0.06 * tiles + (double)n * step;
     return stream < 0.9 * systolic;
 }
 

@@ -891,8 +891,7 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
             // other masks: cells outside the domain have dt/eps (and c_a) 0, as the
             // coefficient shells are zero-filled there, so their E stays 0; their H
             // is only read by such cells and by that tangential E; and the x-shell
-            // lane and the y-shell warp compute values that their refills
-            // overwrite.)
+            // lane computes values that its refill overwrites.)
             const bool walls = bx < 1 || by < 1 || bz < 1;
             // physical x of this lane's column after the refills (the x-shell
             // lane moves to bx - 1)
