@@ -279,8 +279,16 @@ void build_tiles(const fdtd_grid &g, const Layout &L, int order, unsigned seed,
     std::vector<TileEntry> v;
     v.reserve((size_t)std::min<long long>(L.ntiles_max, 1ll << 26));
     for (int K = 0; K < L.gz; ++K)
-        for (int J = 0; J < L.gy; ++J)
-            for (int Pp = 0; Pp < gxp; ++Pp) {
+        for (int J = 0; J < L.gy; ++J) {
+            // only tiles near the diagonal are ever active: the range of I in which
+            // one can be (64^3, 1024 steps: 3 of 36 for one (J, K) in 20, and none
+            // for the others)
+            const int ay = J * L.ty, az = K * L.tz;
+            const int sj = std::max(0, std::max(ay - g.ny + 1, az - g.nz + 1));
+            const int ej = std::min(T - 1, std::min(ay + L.ty - 1, az + L.tz - 1));
+            if (sj > ej + 1) continue;
+            const int p0 = std::max(0, (sj - L.tx) / L.tx / cl), p1 = std::min(gxp - 1, (ej + g.nx) / L.tx / cl);
+            for (int Pp = p0; Pp <= p1; ++Pp) {
                 int s = 0, e = -1;
                 bool kept = false;
                 for (int r = 0; r < cl; ++r) {
@@ -309,6 +317,7 @@ void build_tiles(const fdtd_grid &g, const Layout &L, int order, unsigned seed,
                 }
                 v.push_back(te);
             }
+        }
     std::sort(v.begin(), v.end(), [](const TileEntry &a, const TileEntry &b) {
         if (a.start != b.start) return a.start < b.start;
         if (a.diag != b.diag) return a.diag < b.diag;
