@@ -105,7 +105,7 @@ typedef struct {
  *     ignored).  The E update becomes E <- ca E + cb (curl H - J) with
  *     ca = (1 - g)/(1 + g), cb = (dt/eps)/(1 + g), g = sigma dt/(2 eps),
  *     formed in FP64 and rounded to FP32 per cell.  Systolic scheme: the
- *     default 31x15x12 tile only.
+ *     default tile only (not a tile asked for by name but 31x15x12).
  *   FDTD_BOUNDARY_LEARNED: a layer of `thickness` cells at every wall with
  *     the graded conductivity above (sigma_max, poly_order; sigma_max = 0:
  *     none) whose termination is learned: every cell takes the Yee step of

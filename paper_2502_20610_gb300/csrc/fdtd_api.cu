@@ -61,19 +61,19 @@ bool conducts(const fdtd_boundary &b)
 // rows at a time) 1860 and 1504, 400 x 24 x 24 (136) 1845 and 1568, 72^3 (186)
 // 1883 and 1566, 80^3 (242) 1913 and 1870, 96^3 (384) 2557 and 2746.  Long
 // columns hand tiles on more often, and the line lies lower: 40 x 40 x 150 (160)
-// 1893 and 1671, 24 x 24 x 270 (153) 1815 and 2038.  Cluster pairs and
-// conducting cells take the 12-row form only, and very long launches keep it
-// (their tile order would be half as long again).
+// 1893 and 1671, 24 x 24 x 270 (153) 1815 and 2038.  Cluster pairs take the
+// 12-row form only, and very long launches keep it (their tile order would be
+// half as long again).
 constexpr int FEW_TILES = 152, FEW_TILES_COLUMN = 100, FEW_TILES_STEPS = 4096;
 
-int pick_variant(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &b)
+int pick_variant(const fdtd_grid &g, const fdtd_coeffs &c)
 {
     if (c.tile[0] == 0 && c.tile[1] == 0 && c.tile[2] == 0) {
         constexpr int ROWS12 = 2, ROWS8 = 3;
         const SysShape sh = systolic_shape(ROWS8);
         const double at_a_time = ((double)g.nx + sh.tx - 1) / sh.tx * (((double)g.ny + sh.ty - 1) / sh.ty) *
                                  (((double)g.nz + sh.tz - 1) / sh.tz);
-        const bool few = c.cluster[0] != 2 && !conducts(b) && c.steps_per_launch <= FEW_TILES_STEPS &&
+        const bool few = c.cluster[0] != 2 && c.steps_per_launch <= FEW_TILES_STEPS &&
                          at_a_time <= (g.nz > 4 * std::max(g.nx, g.ny) ? FEW_TILES_COLUMN : FEW_TILES);
         return few ? ROWS8 : ROWS12;
     }
@@ -131,8 +131,8 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     L.fxs = L.fys = 0;
     L.nzb = L.nzblk = 0;
     L.xface = L.yface = off;
-    if (c.scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(g, c, b) >= 2) {
-        const int tz = systolic_shape(pick_variant(g, c, b)).tz;
+    if (c.scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(g, c) >= 2) {
+        const int tz = systolic_shape(pick_variant(g, c)).tz;
         L.nzblk = ceil_div((long long)g.nz + tz - 1, tz);  // columns are stored whole: see the kernel
         L.nzb = L.nzblk * face_block(tz, L.eb);
         const size_t per = align_up((size_t)L.eb * (size_t)g.nx * g.ny * (size_t)L.nzb);
@@ -148,7 +148,7 @@ bool make_layout(const fdtd_grid &g, const fdtd_coeffs &c, const fdtd_boundary &
     L.steps_per_launch = c.steps_per_launch > 0 ? c.steps_per_launch : DEFAULT_STEPS_PER_LAUNCH;
     L.gx = L.gy = L.gz = 0;
     L.ntiles_max = 0;
-    L.variant = pick_variant(g, c, b);
+    L.variant = pick_variant(g, c);
     if (L.variant < 0) return false;
     L.cl = c.scheme == FDTD_SCHEME_SYSTOLIC && c.cluster[0] == 2 ? 2 : 1;
     const SysShape sh = systolic_shape(L.variant);
@@ -193,14 +193,14 @@ fdtd_status check_args(const fdtd_grid *g, const fdtd_coeffs *c, const fdtd_boun
     for (int a = 0; a < 3; ++a) {
         if (c->tile[a] < 0 || c->cluster[a] < 0) return FDTD_ERR_INVALID_ARG;
     }
-    if (pick_variant(*g, *c, *b) < 0) return FDTD_ERR_UNSUPPORTED;
+    if (pick_variant(*g, *c) < 0) return FDTD_ERR_UNSUPPORTED;
     // the shared-memory systolic kernels (tiles 31x15x15, 31x7x15) hold FP32 only
-    if (c->scheme == FDTD_SCHEME_SYSTOLIC && c->storage != FDTD_STORAGE_F32 && pick_variant(*g, *c, *b) < 2)
+    if (c->scheme == FDTD_SCHEME_SYSTOLIC && c->storage != FDTD_STORAGE_F32 && pick_variant(*g, *c) < 2)
         return FDTD_ERR_UNSUPPORTED;
     // clusters: one CTA, or x pairs {2,1,1} of the lossless 31 x 15 x 12
     // register tile under the systolic scheme
     if (c->cluster[1] > 1 || c->cluster[2] > 1 || c->cluster[0] > 2) return FDTD_ERR_UNSUPPORTED;
-    if (c->cluster[0] == 2 && (c->scheme != FDTD_SCHEME_SYSTOLIC || pick_variant(*g, *c, *b) != 2 || conducts(*b)))
+    if (c->cluster[0] == 2 && (c->scheme != FDTD_SCHEME_SYSTOLIC || pick_variant(*g, *c) != 2 || conducts(*b)))
         return FDTD_ERR_UNSUPPORTED;
     if (b->kind < FDTD_BOUNDARY_PEC || b->kind > FDTD_BOUNDARY_LEARNED) return FDTD_ERR_INVALID_ARG;
     if (b->kind == FDTD_BOUNDARY_GRADED_ABSORBER && !b->model) {
@@ -209,8 +209,10 @@ fdtd_status check_args(const fdtd_grid *g, const fdtd_coeffs *c, const fdtd_boun
             return FDTD_ERR_INVALID_ARG;
     }
     if (b->kind == FDTD_BOUNDARY_GRADED_ABSORBER) {
-        // the register kernel's 31 x 15 x 12 tile is the one built with the lossy update
-        if (c->scheme == FDTD_SCHEME_SYSTOLIC && pick_variant(*g, *c, *b) != 2) return FDTD_ERR_UNSUPPORTED;
+        // the lossy update comes with the default tile (31 x 15 x 12, or its choice
+        // for a small domain)
+        const bool chosen = c->tile[0] != 0 || c->tile[1] != 0 || c->tile[2] != 0;
+        if (c->scheme == FDTD_SCHEME_SYSTOLIC && chosen && pick_variant(*g, *c) != 2) return FDTD_ERR_UNSUPPORTED;
     }
     if (b->kind == FDTD_BOUNDARY_LEARNED) {
         if (b->thickness < 1 || !b->model || !(b->sigma_max >= 0.0) || !std::isfinite(b->sigma_max) ||

@@ -1295,19 +1295,18 @@ __global__ void __launch_bounds__(R::NT, 1) systolic_reg_kernel(const __grid_con
 #undef STORE6
 #undef FACE_STORE
 
-// 31 x 15 x 12 and 31 x 15 x 8 tiles, each for every kernel format; the
-// lossy (absorber) form for the 31 x 15 x 12 tile
+// 31 x 15 x 12 and 31 x 15 x 8 tiles, each for every kernel format and in the
+// lossy (absorber) form
 // the box leaves one y slot of the ring outside (TY = 15): as fast as two
 // outside slots (TY = 14) and updates more cells per step
 constexpr int REG_TY = 15;
 template <int NZ>
 struct RegShape {
-    static constexpr bool HAS_LOSSY = NZ == 12;
     static constexpr bool HAS_PAIRS = NZ == 12;  // x pairs in thread-block clusters: the 31 x 15 x 12 tile
     static cudaError_t configure(int fmt, bool lossy, int cl)
     {
         if (lossy) {
-            if constexpr (HAS_LOSSY) if (cl == 1) DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, true, REG_TY>>());
+            if (cl == 1) DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, true, REG_TY>>());
             return cudaErrorInvalidValue;
         }
         if (cl == 2) {
@@ -1323,8 +1322,7 @@ struct RegShape {
     static int per_sm(int fmt, bool lossy)
     {
         if (lossy) {
-            if constexpr (HAS_LOSSY) DISPATCH_FORMAT(fmt, S, occ<RegTile<NZ, S, true, REG_TY>>());
-            return 0;
+            DISPATCH_FORMAT(fmt, S, occ<RegTile<NZ, S, true, REG_TY>>());
         }
         DISPATCH_FORMAT(fmt, S, occ<RegTile<NZ, S, false, REG_TY>>());
     }
@@ -1336,7 +1334,7 @@ struct RegShape {
     static cudaError_t launch(const SysLaunch &p, int grid, cudaStream_t st, int fmt, int cl)
     {
         if (p.ca) {
-            if constexpr (HAS_LOSSY) if (cl == 1) DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, true, REG_TY>>(p, grid, st));
+            if (cl == 1) DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, true, REG_TY>>(p, grid, st));
             return cudaErrorInvalidValue;
         }
         if (cl == 2) {
