@@ -556,6 +556,25 @@ cudaError_t coop_steps(fdtd_sim *h, int n)
     return e;
 }
 
+// Does the naive schedule run as one cooperative launch, or as two kernels a
+// step?  The first while the state is at most twice L2 (its barriers are cheaper
+// than kernel boundaries: 64^3 14.4 -> 8.0 us a step, 160^3 63 -> 51), except in
+// 16-bit storage inside L2 where the two kernels' blocks of 32 x 8 x 8 cells fill
+// whole waves of 8 an SM: conversions, not launches, are the cost there, and
+// more blocks hide them better (us a step in FP16, two kernels and one launch:
+// 128^3, 1024 blocks, 20.6 and 22.7; 160^3, 2000, 34.4 and 38.3; but 128 x 128 x
+// 96, 768, 20.5 and 18.1; 128 x 128 x 160, 1280, 28.9 and 27.1; 144^3, 1620, 32.8
+// and 32.3; FP32 128^3 20.5 and 19.9).
+bool naive_coop(const fdtd_sim *h)
+{
+    const double cells = (double)h->g.nx * h->g.ny * h->g.nz, state = cells * (6.0 * h->L.eb + 4.0);
+    if (state > 256e6) return false;
+    if (h->L.eb == 4 || state > 80e6) return true;
+    const double blocks = (double)ceil_div(h->g.nx, 32) * ceil_div(h->g.ny, 8) * ceil_div(h->g.nz, 8);
+    const double two = blocks <= 1216.0 ? 20.5 : 16.8 + 0.01 * blocks;
+    return 6.0 + 8.0e-6 * cells < two;
+}
+
 // Does a systolic call of n steps run on the cooperative streaming kernel
 // instead (the same bits)?  A systolic launch first fills its pipeline of
 // tiles: some 5.2 us for each tile along the three axes and 0.06 us for each
@@ -883,12 +902,8 @@ fdtd_status fdtd_step(fdtd_handle h, int64_t n)
             }
             return FDTD_OK;
         }
-        // one cooperative launch a call while the state (six components and
-        // dt/eps) is at most twice L2, where its barriers cost less than kernel
-        // boundaries: FP32, us a step, 32^3 14.4 -> 6.8, 64^3 14.4 -> 7.7, 112^3
-        // 20.5 -> 16.4, 160^3 57 -> 51; beyond, the pair of kernels is level or
-        // ahead (256^3 222 against 227)
-        const bool coop = (double)cells * (6.0 * h->L.eb + 4.0) <= 256e6;
+        // one cooperative launch a call, or two kernels a step
+        const bool coop = naive_coop(h);
         while (coop && n > 0) {
             const int T = (int)std::min<int64_t>(n, 1 << 20);
             CK(coop_steps(h, T));

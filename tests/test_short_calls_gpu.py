@@ -50,6 +50,14 @@ def test_bits_of_the_systolic_kernel(cuda_device, shape, kw):
     assert at == 9 and torch.equal(long, naive)
 
 
+@pytest.mark.parametrize("nz,launches", [(90, 1), (128, 10)])
+def test_16_bit_naive_as_one_launch_or_two_kernels_a_step(cuda_device, nz, launches):
+    shape = (nz, 128, 128)
+    long, _, _ = run(shape, [5], "systolic", [], tile="31x15x12", storage="f16")
+    naive, _, n = run(shape, [5], "naive", [], storage="f16")
+    assert n == launches and torch.equal(long, naive)
+
+
 def test_backward_sweep_of_a_state_beyond_l2(cuda_device):
     """Over 96 MB of state the E half-step sweeps the grid backwards."""
     shape = (150, 161, 170)
