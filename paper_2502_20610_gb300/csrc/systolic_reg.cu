@@ -1310,10 +1310,16 @@ struct RegShape {
             return cudaErrorInvalidValue;
         }
         if (cl == 2) {
-            if constexpr (HAS_PAIRS) DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, false, REG_TY, 2>>());
+            if constexpr (HAS_PAIRS) {
+                if (fmt == FDTD_STORAGE_F32) {  // and its capturing form, for the adjoint
+                    const cudaError_t e = set<RegTile<NZ, StoreF32, false, REG_TY, 2, true>>();
+                    if (e != cudaSuccess) return e;
+                }
+                DISPATCH_FORMAT(fmt, S, set<RegTile<NZ, S, false, REG_TY, 2>>());
+            }
             return cudaErrorInvalidValue;
         }
-        if (fmt == FDTD_STORAGE_F32) {  // and its capturing form, for the adjoint
+        if (fmt == FDTD_STORAGE_F32) {  // and its capturing form
             const cudaError_t e = set<RegTile<NZ, StoreF32, false, REG_TY, 1, true>>();
             if (e != cudaSuccess) return e;
         }
@@ -1333,6 +1339,12 @@ struct RegShape {
     }
     static cudaError_t launch(const SysLaunch &p, int grid, cudaStream_t st, int fmt, int cl)
     {
+        if (p.cap) {  // the capturing forms: lossless FP32 (a launch with no such form stores nothing there: an error)
+            if (p.ca || fmt != FDTD_STORAGE_F32) return cudaErrorInvalidValue;
+            if (cl == 1) return go<RegTile<NZ, StoreF32, false, REG_TY, 1, true>>(p, grid, st);
+            if constexpr (HAS_PAIRS) return go<RegTile<NZ, StoreF32, false, REG_TY, 2, true>>(p, grid, st);
+            return cudaErrorInvalidValue;
+        }
         if (p.ca) {
             if (cl == 1) DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, true, REG_TY>>(p, grid, st));
             return cudaErrorInvalidValue;
@@ -1340,10 +1352,6 @@ struct RegShape {
         if (cl == 2) {
             if constexpr (HAS_PAIRS) DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, false, REG_TY, 2>>(p, grid, st));
             return cudaErrorInvalidValue;
-        }
-        if (p.cap) {
-            if (fmt != FDTD_STORAGE_F32) return cudaErrorInvalidValue;
-            return go<RegTile<NZ, StoreF32, false, REG_TY, 1, true>>(p, grid, st);
         }
         DISPATCH_FORMAT(fmt, S, go<RegTile<NZ, S, false, REG_TY>>(p, grid, st));
     }
