@@ -579,8 +579,11 @@ __global__ void __launch_bounds__(32 * RW) record_kernel(const float *__restrict
 // dropped lo*lo term below FP32 rounding of the sum, so the layer keeps
 // FP32 accuracy.
 // x rounded to TF32 (13 bits fewer, to nearest, ties away) as two integer
-// operations: cvt.rna.tf32.f32 gives the same for finite values, as a longer
-// sequence on this part.  (A NaN may lose its mark in hi; lo = x - hi keeps it.)
+// operations: cvt.rna.tf32.f32 gives the same for finite values and infinities,
+// as a longer sequence on this part.  A NaN comes out as a number (the carry of
+// 0x7fffffff, which arithmetic makes, leaves -0), in lo as in hi, and so does the
+// inf - inf of an infinity's lo.  split_tf32 is for values whose NaN is found
+// elsewhere; split_tf32_nan has one in hi where x is not finite.
 __device__ __forceinline__ unsigned tf32_rna(float x)
 {
     return (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
@@ -589,6 +592,13 @@ __device__ __forceinline__ void split_tf32(float x, unsigned &hi, unsigned &lo)
 {
     hi = tf32_rna(x);
     lo = tf32_rna(__fsub_rn(x, __uint_as_float(hi)));
+}
+__device__ __forceinline__ void split_tf32_nan(float x, unsigned &hi, unsigned &lo)
+{
+    hi = tf32_rna(x);
+    const float d = __fsub_rn(x, __uint_as_float(hi));
+    lo = tf32_rna(d);
+    if (d != d) hi = 0x7fc00000u;
 }
 __device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1)
 {
@@ -675,13 +685,18 @@ __global__ void __launch_bounds__(256) weight_image_kernel(const float *__restri
         const int u = e % NH, q = (e / NH) % 4, step = (e / (4 * NH)) % (KF / 8), f = e / (4 * NH * (KF / 8));
         const int tap = step / 3, p = 8 * (step % 3) + q;
         for (int i = 0; i < 2; ++i) v[i] = P[OFF_W1 + u * NI + face_input(f, p + 4 * i, tap / 3, tap % 3)];
+        // a weight of the third left out that is not finite makes its unit NaN too
+        // (times the zeros beyond the wall), here in the unit's first row
+        if (step == 0 && q == 0)
+            for (int k = 0; k < NI; ++k)
+                if (!isfinite(P[OFF_W1 + u * NI + k])) v[0] = nanf("");
     } else {
         const int r = e - N1, u = r % NH, q = (r / NH) % 4, j = r / (4 * NH);
         for (int i = 0; i < 2; ++i) v[i] = P[OFF_W2 + u * NH + 8 * j + 2 * q + i];
     }
     uint4 o;
-    split_tf32(v[0], o.x, o.z);
-    split_tf32(v[1], o.y, o.w);
+    split_tf32_nan(v[0], o.x, o.z);
+    split_tf32_nan(v[1], o.y, o.w);
     img[e] = o;
 }
 
@@ -882,10 +897,14 @@ __global__ void __launch_bounds__(256, 1) layer_kernel(const __grid_constant__ L
             ss1 = __fadd_rn(ss1, __shfl_xor_sync(0xffffffffu, ss1, d));
         }
         const float r0 = sqrtf(ss0 / NI), r1 = sqrtf(ss1 / NI);
-        const bool live0 = r0 >= R_MIN, live1 = r1 >= R_MIN;  // smaller r: the cell keeps its value
+        // smaller r: the cell keeps its value; a NaN in the stencil is in r, and so in
+        // the correction
+        const bool live0 = !(r0 < R_MIN), live1 = !(r1 < R_MIN);
         const float ir0 = live0 ? 1.f / r0 : 0.f, ir1 = live1 ? 1.f / r1 : 0.f;
         if (it == 0 && grp == 0 && seg + 1 < seg_end) asm volatile("bar.arrive 3, 256;" ::: "memory");
-        // H1 = tanh((W1 x) / r + b1), in place
+        // H1 = tanh((W1 x) / r + b1), in place.  A NaN among a row's (a weight's, an
+        // overflow's) is the one with bit 30 set, and goes into its sums of layer 3
+        unsigned m0 = 0, m1 = 0;
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
             const float2 b = *reinterpret_cast<const float2 *>(b1 + 8 * n + 2 * q);
@@ -893,6 +912,8 @@ __global__ void __launch_bounds__(256, 1) layer_kernel(const __grid_constant__ L
             acc[n][1] = tanh_fast(__fmaf_rn(acc[n][1], ir0, b.y));
             acc[n][2] = tanh_fast(__fmaf_rn(acc[n][2], ir1, b.x));
             acc[n][3] = tanh_fast(__fmaf_rn(acc[n][3], ir1, b.y));
+            m0 |= __float_as_uint(acc[n][0]) | __float_as_uint(acc[n][1]);
+            m1 |= __float_as_uint(acc[n][2]) | __float_as_uint(acc[n][3]);
         }
         // layer 2: operand fragment j from accumulator fragment j
         float acc2[8][4];
@@ -913,7 +934,10 @@ __global__ void __launch_bounds__(256, 1) layer_kernel(const __grid_constant__ L
         // layer 3 in FP32: a lane's 16 units of its two rows, then the four lanes of a row
         float y0[NO], y1[NO];
 #pragma unroll
-        for (int o = 0; o < NO; ++o) y0[o] = y1[o] = 0.f;
+        for (int o = 0; o < NO; ++o) {
+            y0[o] = m0 & 0x40000000u ? nanf("") : 0.f;
+            y1[o] = m1 & 0x40000000u ? nanf("") : 0.f;
+        }
 #pragma unroll
         for (int n = 0; n < 8; ++n) {
             const float2 b = *reinterpret_cast<const float2 *>(b2 + 8 * n + 2 * q);
