@@ -89,7 +89,7 @@ typedef struct {
                                  the downwind one through distributed shared memory,
                                  the pair's outer faces go through global memory.
                                  Lossless boundaries only; other shapes UNSUPPORTED. */
-    double wait_timeout_s;    /* bound on any device-side wait; <= 0 = 2 s */
+    double wait_timeout_s;    /* bound on any device-side wait; <= 0 = 2 s (naive scheme: 2 s at least) */
     int32_t max_source_steps; /* capacity of each source table; <= 0 = 65536 */
     int32_t steps_per_launch; /* systolic: steps per persistent launch; <= 0 = 1024 */
 } fdtd_coeffs;

@@ -545,7 +545,10 @@ cudaError_t naive_step(fdtd_sim *h)
 // n steps of the naive schedule in one cooperative launch.
 cudaError_t coop_steps(fdtd_sim *h, int n)
 {
-    const double to = std::max(h->c.wait_timeout_s, 2.0);  // a half-step of a large grid takes milliseconds
+    // the caller's limit, as in the systolic kernel; but a naive handle's barriers
+    // took the place of kernel boundaries, which waited under any limit
+    double to = h->c.wait_timeout_s > 0 ? h->c.wait_timeout_s : 2.0;
+    if (h->c.scheme == FDTD_SCHEME_NAIVE) to = std::max(to, 2.0);
     const cudaError_t e = launch_naive_coop(h->f[0], (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb, h->fmt, h->ce,
                                             h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -(float)h->c.dt, h->step, n,
                                             h->src, h->sc, h->ctrl + CTRL_BARRIER, h->ctrl + 1, (long long)(to * 1e9),

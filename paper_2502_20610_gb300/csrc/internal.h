@@ -52,7 +52,7 @@ cudaError_t launch_naive_block(void *const f[6], int fmt, const float *ce, const
 // CTA per SM (`sms`), grid barriers between the half-steps; component c at
 // f + c*fs.  bar: 8 ints of device memory that start at zero and belong to
 // these launches; err: the device error word a barrier sets (and reads) when
-// it waits longer than timeout_ns.
+// it waits longer than timeout_ns, and two words of details.
 cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, const float *ca, int nx, int ny, int nz,
                               int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc,
                               int *bar, int *err, long long timeout_ns, int sms, cudaStream_t st);

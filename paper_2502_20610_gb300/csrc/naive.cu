@@ -184,7 +184,8 @@ constexpr int COOP_NT = 1024;
 
 // Grid barrier: count of arrivals in bar[0], generation in bar[4]; the last
 // arrival resets the count and bumps the generation, so a launch needs no
-// state from the host.  Bounded wait; false (in every thread) past it.
+// state from the host.  Bounded wait; false (in every thread) past it, with the
+// block and -5 behind the error word.
 __device__ bool grid_barrier(int *bar, unsigned &gen, int *err, long long timeout_ns)
 {
     __shared__ int ok;
@@ -204,7 +205,10 @@ __device__ bool grid_barrier(int *bar, unsigned &gen, int *err, long long timeou
                     break;
                 }
                 if (sysc::globaltimer() - t0 > (unsigned long long)timeout_ns) {
-                    atomicCAS(err, DEV_OK, DEV_ERR_TIMEOUT);
+                    if (atomicCAS(err, DEV_OK, DEV_ERR_TIMEOUT) == DEV_OK) {
+                        err[1] = (int)blockIdx.x;
+                        err[2] = -5;
+                    }
                     good = 0;
                     break;
                 }
