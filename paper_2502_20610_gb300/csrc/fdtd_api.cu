@@ -510,10 +510,11 @@ cudaError_t copy_rows(float *dst, size_t dpitch, const float *src, size_t spitch
                              cudaMemcpyDefault, st);
 }
 
-// True if `p` is memory that kernels on device `dev` can read and write: its
-// own, or managed.
+// True if `p` is memory that kernels on device `dev` can read and write floats
+// in: its own, or managed, and aligned to them (the copies take any address).
 bool is_local_pointer(const void *p, int dev)
 {
+    if ((uintptr_t)p % sizeof(float) != 0) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();  // pageable host memory on older runtimes

@@ -1,0 +1,32 @@
+"""fdtd_write_fields and fdtd_read_fields on device addresses that no float may have:
+copied byte by byte, as they were before a kernel took the aligned ones.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2502_20610_gb300 import fdtd
+from paper_2502_20610_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kw", [{}, {"storage": "f16"}, {"storage": "bf16"}])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_addresses_between_floats(cuda_device, kw, offset):
+    shape = (4, 7, 36)
+    f = wl.random_fields(shape, 7, zero_pec_walls=False)
+    sim = fdtd.Sim(shape, 2.0, wl.DT_DEFAULT, **kw)
+    sim.write_fields(f)
+    host = np.empty((6,) + shape, np.float32)
+    sim.read_fields_ptr(0x3F, host.ctypes.data)
+    src = torch.zeros(f.nbytes + 16, dtype=torch.uint8, device="cuda")
+    src[offset:offset + f.nbytes] = torch.from_numpy(f.reshape(-1).view(np.uint8).copy()).cuda()
+    sim.write_fields(np.zeros_like(f))
+    sim.write_fields_ptr(src.data_ptr() + offset)
+    dst = torch.full((2 * f.nbytes // 6 + 16,), 7, dtype=torch.uint8, device="cuda")
+    sim.read_fields_ptr(0x12, dst.data_ptr() + offset)
+    sim.close()
+    got = dst.cpu().numpy()
+    assert np.array_equal(got[offset:offset + 2 * f.nbytes // 6], host[[1, 4]].reshape(-1).view(np.uint8))
+    assert (got[:offset] == 7).all() and (got[offset + 2 * f.nbytes // 6:] == 7).all()
