@@ -300,15 +300,26 @@ def time_storage_variant(shape, eps, J, src, storage, device, stream, n_calls=1)
     return out
 
 
-def naive_threads(shape):
-    """Threads the library's naive scheme launches on a (nz, ny, nx) grid: one
-    per cell in a single CTA up to 1024 cells, else 32 x 8 CTAs in x-y with
-    each thread marching 8 cells in z."""
+def naive_threads(shape, sms=152):
+    """Threads the library's naive scheme launches on an FP32 (nz, ny, nx) grid
+    on a GPU of `sms` SMs: one per cell in a single CTA up to 1024 cells; up to
+    256 MB of state (28 bytes a cell) CTAs of 1024 threads, one per SM at most,
+    whose warps take 32 x of kz rows in z in turn (kz: the fewest row steps on
+    the busiest warp, a column's start counted as half a row); else 32 x 8 CTAs
+    in x-y with each thread marching 8 cells in z."""
     nz, ny, nx = shape
     cells = nx * ny * nz
     if cells <= 1024:
         return (cells + 31) // 32 * 32
-    return -(-nx // 32) * -(-ny // 8) * -(-nz // 8) * 256
+    if cells * 28 > 256e6:
+        return -(-nx // 32) * -(-ny // 8) * -(-nz // 8) * 256
+    rows, warps = -(-nx // 32) * ny, sms * 32
+
+    def cost(k):
+        return -(-rows * -(-nz // k) // warps) * (k + 0.5)
+
+    kz = min(range(1, min(nz, 24) + 1), key=cost)  # (the first of equals)
+    return min(sms, -(-rows * -(-nz // kz) // 32)) * 1024
 
 
 def sweep_shapes(min_cells=32, max_cells=1 << 28):
@@ -371,7 +382,7 @@ def run_sweep(args):
             eps = np.ones(shape)
             row = {"grid_xyz": list(shape[::-1]), "cells": cells, "bytes_fields": 24 * cells, "steps": steps}
             g, t, nl = measure(shape, "naive", "f32", steps, eps)
-            thr = naive_threads(shape)
+            thr = naive_threads(shape, info["sm_count"])
             resident = min(thr, info["sm_count"] * 2048)  # at most 2048 resident threads per SM
             row.update({"naive_gcups": g, "naive_threads": thr, "naive_launches": nl,
                         "naive_updates_per_us_per_thread": g * 1e3 / thr,
