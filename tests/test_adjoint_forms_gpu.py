@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import adjoint as adj
 from paper_2502_20610_gb300 import fdtd
 from paper_2502_20610_gb300 import workloads as wl
 
@@ -46,3 +47,18 @@ def test_cluster_pairs(cuda_device, shape, steps, window, every):
     naive = gradient(shape, steps, window, every, scheme="naive")
     assert pair[0] == naive[0] and pair[0] > 0.0
     assert torch.equal(pair[1], naive[1]) and torch.equal(pair[2], naive[2])
+
+
+def test_twelve_row_tile(cuda_device):
+    """The capturing kernel of larger domains, against the float64 adjoint as well."""
+    shape, steps, window, every = (26, 24, 30), 60, 25, 20
+    eps, lo, hi, mode, src = problem(shape, steps)
+    loss, grad, state = gradient(shape, steps, window, every, tile="31x15x12")
+    naive = gradient(shape, steps, window, every, scheme="naive")
+    assert loss == naive[0] and torch.equal(grad, naive[1]) and torch.equal(state, naive[2])
+    obj = adj.Objective(hi[2] + 3, mode.astype(np.float64), window)
+    ref_loss, ref = adj.gradient(shape, eps, np.zeros((6,) + shape), steps, [src], obj, DT, quantize=True)
+    ref = ref[lo[2]:hi[2], lo[1]:hi[1], lo[0]:hi[0]]
+    # the gradient's bound of the adjoint tests: FP32 rounding over the steps
+    assert abs(loss - ref_loss) <= 1e-4 * ref_loss
+    assert np.linalg.norm(grad.cpu().numpy() - ref) <= 1e-4 * np.linalg.norm(ref)
