@@ -736,8 +736,8 @@ __global__ void __launch_bounds__(256) snapshot_kernel(const __grid_constant__ L
 // Lambert's continued fraction x / (1 + x^2 / (3 + x^2 / (5 + ...))) as x less
 // x times a quotient of polynomials in x^2 (its truncation error is under 1e-9
 // there), above it 1 - 2 / (exp(2 |x|) + 1); one reciprocal for both, refined
-// by a Newton step.  At most 2 units in the last place off (1.3 in a
-// float32 emulation over the range; tanhf is allowed 2), odd, NaN for NaN.
+// by a Newton step.  Over all floats of [2^-14, 12] on this GPU: 1.25 units in the
+// last place at most, near 1 (tanhf: 1.82); odd, NaN for NaN.
 __device__ __forceinline__ float tanh_fast(float x)
 {
     const float a = fabsf(x) > 10.f ? 10.f : fabsf(x), t = __fmul_rn(a, a);  // (NaN stays)
