@@ -172,13 +172,19 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src);
 
 /* Advance n >= 0 whole steps with the handle's scheme.  The naive scheme runs
  * a grid of at most 1024 cells in one thread block per call, with block
- * barriers between the half-steps, a grid whose state is at most twice the
- * GPU's L2 in one cooperative launch, with grid barriers, and a larger one as
- * a kernel per half-step.  A systolic handle takes calls of one or two steps
- * as such a cooperative launch too (the results are the same bits).
- * Asynchronous:
+ * barriers between the half-steps; a larger one whose state (six fields and
+ * dt/eps) is at most 256 MB, twice the GPU's L2, in one cooperative launch
+ * with grid barriers, or, in 16-bit storage inside L2, as a kernel per
+ * half-step where that is estimated faster; and one larger still, or with a
+ * learned boundary, as a kernel per half-step.  A systolic handle without
+ * cluster pairs takes calls of one or two steps as such a cooperative launch
+ * too, and one with the default tile every call that an estimate from the
+ * grid's extents finds too short to fill the pipeline of tiles (FP32: up to 15
+ * steps of 64^3, 5 of 160^3, 26 of 40 x 40 x 300).  The results are the same
+ * bits.  Asynchronous:
  * returns once the kernels are enqueued; launch errors are returned here,
- * device-side wait timeouts at the next fdtd_sync / fdtd_read_fields.
+ * device-side wait timeouts (of either scheme) at the next fdtd_sync /
+ * fdtd_read_fields.
  * Errors: INVALID_ARG (n < 0), STATE (an earlier device error not cleared
  * by fdtd_write_fields), CUDA. */
 fdtd_status fdtd_step(fdtd_handle h, int64_t n);
@@ -223,6 +229,8 @@ void fdtd_destroy(fdtd_handle h);
  *   FDTD_DEBUG_ORDER         hand out subdomains in another valid
  *                            topological order (param: 1 = random tie-break
  *                            seeded by ticket, 2 = lexicographic k,j,i).
+ * While a hook is set (an order other than the usual one included), calls of
+ * few steps stay on the systolic kernel.
  * Errors: INVALID_ARG. */
 enum { FDTD_DEBUG_NONE = 0, FDTD_DEBUG_SKIP_PUBLISH = 1, FDTD_DEBUG_DELAY = 2, FDTD_DEBUG_ORDER = 3 };
 fdtd_status fdtd_debug_set(fdtd_handle h, int32_t kind, int64_t ticket, int64_t param, int64_t param2);
