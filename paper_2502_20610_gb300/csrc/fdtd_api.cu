@@ -543,7 +543,8 @@ cudaError_t naive_step(fdtd_sim *h)
     return e;
 }
 
-// n steps of the naive schedule in one cooperative launch.
+// n steps of the naive schedule in one cooperative launch, where the stream has
+// the SMs for it.
 cudaError_t coop_steps(fdtd_sim *h, int n)
 {
     // the caller's limit, as in the systolic kernel; but a naive handle's barriers
@@ -554,6 +555,14 @@ cudaError_t coop_steps(fdtd_sim *h, int n)
                                             h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -(float)h->c.dt, h->step, n,
                                             h->src, h->sc, h->ctrl + CTRL_BARRIER, h->ctrl + 1, (long long)(to * 1e9),
                                             h->sms, h->stream);
+    // a stream that owns a part of the SMs only (a green context's) cannot hold the
+    // grid at once: two kernels a step, the same bits
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        cudaError_t s = cudaSuccess;
+        for (int k = 0; k < n && s == cudaSuccess; ++k) s = naive_step(h);
+        return s;
+    }
     if (e != cudaSuccess) return e;
     h->launches += 1;
     h->step += n;
