@@ -353,6 +353,22 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
+// Does the stream own a part of the SMs only (a green context's)?  A cooperative
+// grid of a CTA on every SM is refused there, or, captured into a graph, where
+// nothing checks it, is never placed.
+static bool partitioned(cudaStream_t st)
+{
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &p, 12040, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();  // a driver without them
+        return false;
+    }
+    CUgreenCtx ctx = nullptr;
+    return ((PFN_cuStreamGetGreenCtx_v12040)p)((CUstream)st, &ctx) == CUDA_SUCCESS && ctx;
+}
+
 bool encode_shell_maps(CUtensorMap tm[3][2], void *fbase, long long fstride, const float *ce, const float *ca,
                        int storage, int nx, int ny, int nz, int pitch, int nr, int bz, void *xf, long long fxs,
                        void *yf, long long fys, int nzb)
@@ -480,6 +496,7 @@ struct fdtd_sim {
     long long cap_bc = 0, cap_s0 = 0;
     long long launches;
     int dev, sms;  // the handle's device and its SMs
+    bool coop;     // cooperative launches of a CTA on every SM can run on the stream
     int max_ctas;
     std::vector<long long> count_le;  // tiles with start <= s
     int dbg_kind;
@@ -543,26 +560,21 @@ cudaError_t naive_step(fdtd_sim *h)
     return e;
 }
 
-// n steps of the naive schedule in one cooperative launch, where the stream has
-// the SMs for it.
+// n steps of the naive schedule in one cooperative launch, where the handle can.
 cudaError_t coop_steps(fdtd_sim *h, int n)
 {
     // the caller's limit, as in the systolic kernel; but a naive handle's barriers
     // took the place of kernel boundaries, which waited under any limit
     double to = h->c.wait_timeout_s > 0 ? h->c.wait_timeout_s : 2.0;
     if (h->c.scheme == FDTD_SCHEME_NAIVE) to = std::max(to, 2.0);
-    const cudaError_t e = launch_naive_coop(h->f[0], (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb, h->fmt, h->ce,
-                                            h->ca, h->g.nx, h->g.ny, h->g.nz, h->L.pitch, -(float)h->c.dt, h->step, n,
-                                            h->src, h->sc, h->ctrl + CTRL_BARRIER, h->ctrl + 1, (long long)(to * 1e9),
-                                            h->sms, h->stream);
-    // a stream that owns a part of the SMs only (a green context's) cannot hold the
-    // grid at once: two kernels a step, the same bits
-    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
-        cudaGetLastError();
-        cudaError_t s = cudaSuccess;
-        for (int k = 0; k < n && s == cudaSuccess; ++k) s = naive_step(h);
-        return s;
+    cudaError_t e = cudaSuccess;
+    if (!h->coop) {  // two kernels a step, the same bits
+        for (int k = 0; k < n && e == cudaSuccess; ++k) e = naive_step(h);
+        return e;
     }
+    e = launch_naive_coop(h->f[0], (long long)(h->L.fields[1] - h->L.fields[0]) / h->L.eb, h->fmt, h->ce, h->ca, h->g.nx, h->g.ny,
+                          h->g.nz, h->L.pitch, -(float)h->c.dt, h->step, n, h->src, h->sc, h->ctrl + CTRL_BARRIER, h->ctrl + 1,
+                          (long long)(to * 1e9), h->sms, h->stream);
     if (e != cudaSuccess) return e;
     h->launches += 1;
     h->step += n;
@@ -779,6 +791,10 @@ fdtd_status fdtd_create(const fdtd_grid *grid, const double *eps, const fdtd_coe
     if (e != cudaSuccess) return fail(cuda_status(e));
     h->dev = dev;
     h->sms = sms;
+    int can = 0;
+    e = cudaDeviceGetAttribute(&can, cudaDevAttrCooperativeLaunch, dev);
+    if (e != cudaSuccess) return fail(cuda_status(e));
+    h->coop = can && !partitioned(h->stream);
     if (coeffs->scheme == FDTD_SCHEME_SYSTOLIC) {
         e = systolic_configure(L.variant, h->fmt, h->ca != nullptr, L.cl);
         if (e != cudaSuccess) return fail(cuda_status(e));

@@ -1,6 +1,6 @@
 """Steps on a stream that owns a part of the SMs only (a green context of this process):
 a cooperative grid of a CTA on every SM doesn't fit there, and the calls that would
-use one run all the same.
+use one run as two kernels a step.
 """
 import contextlib
 import ctypes
@@ -47,17 +47,17 @@ def stepped(shape, calls, **kw):
     sim.write_fields(torch.as_tensor(wl.random_fields(shape, 3)).cuda())
     for n in calls:
         sim.step(n)
-    out, at = sim.read_fields(), sim.current_step
+    out, at, launches = sim.read_fields(), sim.current_step, sim.launch_count
     sim.close()
-    return out.view(torch.int32), at
+    return out.view(torch.int32), at, launches
 
 
-@pytest.mark.parametrize("kw,calls", [({"scheme": "naive"}, [5, 2]), ({"scheme": "systolic"}, [1, 2, 4]),
-                                      ({"scheme": "systolic", "tile": "31x15x12"}, [2, 5]),
-                                      ({"scheme": "naive", "storage": "f16"}, [7])])
-def test_every_schedule_runs_on_a_part_of_the_chip(cuda_device, kw, calls):
+@pytest.mark.parametrize("kw,calls,launches", [
+    ({"scheme": "naive"}, [5, 2], 14), ({"scheme": "systolic"}, [1, 2, 4], 14),
+    ({"scheme": "systolic", "tile": "31x15x12"}, [2, 5], 5), ({"scheme": "naive", "storage": "f16"}, [7], 14)])
+def test_every_schedule_runs_on_a_part_of_the_chip(cuda_device, kw, calls, launches):
     shape = (60, 66, 70)
-    whole, _ = stepped(shape, calls, **kw)
+    whole, _, _ = stepped(shape, calls, **kw)
     with partition(16):
-        part, at = stepped(shape, calls, **kw)
-    assert at == sum(calls) and torch.equal(whole, part)
+        part, at, n = stepped(shape, calls, **kw)
+    assert at == sum(calls) and n == launches and torch.equal(whole, part)
