@@ -616,7 +616,7 @@ bool naive_coop(const fdtd_sim *h)
 // cluster pairs, which are the systolic kernel's own.
 bool short_call(const fdtd_sim *h, int64_t n)
 {
-    if (h->cap || h->dbg_kind != FDTD_DEBUG_NONE || h->dbg_order != 0 || h->L.cl != 1) return false;
+    if (n == 0 || h->cap || h->dbg_kind != FDTD_DEBUG_NONE || h->dbg_order != 0 || h->L.cl != 1) return false;
     if (n <= 2) return true;
     if (h->c.tile[0] != 0 || n > h->L.steps_per_launch) return false;
     const double nx = h->g.nx, ny = h->g.ny, nz = h->g.nz, cells = nx * ny * nz, k = cells * 1e-6;
