@@ -590,10 +590,30 @@ cudaError_t coop_steps(fdtd_sim *h, int n)
 // 128^3, 1024 blocks, 20.6 and 22.7; 160^3, 2000, 34.4 and 38.3; but 128 x 128 x
 // 96, 768, 20.5 and 18.1; 128 x 128 x 160, 1280, 28.9 and 27.1; 144^3, 1620, 32.8
 // and 32.3; FP32 128^3 20.5 and 19.9).
-bool naive_coop(const fdtd_sim *h)
+// On thin grids (16 planes at most, or rows of 12 cells) the columns are too few or
+// too short for the launch's co-resident warps, or leave most lanes of a warp idle,
+// and both forms are estimated: the launch by its barriers and the row steps of its
+// busiest warp (and 2.4 us a call), the two kernels by the rows that a thread
+// marches, the rows of all warps, and the blocks past a wave of 8 an SM.  Both
+// estimates are within 11 % on eight of ten, and 32 % on all, of 170 grids a type
+// (us a step in FP32, two kernels and one launch: 1000 x 1000 x 1 14.9 and 20.5, 700
+// x 700 x 4 23.0 and 28.7, 1 x 450 x 450 47.9 and 57.4; but 300 x 300 x 4 13.3 and
+// 12.7, 60 x 60 x 2 9.9 and 7.5, 5 x 150 x 150 17.0 and 12.0; FP16 700 x 700 x 9 34.1
+// and 49.5).
+bool naive_coop(const fdtd_sim *h, int64_t n)
 {
     const double cells = (double)h->g.nx * h->g.ny * h->g.nz, state = cells * (6.0 * h->L.eb + 4.0);
     if (state > 256e6) return false;
+    if ((h->g.nz <= 16 || h->g.nx <= 12) && state <= 96e6) {
+        const bool wide = h->L.eb == 4;
+        const double rows = (double)ceil_div(h->g.nx, 32) * h->g.ny * h->g.nz * 1e-3;
+        const double blocks = (double)ceil_div(h->g.nx, 32) * ceil_div(h->g.ny, 8) * ceil_div(h->g.nz, 8) * 1e-3;
+        const double march = std::min(h->g.nz, 8), over = std::max(0.0, blocks - 8e-3 * h->sms);
+        const double one = 5.4 + (wide ? 1.07 : 1.19) * naive_coop_row_steps(h->g.nx, h->g.ny, h->g.nz, h->sms) + 2.4 / (double)n;
+        const double two = wide ? 7.6 + 0.96 * march + 0.155 * rows + 0.16 * blocks + 1.09 * over
+                                : 7.1 + 1.09 * march + 0.176 * rows + 1.88 * over;
+        return one < std::max(8.3, two);
+    }
     if (h->L.eb == 4 || state > 80e6) return true;
     const double blocks = (double)ceil_div(h->g.nx, 32) * ceil_div(h->g.ny, 8) * ceil_div(h->g.nz, 8);
     const double two = blocks <= 1216.0 ? 20.5 : 16.8 + 0.01 * blocks;
@@ -932,7 +952,7 @@ fdtd_status fdtd_step(fdtd_handle h, int64_t n)
             return FDTD_OK;
         }
         // one cooperative launch a call, or two kernels a step
-        const bool coop = naive_coop(h);
+        const bool coop = n > 0 && naive_coop(h, n);
         while (coop && n > 0) {
             const int T = (int)std::min<int64_t>(n, 1 << 20);
             CK(coop_steps(h, T));
@@ -1326,9 +1346,9 @@ fdtd_status fdtd_adjoint_gradient(fdtd_handle h, const fdtd_overlap_objective *o
     // kernel pair, which the systolic schedule reproduces bit for bit
     const bool reg_kernel = h->c.scheme == FDTD_SCHEME_SYSTOLIC && h->L.variant >= 2;
     auto one_step = [&]() -> cudaError_t {
-        // one cooperative launch, as for a naive handle, unless the state is far
-        // beyond L2 (200 x 200 x 100: 57 -> 51 us a step)
-        return (double)h->g.nx * h->g.ny * h->g.nz * 28.0 <= 256e6 ? coop_steps(h, 1) : naive_step(h);
+        // one cooperative launch, or two kernels, as for a naive handle (200 x 200 x
+        // 100: 57 us a step as two kernels, 51 as one launch)
+        return naive_coop(h, 1) ? coop_steps(h, 1) : naive_step(h);
     };
     // m steps of h, the box's E after step r (r = 1..m) into plane p0 + r of
     // buf: captured by the register kernel, or copied after single steps

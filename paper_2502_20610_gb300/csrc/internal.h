@@ -57,6 +57,10 @@ cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, c
                               int pitch, float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc,
                               int *bar, int *err, long long timeout_ns, int sms, cudaStream_t st);
 
+// Row steps of its busiest warp in a half-step, a column's start counted as one:
+// what a launch's time goes by.
+double naive_coop_row_steps(int nx, int ny, int nz, int sms);
+
 // Fields between dense FP32 components (nx*ny*nz values each, packed in the
 // order of `comps`, 4 bits each) and the arrays in storage format (component
 // c at arrays + c*fs, rows of `pitch` elements), one launch (convert.cu);

@@ -376,15 +376,11 @@ cudaError_t launch_block(void *const f[6], const float *ce, const float *ca, int
     return cudaGetLastError();
 }
 
-template <class S, bool LOSSY>
-cudaError_t launch_coop(void *f, long long fs, const float *ce, const float *ca, int nx, int ny, int nz, int pitch,
-                        float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc, int *bar, int *err,
-                        long long timeout_ns, int sms, cudaStream_t st)
+// Rows in z per warp of the cooperative launch: the fewest row steps on the
+// busiest warp, a column's start (its two z-neighbour loads) counted as half a
+// row; a remainder round of full-height columns would double a half-step.
+int rows_per_warp(int nx, int ny, int nz, int sms)
 {
-    using T = typename S::T;
-    // rows in z per warp: the fewest row steps on the busiest warp, a column's
-    // start (its two z-neighbour loads) counted as half a row; a remainder
-    // round of full-height columns would double a half-step
     const long long rows = (long long)((nx + 31) / 32) * ny, warps = (long long)sms * (COOP_NT / 32);
     int kz = 1;
     double least = 0.0;
@@ -395,6 +391,17 @@ cudaError_t launch_coop(void *f, long long fs, const float *ce, const float *ca,
             kz = k;
         }
     }
+    return kz;
+}
+
+template <class S, bool LOSSY>
+cudaError_t launch_coop(void *f, long long fs, const float *ce, const float *ca, int nx, int ny, int nz, int pitch,
+                        float neg_dt, long long step0, int nsteps, const SrcSet &src, const Scales &sc, int *bar, int *err,
+                        long long timeout_ns, int sms, cudaStream_t st)
+{
+    using T = typename S::T;
+    const int kz = rows_per_warp(nx, ny, nz, sms);
+    const long long rows = (long long)((nx + 31) / 32) * ny;
     const long long items = rows * ((nz + kz - 1) / kz);
     const int grid = (int)std::min<long long>(sms, (items + COOP_NT / 32 - 1) / (COOP_NT / 32));
     cudaLaunchAttribute at[1];
@@ -421,6 +428,13 @@ cudaError_t launch_naive_coop(void *f, long long fs, int fmt, const float *ce, c
                                                      err, timeout_ns, sms, st));
     DISPATCH_FORMAT(fmt, S, launch_coop<S, false>(f, fs, ce, ca, nx, ny, nz, pitch, neg_dt, step0, nsteps, src, sc, bar, err,
                                                   timeout_ns, sms, st));
+}
+
+double naive_coop_row_steps(int nx, int ny, int nz, int sms)
+{
+    const int kz = rows_per_warp(nx, ny, nz, sms);
+    const long long warps = (long long)sms * (COOP_NT / 32), items = (long long)((nx + 31) / 32) * ny * ((nz + kz - 1) / kz);
+    return (double)((items + warps - 1) / warps) * (kz + 1);
 }
 
 int naive_block_max_cells() { return NAIVE_BLOCK_CELLS; }
