@@ -648,6 +648,12 @@ bool short_call(const fdtd_sim *h, int64_t n)
     const double stream = (double)n * (6.0 + k * per);
     const double step = std::max(h->L.tz < 12 ? 3.5 : 4.5, 2.2 + 4.7 * k);
     const double systolic = 5.2 * hops + 0.06 * tiles + (double)n * step;
+    // a sheet across x: the streaming kernel takes 230 ns for a thousand rows of up to
+    // 32 cells (a warp's, however many of its lanes have one), where it has more of
+    // them than the cells say: 3 x 700 x 700 119 us a step, and calls of 8 to 76 steps
+    // were up to 1.5 times as long as the systolic kernel's; 33 x 300 x 300 57
+    const double rows = (double)ceil_div(h->g.nx, 32) * ny * nz * 1e-3;
+    if (ny >= 128 && nz >= 128 && (double)n * (5.4 + 0.23 * rows) >= systolic) return false;
     return stream < 0.9 * systolic;
 }
 

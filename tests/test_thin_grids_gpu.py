@@ -30,3 +30,31 @@ def test_form_and_bits(cuda_device, shape, storage, launches):
     assert n == launches
     systolic, _ = stepped(shape, scheme="systolic", storage=storage, tile="31x15x12")
     assert torch.equal(naive, systolic)
+
+
+def form_of_a_call(shape, steps):
+    """(fields after the call, did the cooperative kernel run it).  Its grid barrier counts generations in word 20 of the
+    handle's control words, the last 256 bytes of the workspace."""
+    sim = fdtd.Sim(shape, 3.0, wl.DT_DEFAULT)
+    sim.write_fields(torch.as_tensor(wl.random_fields(shape, 5, zero_pec_walls=False)).cuda())
+    sim.step(steps)
+    out = sim.read_fields().view(torch.int32)
+    generations = int(sim.workspace[-256:].view(torch.int32)[20])
+    sim.close()
+    assert generations in (0, 2 * steps - 1)
+    return out, generations > 0
+
+
+# sheets across x, whose rows leave most lanes of a warp idle, and grids that fill them
+@pytest.mark.parametrize("shape,steps,streaming", [
+    ((450, 450, 1), 20, False), ((700, 700, 3), 12, False), ((700, 700, 3), 3, True), ((300, 300, 33), 18, False),
+    ((300, 300, 33), 5, True), ((2000, 10, 10), 60, True), ((300, 40, 40), 18, True), ((64, 64, 64), 8, True),
+    ((64, 64, 64), 40, False), ((500, 100, 20), 25, True)])
+def test_which_calls_of_few_steps_stream(cuda_device, shape, steps, streaming):
+    out, streamed = form_of_a_call(shape, steps)
+    assert streamed == streaming
+    sim = fdtd.Sim(shape, 3.0, wl.DT_DEFAULT, scheme="naive")
+    sim.write_fields(torch.as_tensor(wl.random_fields(shape, 5, zero_pec_walls=False)).cuda())
+    sim.step(steps)
+    assert torch.equal(out, sim.read_fields().view(torch.int32))
+    sim.close()
