@@ -1,5 +1,6 @@
 """fdtd_write_fields and fdtd_read_fields on device addresses that no float may have:
-copied byte by byte, as they were before a kernel took the aligned ones.
+copied byte by byte, as they were before a kernel took the aligned ones; and rows of
+a few values, which take fewer threads than a quarter warp.
 """
 import numpy as np
 import pytest
@@ -30,3 +31,18 @@ def test_addresses_between_floats(cuda_device, kw, offset):
     got = dst.cpu().numpy()
     assert np.array_equal(got[offset:offset + 2 * f.nbytes // 6], host[[1, 4]].reshape(-1).view(np.uint8))
     assert (got[:offset] == 7).all() and (got[offset + 2 * f.nbytes // 6:] == 7).all()
+
+
+@pytest.mark.parametrize("kw", [{}, {"storage": "f16"}])
+@pytest.mark.parametrize("nx", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("rows", [(1, 1), (300, 7), (2, 2500)])
+def test_narrow_rows(cuda_device, kw, nx, rows):
+    shape = (*rows, nx)
+    f = wl.random_fields(shape, 9, zero_pec_walls=False)
+    sim = fdtd.Sim(shape, 2.0, wl.DT_DEFAULT, **kw)
+    sim.write_fields(torch.from_numpy(f).cuda())
+    got = sim.read_fields().cpu().numpy()
+    one = sim.read_fields(mask=0x20).cpu().numpy()
+    sim.close()
+    ref = f.astype(np.float16).astype(np.float32) if kw else f
+    assert np.array_equal(got, ref) and np.array_equal(one[0], ref[5])
