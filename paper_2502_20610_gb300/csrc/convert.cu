@@ -68,6 +68,52 @@ fields_kernel(typename S::T *arrays, long long fs, float *dense, long long n, in
     }
 }
 
+// The same for rows that leave most of such a grid idle.  PARTS: few rows, whose
+// parts go over y blocks.  Else: many rows that are not in groups of four values,
+// four of them, next to one another, in flight a thread.  (Forms of their own: in
+// the one above, four rows a grid apart made 128^3 slower to write, 25 -> 30 us in
+// FP32, and a stride over y blocks 23 -> 26 in FP16.)
+template <class S, bool IN, bool VEC, bool PARTS>
+__global__ void __launch_bounds__(256)
+odd_rows_kernel(typename S::T *arrays, long long fs, float *dense, long long n, int nx, long long rows, int pitch,
+                unsigned comps, const Scales sc, int *zero, int nzero, const int *err)
+{
+    static_assert(PARTS || !VEC, "groups of four values need no more rows in flight");
+    if (!IN && *err != DEV_OK) return;
+    if (IN && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.y == 0)
+        for (int q = threadIdx.x; q < nzero; q += blockDim.x) zero[q] = 0;
+    const int c = (comps >> (4 * blockIdx.z)) & 15;
+    typename S::T *const f = arrays + c * fs;
+    float *const d = dense + blockIdx.z * n;
+    constexpr int Q = PARTS ? 1 : 4;
+    const int x0 = blockIdx.y * blockDim.x + threadIdx.x, dx = gridDim.y * blockDim.x;
+    for (long long r = Q * (blockIdx.x * (long long)blockDim.y + threadIdx.y); r < rows;
+         r += Q * (long long)gridDim.x * blockDim.y) {
+        typename S::T *const fr = f + r * pitch;
+        float *const dr = d + r * nx;
+        if constexpr (VEC) {
+            for (int x = 4 * x0; x < nx; x += 4 * dx) {
+                if (IN) put4<S>(fr + x, *reinterpret_cast<const float4 *>(dr + x), sc.is[c]);
+                else *reinterpret_cast<float4 *>(dr + x) = get4<S>(fr + x, sc.s[c]);
+            }
+        } else {
+            const int live = (int)min((long long)Q, rows - r);
+            for (int x = x0; x < nx; x += dx) {
+                float v[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (q < live) v[q] = IN ? dr[q * nx + x] : S::dec(fr[q * pitch + x], sc.s[c]);
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (q < live) {
+                        if (IN) fr[q * pitch + x] = S::enc(v[q], sc.is[c]);
+                        else dr[q * nx + x] = v[q];
+                    }
+            }
+        }
+    }
+}
+
 template <class S, bool IN>
 cudaError_t go(void *arrays, long long fs, float *dense, int nx, int ny, int nz, int pitch, unsigned comps, int ncomp,
                const Scales &sc, int *zero, int nzero, const int *err, cudaStream_t st)
@@ -81,13 +127,22 @@ cudaError_t go(void *arrays, long long fs, float *dense, int nx, int ny, int nz,
     int bx = 1;
     while (bx < 256 && bx < per_row) bx *= 2;
     const dim3 block((unsigned)bx, 256u / bx);
-    const dim3 grid((unsigned)std::min<long long>((rows + block.y - 1) / block.y, 152 * 8), 1, (unsigned)ncomp);
-    if (vec)
-        fields_kernel<S, IN, true><<<grid, block, 0, st>>>((typename S::T *)arrays, fs, dense, (long long)nx * rows, nx, rows,
-                                                           pitch, comps, sc, zero, nzero, err);
-    else
-        fields_kernel<S, IN, false><<<grid, block, 0, st>>>((typename S::T *)arrays, fs, dense, (long long)nx * rows, nx, rows,
-                                                            pitch, comps, sc, zero, nzero, err);
+    // where rows are few, a row's parts go over blocks too (nine rows of 20000 values in
+    // FP16 from pinned memory: 170 us by nine blocks a component, 107 so); where they are
+    // many and not in groups of four values, four rows a thread (a component of 30 x 600
+    // x 600 in FP16 read in 60 us with one row in flight, 46 so)
+    constexpr long long BLOCKS = 152 * 8;
+    const long long blocks = (rows + block.y - 1) / block.y;
+    const unsigned gx = (unsigned)std::min(blocks, BLOCKS);
+    const unsigned parts = std::min((unsigned)((per_row + bx - 1) / bx), (unsigned)(BLOCKS / gx));
+    const dim3 grid(gx, parts, (unsigned)ncomp);
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, block, 0, st>>>((typename S::T *)arrays, fs, dense, (long long)nx * rows, nx, rows, pitch, comps, sc, zero,
+                                       nzero, err);
+    };
+    if (parts > 1) launch(vec ? odd_rows_kernel<S, IN, true, true> : odd_rows_kernel<S, IN, false, true>);
+    else if (!vec && blocks >= 4 * BLOCKS) launch(odd_rows_kernel<S, IN, false, false>);
+    else launch(vec ? fields_kernel<S, IN, true> : fields_kernel<S, IN, false>);
     return cudaGetLastError();
 }
 

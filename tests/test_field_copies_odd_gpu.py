@@ -46,3 +46,23 @@ def test_narrow_rows(cuda_device, kw, nx, rows):
     sim.close()
     ref = f.astype(np.float16).astype(np.float32) if kw else f
     assert np.array_equal(got, ref) and np.array_equal(one[0], ref[5])
+
+
+# few rows, whose parts go over blocks (in groups of four values and not), and rows
+# enough that a thread takes four, the last of them short of four
+@pytest.mark.parametrize("kw", [{}, {"storage": "f16"}])
+@pytest.mark.parametrize("shape", [(1, 1, 20001), (1, 1, 20000), (3, 3, 1030), (2, 3, 1028), (300, 131, 30), (301, 131, 29),
+                                   (250, 160, 17)])
+def test_few_long_rows_and_many_short_ones(cuda_device, kw, shape):
+    f = wl.random_fields(shape, 11, zero_pec_walls=False)
+    sim = fdtd.Sim(shape, 2.0, wl.DT_DEFAULT, scheme="naive", **kw)
+    ref = f.astype(np.float16).astype(np.float32) if kw else f
+    sim.write_fields(torch.from_numpy(f).cuda())
+    got = sim.read_fields().cpu().numpy()
+    assert np.array_equal(got, ref)
+    sim.write_fields(np.zeros_like(f))
+    sim.write_fields(f)  # from the host: a component at a time
+    host = np.empty((2,) + shape, np.float32)
+    sim.read_fields_ptr(0x28, host.ctypes.data)
+    sim.close()
+    assert np.array_equal(host, ref[[3, 5]])
