@@ -306,7 +306,8 @@ def naive_threads(shape, sms=152):
     256 MB of state (28 bytes a cell) CTAs of 1024 threads, one per SM at most,
     whose warps take 32 x of kz rows in z in turn (kz: the fewest row steps on
     the busiest warp, a column's start counted as half a row); else 32 x 8 CTAs
-    in x-y with each thread marching 8 cells in z."""
+    in x-y with each thread marching 8 cells in z.  (Of balanced grids, as the
+    sweep's are: large thin ones below 256 MB run in the last form too.)"""
     nz, ny, nx = shape
     cells = nx * ny * nz
     if cells <= 1024:

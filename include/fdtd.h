@@ -174,14 +174,15 @@ fdtd_status fdtd_write_fields(fdtd_handle h, const float *src);
  * a grid of at most 1024 cells in one thread block per call, with block
  * barriers between the half-steps; a larger one whose state (six fields and
  * dt/eps) is at most 256 MB, twice the GPU's L2, in one cooperative launch
- * with grid barriers, or, in 16-bit storage inside L2, as a kernel per
- * half-step where that is estimated faster; and one larger still, or with a
+ * with grid barriers, or, in 16-bit storage or on a thin grid inside L2, as a
+ * kernel per half-step where that is estimated faster; and one larger still, or
+ * on a stream that owns a part of the SMs only (a green context's), or with a
  * learned boundary, as a kernel per half-step.  A systolic handle without
  * cluster pairs takes calls of one or two steps as such a cooperative launch
  * too, and one with the default tile every call that an estimate from the
  * grid's extents finds too short to fill the pipeline of tiles (FP32: up to 15
- * steps of 64^3, 5 of 160^3, 26 of 40 x 40 x 300).  The results are the same
- * bits.  Asynchronous:
+ * steps of 64^3, 5 of 160^3, 26 of 40 x 40 x 300, 6 of 3 x 700 x 700).  The
+ * results are the same bits.  Asynchronous:
  * returns once the kernels are enqueued; launch errors are returned here,
  * device-side wait timeouts (of either scheme) at the next fdtd_sync /
  * fdtd_read_fields.
